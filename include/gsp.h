@@ -189,8 +189,11 @@ gsp_status gsp_scene_set_materials(gsp_scene* scene, const gsp_material* mats, i
  * which only corrupt links can reach). A ray that reaches the bound ends early and the first
  * such event sets GSP_ERR_TRAVERSAL_LIMIT in the context's status word, which the next
  * gsp_context_sync / gsp_sppm_sync returns (and clears); nothing traps and the context stays
- * usable. Applies to launches made after the call (renderers read it per pass). For bounding
- * worst-case work, and for testing the failure path without corrupting a BVH. */
+ * usable. Applies to launches made after the call (renderers read it per pass). While a limit is
+ * set, rays follow the hit/miss links, whose box tests it counts; without one, those of a scene with
+ * six link sets walk the tree's four-wide form (gsp_trace_closest_hit), with the same hits. For
+ * bounding worst-case work, for measuring the links' walk itself (a limit of INT32_MAX), and for
+ * testing the failure path without corrupting a BVH. */
 gsp_status gsp_scene_set_step_limit(gsp_scene* scene, int32_t max_box_tests);
 
 /* Per-vertex shading data (Sec. 3.1: the threaded BVH's triangle record carries a normal and
@@ -238,6 +241,10 @@ gsp_status gsp_build_bvh_device(gsp_scene* scene, int32_t link_sets, int32_t max
  * smallest (t, triangle index) among tmin < t < tmax, Moller-Trumbore in FP32; when the FP32
  * t of the winner may be inaccurate (origin far from the triangle compared with t, grazing
  * ray), its t and (u, v) are re-evaluated in FP64 from the exact vertices and rounded to FP32.
+ * A scene with six link sets, no step limit, a tree at most 38 levels deep and a bounding box
+ * diagonal of at most 1e8 is walked in the tree's four-wide form: each node holds the boxes of a
+ * binary node's grandchildren, the nearest one hit is visited next and the others wait on a stack
+ * (about a quarter of the fetches that depend on one another). Other scenes follow the hit/miss links.
  *  d_rays [n][8] float: ox, oy, oz, tmin, dx, dy, dz, tmax (d need not be unit length)
  *  d_tri  [n] int32 out: triangle index in the uploaded order, -1 on a miss
  *  d_t    [n] float out: hit distance (in units of |d|), +inf on a miss
@@ -327,7 +334,7 @@ gsp_status gsp_sppm_pass(gsp_sppm* r, int32_t npasses, void* stream);
  * traversal: GSP_TRAVERSAL_MTBVH (default) or GSP_TRAVERSAL_STACK for the persistent path kernel
  * (0 = keep); the closest hits, hence the results, are the same. The stack needs a tree less
  * than 64 levels deep (GSP_ERR_INVALID_ARG otherwise). */
-#define GSP_TRAVERSAL_MTBVH 1 /* the path kernel follows the hit/miss links (the paper's traversal) */
+#define GSP_TRAVERSAL_MTBVH 1 /* the path kernel walks the tree as gsp_trace_closest_hit does */
 #define GSP_TRAVERSAL_STACK 2 /* the path kernel walks the child-pair layout with a stack */
 gsp_status gsp_sppm_tune(gsp_sppm* r, int32_t eye_steps, int32_t photon_steps, float refine_factor,
                          int32_t gather_lanes, int32_t traversal);
@@ -459,7 +466,8 @@ gsp_status gsp_batch_autotune(gsp_batch* b, int32_t trial_passes, gsp_tune_resul
  * device, copies the counts accumulated since the previous call to h_counts [GSP_WORK_COUNTS]
  * (if not NULL), zeroes them, and switches counting on (on != 0) or off for the passes and
  * gradients that follow. Counting costs a few atomics per warp and per hit point; the estimate is
- * unchanged. It covers the persistent path kernels with the stackless traversal: GSP_ERR_BAD_STATE
+ * unchanged. While it is on, the path kernels follow the hit/miss links, whose box and triangle
+ * tests it counts (hits, hence renders, are the same). GSP_ERR_BAD_STATE
  * if the renderer traces some bounces as wavefront steps or walks with a stack
  * (gsp_sppm_tune), and while it counts, gsp_sppm_tune to those settings, gsp_sppm_autotune,
  * gsp_batch_autotune and gsp_batch_pass with this renderer fail with GSP_ERR_BAD_STATE. */

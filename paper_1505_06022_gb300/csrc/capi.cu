@@ -9,6 +9,7 @@
 #include "gsp_internal.h"
 #include "launch.h"
 #include "persist.cuh"
+#include "wide.cuh"
 
 namespace {
 thread_local std::string g_last_error;
@@ -48,8 +49,8 @@ k_trace(DevScene S, const float4* __restrict__ rays, int64_t n, const uint32_t* 
     Trav st;
     st.node = -1;
     st.slot = -1;
-    WarpQueue<> wq;
-    wq.init((int32_t)n);  // ray indices fit in 31 bits (the entry point rejects larger batches)
+    WarpQueue wq;
+    wq.init((int32_t)n, kTraceChunk);  // ray indices fit in 31 bits (the entry point rejects larger batches)
     int32_t ray = -1;
     int32_t pend = -1;  // leaf word of a postponed leaf, -1 = none
     uint32_t ntri = 0;  // not reported by this kernel
@@ -101,8 +102,8 @@ k_trace_stack(DevScene S, const float4* __restrict__ rays, int64_t n, int32_t* _
               int2* __restrict__ rlist, float refine_factor) {
     const int lane = threadIdx.x & 31;
     const uint32_t lt = lanemask_lt();
-    WarpQueue<> wq;
-    wq.init((int32_t)n);
+    WarpQueue wq;
+    wq.init((int32_t)n, kTraceChunk);
     Trav st;
     st.slot = -1;
     const int32_t cap = trav_cap(S);
@@ -127,6 +128,64 @@ k_trace_stack(DevScene S, const float4* __restrict__ rays, int64_t n, int32_t* _
             if (st.slot >= 0)
                 flag = hit_needs_refine(S.tris + 3 * st.slot, st.o, st.d, st.tbest, refine_factor, uv != nullptr, u, v);
             __stcs(tri + ray, st.best);
+            __stcs(tout + ray, st.best >= 0 ? st.tbest : __int_as_float(0x7f800000));
+            if (uv) __stcs(uv + ray, make_float2(u, v));
+        }
+        const uint32_t fm = __ballot_sync(0xffffffffu, flag);
+        if (fm) {
+            const int leader = __ffs(fm) - 1;
+            unsigned long long b = 0;
+            if (lane == leader) b = atomicAdd(ctr + 1, (unsigned long long)__popc(fm));
+            b = __shfl_sync(0xffffffffu, b, leader);
+            if (flag) rlist[b + __popc(fm & lt)] = make_int2((int)ray, st.slot);
+        }
+        if (fin) ray = -1;
+    }
+}
+
+// Closest hit through the four-wide form of the tree (wide.cuh): the kernel of scenes that have
+// one, with k_trace's work distribution, outputs and list of hits for FP64 re-evaluation.
+__global__ void __launch_bounds__(kTraceThreads, GSP_WIDE_MIN_BLOCKS)
+k_trace_wide(DevScene S, const float4* __restrict__ rays, int64_t n, const uint32_t* __restrict__ d_n,
+             int32_t* __restrict__ tri, float* __restrict__ tout, float2* __restrict__ uv,
+             unsigned long long* __restrict__ ctr, int2* __restrict__ rlist, float refine_factor, int32_t out_slot,
+             int32_t chunk) {
+    if (d_n) n = min(n, (int64_t)*d_n);
+    const int lane = threadIdx.x & 31;
+    const uint32_t lt = lanemask_lt();
+    __shared__ CoopScratch scratch[kTraceThreads / 32];
+    WarpQueue wq;
+    wq.init((int32_t)n, chunk);
+    WideRay st;
+    st.slot = -1;
+    WideWalk w;
+    int2 stk[kWideStack];
+    w.cur = kWalkDone;
+    w.sp = 0;
+    int32_t ray = -1;
+    while (true) {
+        const int32_t got = wq.take(ray < 0, ctr);
+        if (got >= 0) {
+            ray = got;
+            const float4 a = __ldcs(rays + 2 * (int64_t)ray), b = __ldcs(rays + 2 * (int64_t)ray + 1);
+            wide_ray(f3(a), f3(b), a.w, b.w, st);
+            wide_init(w);
+        }
+        if (__ballot_sync(0xffffffffu, ray >= 0) == 0) break;
+        const uint32_t act = __ballot_sync(0xffffffffu, ray >= 0);
+        if (wq.done && !(act & (act - 1))) {  // no rays left to take and one lane walks: all lanes walk its ray
+            st = coop_wide(S.wide, S.tris, st, w, stk, __ffs(act) - 1, &scratch[threadIdx.x >> 5]);
+            w.cur = kWalkDone;
+        } else {
+            wide_steps<GSP_WIDE_KEEP_TRACE>(S.wide, S.tris, st, w, stk, ray >= 0);
+        }
+        const bool fin = ray >= 0 && w.cur == kWalkDone;
+        bool flag = false;
+        if (fin) {
+            float u = 0.0f, v = 0.0f;
+            if (st.slot >= 0)
+                flag = hit_needs_refine(S.tris + 3 * st.slot, st.o, st.d, st.tbest, refine_factor, uv != nullptr, u, v);
+            __stcs(tri + ray, out_slot ? st.slot : st.best);
             __stcs(tout + ray, st.best >= 0 ? st.tbest : __int_as_float(0x7f800000));
             if (uv) __stcs(uv + ray, make_float2(u, v));
         }
@@ -190,6 +249,32 @@ int gsp_trace_grid(int device) {
     return g;
 }
 
+// The same for the four-wide kernel.
+static int trace_wide_grid(int device) {
+    static int cached[64] = {0};
+    if (device >= 0 && device < 64 && cached[device]) return cached[device];
+    int sms = 0, per_sm = 0;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, gspd::k_trace_wide, kTraceThreads, 0);
+    int g = std::max(1, sms) * std::max(1, per_sm);
+    if (device >= 0 && device < 64) cached[device] = g;
+    return g;
+}
+
+// The closest-hit kernel that S is walked with.
+static void run_trace(const gspd::DevScene& S, int device, const float4* rays, int64_t n, const uint32_t* d_n,
+                      int32_t* tri, float* t, float2* uv, unsigned long long* ctr, int2* rlist, float refine_factor,
+                      int32_t out_slot, cudaStream_t st) {
+    if (S.wide) {
+        constexpr int kWarps = kTraceThreads / 32;
+        const int64_t grid = std::min<int64_t>(trace_wide_grid(device), (n + kWarps - 1) / kWarps);
+        gspd::k_trace_wide<<<(unsigned)grid, kTraceThreads, 0, st>>>(S, rays, n, d_n, tri, t, uv, ctr, rlist, refine_factor,
+                                                                     out_slot, gsp_chunk(n, grid * kWarps, kTraceChunk));
+    } else
+        gspd::k_trace<<<gsp_trace_grid(device), kTraceThreads, 0, st>>>(S, rays, n, d_n, tri, t, uv, ctr, rlist,
+                                                                        refine_factor, out_slot);
+}
+
 // One closest-hit call on device buffers: counters zeroed, k_trace, FP64 refinement of the
 // flagged hits. ctr (2 u64) and rlist (n entries) belong to this call's stream.
 // With e0 and e1 (gsp_trace_time_launches), the two events bracket the k_trace launch alone.
@@ -201,9 +286,10 @@ static void launch_trace(const gsp_scene* s, const float4* rays, int64_t n, int3
     gspd::k_zero_u64x2<<<1, 1, 0, st>>>(ctr);
     const int grid = gsp_trace_grid(s->ctx->device);
     if (e0) cudaEventRecord(e0, st);
-    gspd::k_trace<<<grid, kTraceThreads, 0, st>>>(S, rays, n, nullptr, tri, t, uv, ctr, rlist, GSP_REFINE_FACTOR, 0);
+    run_trace(S, s->ctx->device, rays, n, nullptr, tri, t, uv, ctr, rlist, GSP_REFINE_FACTOR, 0, st);
     if (e1) cudaEventRecord(e1, st);
-    gspd::k_refine<<<std::max(1, grid / 2), 256, 0, st>>>(S, rays, rlist, ctr, t, uv);
+    gspd::k_refine<<<(unsigned)std::min<int64_t>(std::max(1, grid / 2), (n + 255) / 256), 256, 0, st>>>(S, rays, rlist, ctr,
+                                                                                                    t, uv);
 }
 
 cudaError_t gsp_trace_queue(const gsp_scene* s, const float4* rays, int64_t max_n, const uint32_t* d_n, int32_t* tri,
@@ -213,8 +299,7 @@ cudaError_t gsp_trace_queue(const gsp_scene* s, const float4* rays, int64_t max_
     const int grid = gsp_trace_grid(s->ctx->device);
     const bool list = refine_factor < INFINITY;
     if (list || zero_counters) gspd::k_zero_u64x2<<<1, 1, 0, st>>>(ctr);
-    gspd::k_trace<<<grid, kTraceThreads, 0, st>>>(S, rays, max_n, d_n, tri, t, nullptr, ctr, rlist, refine_factor,
-                                                  out_slot ? 1 : 0);
+    run_trace(S, s->ctx->device, rays, max_n, d_n, tri, t, nullptr, ctr, rlist, refine_factor, out_slot ? 1 : 0, st);
     if (list) gspd::k_refine<<<std::max(1, grid / 2), 256, 0, st>>>(S, rays, rlist, ctr, t, nullptr);
     return cudaGetLastError();
 }
@@ -225,6 +310,12 @@ gspd::DevScene gsp_dev_scene(const gsp_scene* s) {
     d.tris = s->d_tris;
     d.bin = s->d_bin;
     d.bin_root = s->bvh.bin_root;
+    // a step limit counts the box tests of the links' walk; a single link set is there to be walked
+    // in its one order (Fig. 4); and a deeper tree could need more than the wide walk's stack
+    d.wide = s->step_limit == 0 && s->bvh.link_sets == 6 && s->bvh.depth <= kWideMaxDepth &&
+                     s->extent <= kWideMaxExtent
+                 ? s->d_wide
+                 : nullptr;
     d.step_limit = s->step_limit;
     d.shade = s->d_shade;
     d.nlo = s->d_nlo;
@@ -326,6 +417,8 @@ static void scene_free_bvh(gsp_scene* s) {
     cudaFree(s->d_nodes);
     cudaFree(s->d_tris);
     cudaFree(s->d_bin);
+    cudaFree(s->d_wide);
+    s->d_wide = nullptr;
     s->d_nodes = nullptr;
     s->d_tris = nullptr;
     s->d_bin = nullptr;
@@ -598,6 +691,11 @@ gsp_status gsp_build_bvh(gsp_scene* s, const gsp_bvh_params* params, gsp_bvh_sta
         GSP_CUDA_TRY(cudaMalloc(&s->d_bin, bb));
         if (!bvh.bin.empty())
             GSP_CUDA_TRY(cudaMemcpy(s->d_bin, bvh.bin.data(), bvh.bin.size() * sizeof(float4), cudaMemcpyHostToDevice));
+        if (!bvh.wide.empty()) {
+            GSP_CUDA_TRY(cudaMalloc(&s->d_wide, bvh.wide.size() * sizeof(float4)));
+            GSP_CUDA_TRY(cudaMemcpy(s->d_wide, bvh.wide.data(), bvh.wide.size() * sizeof(float4), cudaMemcpyHostToDevice));
+            std::vector<float4>().swap(bvh.wide);  // only the device walks it
+        }
     }
     s->bvh = std::move(bvh);
     s->built = true;
@@ -861,11 +959,12 @@ gsp_status gsp_bvh_export(gsp_scene* s, int32_t set, float* h_nodes, float* h_tr
 
 }  // extern "C"
 
-void gsp_scene_adopt_bvh(gsp_scene* s, HostBVH&& bvh, float4* d_nodes, float4* d_tris, float4* d_bin) {
+void gsp_scene_adopt_bvh(gsp_scene* s, HostBVH&& bvh, float4* d_nodes, float4* d_tris, float4* d_bin, float4* d_wide) {
     scene_free_bvh(s);
     s->d_nodes = d_nodes;
     s->d_tris = d_tris;
     s->d_bin = d_bin;
+    s->d_wide = d_wide;
     s->device_bytes = (int64_t)((bvh.nodes.size() + bvh.tris.size()) * sizeof(float4)) + s->nt * (int64_t)sizeof(float4);
     s->bvh = std::move(bvh);
     s->built = true;

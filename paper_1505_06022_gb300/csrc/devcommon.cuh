@@ -106,6 +106,7 @@ struct DevScene {
     const float4* __restrict__ nlo;    // per triangle (upload order): FP32 remainder of the normal
     const float4* __restrict__ mats;   // 2 per material
     const float4* __restrict__ bin;    // child-pair layout of the same tree (stack traversal)
+    const float4* __restrict__ wide;   // four-wide form of the tree (wide.cuh); null: rays follow the links
     const float4* __restrict__ attr;   // per triangle (upload order): vertex normals + texture coordinates, or null
     const float4* __restrict__ texels; // albedo textures
     const int4* __restrict__ mtex;     // per material: {first texel, width, height, 0}, or null
@@ -346,15 +347,14 @@ __device__ __forceinline__ void refine_plane(const float4* __restrict__ tris, co
     if (plane_t(v0, nh, nl, o, d, tt)) t = tt;
 }
 
-// Traversal state of one ray (Fig. 3): current node in the ray's link set, best hit so far.
-struct Trav {
+// A ray and its best hit so far: triangle index in upload order, slot in leaf order (-1 = none).
+struct RayHit {
     float3 o, d, inv;
     float tmin, tbest;
-    int32_t best, slot, node, steps;
-    const float4* __restrict__ nodes;
+    int32_t best, slot;
 };
 
-__device__ __forceinline__ void trav_init(const DevScene& S, float3 o, float3 d, float tmin, float tmax, Trav& st) {
+__device__ __forceinline__ void ray_init(float3 o, float3 d, float tmin, float tmax, RayHit& st) {
     st.o = o;
     st.d = d;
     st.inv = make_float3(safe_inv(d.x), safe_inv(d.y), safe_inv(d.z));
@@ -362,6 +362,16 @@ __device__ __forceinline__ void trav_init(const DevScene& S, float3 o, float3 d,
     st.tbest = tmax;
     st.best = -1;
     st.slot = -1;
+}
+
+// Traversal state of one ray (Fig. 3): current node in the ray's link set.
+struct Trav : RayHit {
+    int32_t node, steps;
+    const float4* __restrict__ nodes;
+};
+
+__device__ __forceinline__ void trav_init(const DevScene& S, float3 o, float3 d, float tmin, float tmax, Trav& st) {
+    ray_init(o, d, tmin, tmax, st);
     st.node = 0;
     st.steps = 0;
     const int c = S.link_sets == 6 ? ray_class(d) : 0;
@@ -388,11 +398,11 @@ __device__ __forceinline__ bool tri_hit(float3 o, float3 d, const float4& P, con
 
 // Moller-Trumbore on the triangles [first, first + cnt) of the leaf-ordered triangle array,
 // keeping the lexicographic (t, triangle index) minimum over tmin < t < best t.
-__device__ __forceinline__ void trav_leaf(const DevScene& S, Trav& st, int32_t first, int32_t cnt) {
+__device__ __forceinline__ void trav_leaf(const float4* __restrict__ tris, RayHit& st, int32_t first, int32_t cnt) {
     for (int32_t k = 0; k < cnt; ++k) {
-        const float4 P = __ldg(S.tris + 3 * (first + k));
-        const float4 V1 = __ldg(S.tris + 3 * (first + k) + 1);
-        const float4 V2 = __ldg(S.tris + 3 * (first + k) + 2);
+        const float4 P = __ldg(tris + 3 * (first + k));
+        const float4 V1 = __ldg(tris + 3 * (first + k) + 1);
+        const float4 V2 = __ldg(tris + 3 * (first + k) + 2);
         float t;
         const int32_t id = __float_as_int(P.w);
         if (tri_hit(st.o, st.d, P, V1, V2, t) && t > st.tmin &&
@@ -402,6 +412,13 @@ __device__ __forceinline__ void trav_leaf(const DevScene& S, Trav& st, int32_t f
             st.slot = first + k;
         }
     }
+}
+
+// 32 bytes at a 32-byte aligned address as one 256-bit read-only vector load.
+__device__ __forceinline__ void ldg32(const float4* p, float4& A, float4& B) {
+    asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=f"(A.x), "=f"(A.y), "=f"(A.z), "=f"(A.w), "=f"(B.x), "=f"(B.y), "=f"(B.z), "=f"(B.w)
+        : "l"(p));
 }
 
 // 64 bytes at a 32-byte aligned address (two adjacent nodes, or a node's two child boxes) as two
@@ -422,7 +439,7 @@ __device__ __forceinline__ void ldg64(const float4* p, float4& A, float4& B, flo
 // t = b inv + (-o inv) saves six instructions per box but errs in absolute terms by about
 // u |o inv|, which needs a per-plane pad held in six more registers per ray; on GB300 the spills
 // and lost residency that cost made the traversal slower: 5,132 against 5,217 Mrays/s.)
-__device__ __forceinline__ bool slab(const Trav& st, float3 lo, float3 hi, float& tn) {
+__device__ __forceinline__ bool slab(const RayHit& st, float3 lo, float3 hi, float& tn) {
     const float3 o = st.o, inv = st.inv;
     const float t0x = __fmul_rn(lo.x - o.x, inv.x), t1x = __fmul_rn(hi.x - o.x, inv.x);
     const float t0y = __fmul_rn(lo.y - o.y, inv.y), t1y = __fmul_rn(hi.y - o.y, inv.y);
@@ -434,7 +451,7 @@ __device__ __forceinline__ bool slab(const Trav& st, float3 lo, float3 hi, float
 
 // Box test of a node {A, B} = {min.xyz, miss | max.xyz, leaf word} against [tmin, best t].
 // Returns true on a hit; `word` and `miss` receive the links.
-__device__ __forceinline__ bool box_hit(const Trav& st, const float4& A, const float4& B, int32_t& word, int32_t& miss) {
+__device__ __forceinline__ bool box_hit(const RayHit& st, const float4& A, const float4& B, int32_t& word, int32_t& miss) {
     float tn;
     miss = __float_as_int(A.w);
     word = __float_as_int(B.w);
@@ -443,7 +460,7 @@ __device__ __forceinline__ bool box_hit(const Trav& st, const float4& A, const f
 
 // Slab test of the box [lo, hi] as box_hit, with the entry distance (stack-based traversal
 // orders children by it).
-__device__ __forceinline__ bool box_entry(const Trav& st, float3 lo, float3 hi, float& tn) {
+__device__ __forceinline__ bool box_entry(const RayHit& st, float3 lo, float3 hi, float& tn) {
     return slab(st, lo, hi, tn);
 }
 
@@ -458,14 +475,14 @@ __device__ __forceinline__ void trav_step(const DevScene& S, Trav& st) {
     if (!box_hit(st, A, B, word, miss)) {
         st.node = miss;
     } else if (word >= 0) {
-        trav_leaf(S, st, word >> 3, word & 7);
+        trav_leaf(S.tris, st, word >> 3, word & 7);
         st.node = miss;
     } else {
         int32_t w2, m2;
         if (!box_hit(st, C, D, w2, m2)) {
             st.node = m2;
         } else if (w2 >= 0) {
-            trav_leaf(S, st, w2 >> 3, w2 & 7);
+            trav_leaf(S.tris, st, w2 >> 3, w2 & 7);
             st.node = m2;
         } else {
             st.node = st.node + 2;

@@ -26,8 +26,23 @@ struct HostBVH {
     // >= 0 is an internal node, < 0 is ~(leaf word). bin_root: ref of the root.
     std::vector<float4> bin;
     int32_t bin_root = 0;
+    // The same tree four-wide (wide.cuh): an entry of eight float4 per internal node of even depth,
+    // whose children are that node's grandchildren (or the child itself where it is a leaf).
+    // Empty for a tree that is a single leaf. The device build keeps none here.
+    std::vector<float4> wide;
     double build_ms = 0, thread_ms = 0;
 };
+
+// Centre and half extent of an interval of the four-wide tree's boxes: c - h <= lo and hi <= c + h
+// with h widened by kWideGrow (1 + 2^-19; wide.cuh says what that covers). lo <= hi.
+#ifdef __CUDACC__
+__host__ __device__
+#endif
+inline void gsp_wide_box(float lo, float hi, float& c, float& h) {
+    c = 0.5f * lo + 0.5f * hi;
+    const float a = hi - c, b = c - lo;  // each within one rounding (2^-24) of the exact value
+    h = (a > b ? a : b) * (1.0f + 0x1p-19f + 0x1p-22f);
+}
 
 // Builds the binned-SAH tree and writes its hit/miss links (one set per ray direction
 // class when link_sets == 6). Returns an empty string on success, else an error message.
@@ -62,6 +77,7 @@ struct gsp_scene {
     float4* d_nodes = nullptr;
     float4* d_tris = nullptr;
     float4* d_bin = nullptr;  // child-pair layout (HostBVH::bin)
+    float4* d_wide = nullptr;  // four-wide layout (HostBVH::wide); null if the tree is one leaf
     unsigned long long* d_counter = nullptr;  // trace kernel: next ray, refine-list length
     int2* d_rlist = nullptr;                  // trace kernel: hits re-evaluated in FP64
     int64_t rlist_cap = 0;
@@ -100,7 +116,7 @@ struct gsp_scene {
 
 // Installs a BVH built elsewhere (host copies + device arrays the scene takes ownership of),
 // replacing the scene's current one.
-void gsp_scene_adopt_bvh(gsp_scene* s, HostBVH&& bvh, float4* d_nodes, float4* d_tris, float4* d_bin);
+void gsp_scene_adopt_bvh(gsp_scene* s, HostBVH&& bvh, float4* d_nodes, float4* d_tris, float4* d_bin, float4* d_wide);
 
 // NVTX range around a host-side stage (header-only NVTX3: a no-op unless a profiler attaches).
 struct NvtxRange {

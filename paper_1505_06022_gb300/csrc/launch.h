@@ -17,6 +17,9 @@ constexpr int kTraceThreads = 128;
 #ifndef GSP_TRACE_MIN_BLOCKS
 #define GSP_TRACE_MIN_BLOCKS 9
 #endif
+#ifndef GSP_WIDE_MIN_BLOCKS
+#define GSP_WIDE_MIN_BLOCKS 8
+#endif
 #ifndef GSP_PATH_CHUNK
 #define GSP_PATH_CHUNK 32
 #endif
@@ -26,11 +29,28 @@ constexpr int kTraceThreads = 128;
 constexpr int kTraceChunk = GSP_TRACE_CHUNK;           // rays a warp takes from the global counter at once
 constexpr int kTraceInner = GSP_TRACE_INNER;           // traversal steps between refills
 constexpr int kTraceLeafBatch = GSP_TRACE_LEAF_BATCH;  // pending leaves that trigger a warp-wide leaf test
+constexpr int kWideStack = 64;     // children a walk of the four-wide tree may keep (at most three per wide level)
+constexpr int kWideMaxDepth = 38;  // depth of the binary tree up to which that is enough
+constexpr float kWideGrow = 1.0f + 0x1p-19f;  // half extents of its boxes are widened by this factor (wide.cuh)
+constexpr float kWideMaxExtent = 1e8f;  // larger scenes: (c - o) / d could overflow for a tiny d inside a box
 constexpr int kPathChunk = GSP_PATH_CHUNK;  // paths a warp of the path kernels takes at once (a block's
                                             // grid share is 128 paths: every warp of a short launch gets some)
 
 // Persistent grid size of the closest-hit kernel: SMs x resident blocks per SM.
 int gsp_trace_grid(int device);
+
+// Items a warp of a persistent kernel takes at once when `warps` warps share n of them: an equal
+// share while that leaves no warp more than its 32 lanes hold, else a quarter of it, so that warps
+// whose items end early take over from others, within 16 and most.
+#ifndef GSP_CHUNK_DIV
+#define GSP_CHUNK_DIV 4
+#endif
+inline int gsp_chunk(int64_t n, int64_t warps, int most) {
+    if (n <= 32 * warps) return (int)((n + warps - 1) / warps);
+    const int64_t c = n / (GSP_CHUNK_DIV * warps);
+    return (int)(c < 16 ? 16 : c > most ? most : c);
+}
+
 gspd::DevScene gsp_dev_scene(const gsp_scene* s);
 
 // Closest hit of rays already on the device (a wavefront queue) whose count is read from d_n.

@@ -8,6 +8,7 @@
 // Radix-tree numbering: internal nodes 0 .. n-2 (root 0), leaves n-1 .. 2n-2 (leaf n-1+i holds
 // the i-th triangle in Morton order). A node covers the sorted triangles [first, last].
 #include <algorithm>
+#include <cfloat>
 #include <chrono>
 #include <cmath>
 #include <cstring>
@@ -244,6 +245,56 @@ __global__ void k_child_pairs(int n, const int32_t* __restrict__ left, const int
     q[3] = make_float4(br.hi[0], br.hi[1], br.hi[2], 0.0f);
 }
 
+// Which internal nodes head an entry of the four-wide tree: those of the final tree at even depth.
+__global__ void k_wide_heads(int n, const int32_t* __restrict__ parent, const int32_t* __restrict__ first,
+                             const int32_t* __restrict__ last, int max_leaf, uint32_t* __restrict__ head) {
+    const int i = (int)((int64_t)blockIdx.x * blockDim.x + threadIdx.x);
+    if (i >= n - 1) return;
+    bool even = in_tree(i, parent, first, last, max_leaf) && !final_leaf(i, n, first, last, max_leaf);
+    if (even)
+        for (int p = parent[i]; p >= 0; p = parent[p]) even = !even;
+    head[i] = even ? 1u : 0u;
+}
+
+// The entries of the four-wide tree (layout in wide.cuh), numbered by a scan of the heads: a head's
+// grandchildren, or a child itself where it is a leaf.
+__global__ void k_wide_nodes(int n, const int32_t* __restrict__ left, const int32_t* __restrict__ right,
+                             const int32_t* __restrict__ first, const int32_t* __restrict__ last, int max_leaf,
+                             const Box* __restrict__ box, const uint32_t* __restrict__ head,
+                             const uint32_t* __restrict__ index, float4* __restrict__ wide) {
+    const int i = (int)((int64_t)blockIdx.x * blockDim.x + threadIdx.x);
+    if (i >= n - 1 || !head[i]) return;
+    int ch[4], m = 0;
+    for (int c : {left[i], right[i]}) {
+        if (final_leaf(c, n, first, last, max_leaf)) {
+            ch[m++] = c;
+        } else {
+            ch[m++] = left[c];
+            ch[m++] = right[c];
+        }
+    }
+    float* q = (float*)(wide + 8 * (size_t)index[i]);
+    for (int k = 0; k < 4; ++k) {
+        int32_t ref = INT32_MIN;  // no child
+        if (k < m) {
+            const int c = ch[k];
+            if (c >= n - 1)
+                ref = ~(((c - (n - 1)) << 3) | 1);
+            else if (final_leaf(c, n, first, last, max_leaf))
+                ref = ~((first[c] << 3) | (last[c] - first[c] + 1));
+            else
+                ref = (int32_t)index[c];
+        }
+        for (int a = 0; a < 3; ++a)
+            if (k < m)
+                gsp_wide_box(box[ch[k]].lo[a], box[ch[k]].hi[a], q[8 * a + k], q[8 * a + 4 + k]);
+            else
+                q[8 * a + k] = 0.0f, q[8 * a + 4 + k] = -FLT_MAX;  // near beyond far on every ray
+        q[24 + k] = __int_as_float(ref);
+        q[28 + k] = 0.0f;
+    }
+}
+
 }  // namespace
 
 extern "C" gsp_status gsp_build_bvh_device(gsp_scene* s, int32_t link_sets, int32_t max_leaf, gsp_bvh_stats* stats) {
@@ -274,7 +325,7 @@ extern "C" gsp_status gsp_build_bvh_device(gsp_scene* s, int32_t link_sets, int3
     };
     float* d_verts;
     int32_t *d_tris, *left, *right, *parent, *first, *last, *size, *d_depth;
-    uint32_t *ka, *va, *kb, *vb, *hist, *stemp, *d_n, *arrived;
+    uint32_t *ka, *va, *kb, *vb, *hist, *stemp, *d_n, *arrived, *head, *windex;
     Box* box;
     const int64_t nn = 2 * (int64_t)n - 1;
     A(&d_verts, 3 * s->nv);
@@ -284,7 +335,7 @@ extern "C" gsp_status gsp_build_bvh_device(gsp_scene* s, int32_t link_sets, int3
     A(&kb, nt);
     A(&vb, nt);
     A(&hist, gsp_sort_hist_elems());
-    A(&stemp, gsp_scan_temp_elems(gsp_sort_hist_elems()));
+    A(&stemp, std::max(gsp_scan_temp_elems(gsp_sort_hist_elems()), gsp_scan_temp_elems(n)));
     A(&d_n, 1);
     A(&left, std::max<int64_t>(1, n - 1));
     A(&right, std::max<int64_t>(1, n - 1));
@@ -295,6 +346,8 @@ extern "C" gsp_status gsp_build_bvh_device(gsp_scene* s, int32_t link_sets, int3
     A(&box, nn);
     A(&arrived, std::max<int64_t>(1, n - 1));
     A(&d_depth, 1);
+    A(&head, n);
+    A(&windex, n);  // [n - 1]: the number of wide nodes
     cudaEvent_t ev[3] = {nullptr, nullptr, nullptr};  // build and threading times
     auto drop_events = [&]() {
         for (cudaEvent_t& x : ev)
@@ -332,22 +385,31 @@ extern "C" gsp_status gsp_build_bvh_device(gsp_scene* s, int32_t link_sets, int3
     if (n > 1) k_internal<<<nblocks(n - 1), kThreads>>>(keys, n, left, right, parent, first, last);
     k_bottom_up<<<nblocks(n), kThreads>>>(d_verts, d_tris, ids, n, left, right, parent, first, last, max_leaf, box,
                                           size, arrived);
+    if (n > 1) {
+        k_wide_heads<<<nblocks(n - 1), kThreads>>>(n, parent, first, last, max_leaf, head);
+        e = gsp_scan_u32(head, windex, n - 1, windex + (n - 1), stemp, nullptr);
+    }
     int32_t nfinal = 0;
-    e = cudaGetLastError();
+    uint32_t nwide = 0;
+    if (e == cudaSuccess) e = cudaGetLastError();
+    if (e == cudaSuccess && n > 1)
+        e = cudaMemcpy(&nwide, windex + (n - 1), sizeof nwide, cudaMemcpyDeviceToHost);
     if (e == cudaSuccess) e = cudaMemcpy(&nfinal, size, sizeof nfinal, cudaMemcpyDeviceToHost);  // root: node 0
     if (e != cudaSuccess) return fail(e);
     cudaEventRecord(ev[1]);
     // final tree: nfinal nodes per link set (+ one padding node); triangles in Morton order
     const int64_t stride = (int64_t)nfinal + 1;
-    float4 *d_nodes = nullptr, *d_tri4 = nullptr, *d_bin = nullptr;
+    float4 *d_nodes = nullptr, *d_tri4 = nullptr, *d_bin = nullptr, *d_wide = nullptr;
     const int64_t nb = std::max<int64_t>(1, n - 1) * 4;
     e = cudaMalloc(&d_nodes, (size_t)link_sets * stride * 2 * sizeof(float4));
     if (e == cudaSuccess) e = cudaMalloc(&d_tri4, (size_t)nt * 3 * sizeof(float4));
     if (e == cudaSuccess) e = cudaMalloc(&d_bin, (size_t)nb * sizeof(float4));
+    if (e == cudaSuccess && nwide) e = cudaMalloc(&d_wide, (size_t)nwide * 8 * sizeof(float4));
     if (e != cudaSuccess) {
         cudaFree(d_nodes);
         cudaFree(d_tri4);
         cudaFree(d_bin);
+        cudaFree(d_wide);
         return fail(e);
     }
     // (n == 1: the single leaf is node 0 of the radix numbering, n - 1 + 0 = 0)
@@ -356,6 +418,7 @@ extern "C" gsp_status gsp_build_bvh_device(gsp_scene* s, int32_t link_sets, int3
     k_padding<<<1, 32>>>(link_sets, nfinal, stride, d_nodes);
     k_leaf_tris<<<nblocks(nt), kThreads>>>(d_verts, d_tris, ids, nt, d_tri4);
     k_child_pairs<<<nblocks(n), kThreads>>>(n, left, right, parent, first, last, max_leaf, box, d_bin);
+    if (nwide) k_wide_nodes<<<nblocks(n - 1), kThreads>>>(n, left, right, first, last, max_leaf, box, head, windex, d_wide);
     cudaEventRecord(ev[2]);
     e = cudaEventSynchronize(ev[2]);
     if (e == cudaSuccess) e = cudaGetLastError();
@@ -381,6 +444,7 @@ extern "C" gsp_status gsp_build_bvh_device(gsp_scene* s, int32_t link_sets, int3
         cudaFree(d_nodes);
         cudaFree(d_tri4);
         cudaFree(d_bin);
+        cudaFree(d_wide);
         return fail(e);
     }
     for (void* p : tmp) cudaFree(p);
@@ -403,7 +467,7 @@ extern "C" gsp_status gsp_build_bvh_device(gsp_scene* s, int32_t link_sets, int3
     bvh.link_sets = link_sets;
     bvh.build_ms = build_ms;
     bvh.thread_ms = thread_ms;
-    gsp_scene_adopt_bvh(s, std::move(bvh), d_nodes, d_tri4, d_bin);
+    gsp_scene_adopt_bvh(s, std::move(bvh), d_nodes, d_tri4, d_bin, d_wide);
     if (stats) {
         stats->nodes = s->bvh.nnodes;
         stats->leaves = s->bvh.nleaves;

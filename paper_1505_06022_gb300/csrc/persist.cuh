@@ -13,22 +13,22 @@ __device__ __forceinline__ uint32_t lanemask_lt() {
     return m;
 }
 
-// Work distribution of a persistent kernel over items [0, n). A warp takes CHUNK consecutive
+// Work distribution of a persistent kernel over items [0, n). A warp takes `chunk` consecutive
 // items at a time and hands them to its lanes as they become free, so a lane whose item has
 // finished starts the next one without waiting for the rest of the warp. Each warp's first chunk
 // is static (an empty or short launch costs no atomics); later chunks come from a counter that
 // the caller has zeroed and that counts past the static chunks. All fields are warp-uniform.
-template <int CHUNK = kTraceChunk>
 struct WarpQueue {
-    int32_t n, static_end, qbase, qend;
+    int32_t n, static_end, qbase, qend, chunk;
     bool done;
 
-    __device__ __forceinline__ void init(int32_t n_) {
+    __device__ __forceinline__ void init(int32_t n_, int32_t chunk_) {
         n = n_;
+        chunk = chunk_;
         const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-        static_end = (int32_t)min(warps * CHUNK, (int64_t)n);
-        qbase = (int32_t)min(((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * CHUNK, (int64_t)n);
-        qend = min(qbase + CHUNK, n);
+        static_end = (int32_t)min(warps * chunk, (int64_t)n);
+        qbase = (int32_t)min(((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * chunk, (int64_t)n);
+        qend = min(qbase + chunk, n);
         done = false;
     }
 
@@ -42,10 +42,10 @@ struct WarpQueue {
         while (m) {
             if (qbase >= qend) {
                 CounterT b = 0;
-                if (static_end < n && (threadIdx.x & 31) == 0) b = atomicAdd(ctr, (CounterT)CHUNK);
+                if (static_end < n && (threadIdx.x & 31) == 0) b = atomicAdd(ctr, (CounterT)chunk);
                 b = __shfl_sync(0xffffffffu, b, 0);
                 qbase = (int32_t)min((int64_t)static_end + (int64_t)b, (int64_t)n);
-                qend = min(qbase + CHUNK, n);
+                qend = min(qbase + chunk, n);
                 if (qbase >= n) {
                     done = true;
                     break;
@@ -117,7 +117,7 @@ __device__ __forceinline__ void trav_steps(const DevScene& S, Trav& st, int32_t&
         const uint32_t urgent = __ballot_sync(0xffffffffu, waiting || (pend >= 0 && st.node < 0));
         if (urgent || __popc(pm) >= kTraceLeafBatch) {
             if (pend >= 0) {
-                trav_leaf(S, st, pend >> 3, pend & 7);
+                trav_leaf(S.tris, st, pend >> 3, pend & 7);
                 ntri += (uint32_t)(pend & 7);
                 pend = -1;
             }
@@ -301,7 +301,7 @@ __device__ __forceinline__ void stack_steps(const DevScene& S, Trav& st, StackWa
                     w.node = stack_pop(st, w);
                 }
             } else {
-                trav_leaf(S, st, (~w.node) >> 3, (~w.node) & 7);
+                trav_leaf(S.tris, st, (~w.node) >> 3, (~w.node) & 7);
                 w.node = stack_pop(st, w);
             }
         }

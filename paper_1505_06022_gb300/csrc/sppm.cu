@@ -455,28 +455,39 @@ static void launch_gather_exact(int lanes, const GatherDev& G, const PassDev& P,
     }
 }
 
+// The form of the tree that the renderer's path kernels walk.
+static int path_walk(const gsp_sppm* r, const DevScene& S) {
+    if (r->traversal == GSP_TRAVERSAL_STACK) return kStack;
+    return S.wide && !r->count_work ? kWide : kLinks;  // work is counted in box tests of the links' walk
+}
+
 // Grid of a persistent path kernel (k_paths, or k_paths_multi when multi, of the given
 // instantiation): resident blocks on every SM, but no more warps than items.
-static int path_grid(int64_t items, int device, bool stack, bool shade, bool multi = false) {
-    static int per_sm[2][2][2][64] = {};
+static int path_grid(int64_t items, int device, int walk, bool shade, bool multi = false) {
+    static int per_sm[2][3][2][64] = {};
     static int sms[64] = {0};
     if (device < 0 || device >= 64) device = 0;
-    int& ps = per_sm[multi][stack][shade][device];
+    int& ps = per_sm[multi][walk][shade][device];
     if (!ps) {
-        const void* const kernels[2][2][2] = {
-            {{(const void*)k_paths<false, false, false>, (const void*)k_paths<false, true, false>},
-             {(const void*)k_paths<true, false, false>, (const void*)k_paths<true, true, false>}},
-            {{(const void*)k_paths_multi<false, false>, (const void*)k_paths_multi<false, true>},
-             {(const void*)k_paths_multi<true, false>, (const void*)k_paths_multi<true, true>}}};
+        const void* const kernels[2][3][2] = {
+            {{(const void*)k_paths<kLinks, false, false>, (const void*)k_paths<kLinks, true, false>},
+             {(const void*)k_paths<kStack, false, false>, (const void*)k_paths<kStack, true, false>},
+             {(const void*)k_paths<kWide, false, false>, (const void*)k_paths<kWide, true, false>}},
+            {{(const void*)k_paths_multi<kLinks, false>, (const void*)k_paths_multi<kLinks, true>},
+             {(const void*)k_paths_multi<kStack, false>, (const void*)k_paths_multi<kStack, true>},
+             {(const void*)k_paths_multi<kWide, false>, (const void*)k_paths_multi<kWide, true>}}};
         int b = 0;
         cudaDeviceGetAttribute(&sms[device], cudaDevAttrMultiProcessorCount, device);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, kernels[multi][stack][shade], kTraceThreads, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, kernels[multi][walk][shade], kTraceThreads, 0);
         ps = std::max(1, b);
     }
     const int64_t full = (int64_t)std::max(1, sms[device]) * ps;
-    const int64_t need = (items + kTraceThreads - 1) / kTraceThreads;
-    return (int)std::max<int64_t>(1, std::min(full, need));
+    const int64_t per = multi ? kTraceThreads : kTraceThreads / 32;  // items that justify a block
+    return (int)std::max<int64_t>(1, std::min(full, (items + per - 1) / per));
 }
+
+// Paths a warp of k_paths / k_photon_regen takes at once.
+static int path_chunk(int64_t items, unsigned grid) { return gsp_chunk(items, (int64_t)grid * (kTraceThreads / 32), kPathChunk); }
 
 // Eye pass up to the persistent kernel: primary rays, then eye_steps wavefront steps. Returns in
 // b the queue holding the paths still going (none if b > max_eye_depth).
@@ -530,17 +541,19 @@ static gsp_status photon_front(gsp_sppm* r, const PassDev& P, const DepositDev& 
     } else {
         RegenDev R{r->ro, r->rd, r->rphi, r->started};
         GSP_CUDA_TRY(cudaMemsetAsync(r->qctr + 13, 0, sizeof(uint32_t), st));
-        const bool stack = r->traversal == GSP_TRAVERSAL_STACK;
-        const unsigned grid = (unsigned)path_grid(r->np, r->scene->ctx->device, stack, false);
-        if (stack)
-            S.attr ? k_photon_regen<true, true, false><<<grid, kTraceThreads, 0, st>>>(S, E, P, D, R, r->qctr + 13)
-                   : k_photon_regen<true, false, false><<<grid, kTraceThreads, 0, st>>>(S, E, P, D, R, r->qctr + 13);
-        else if (P.work)  // counting the work (never with the stack walk)
-            S.attr ? k_photon_regen<false, true, true><<<grid, kTraceThreads, 0, st>>>(S, E, P, D, R, r->qctr + 13)
-                   : k_photon_regen<false, false, true><<<grid, kTraceThreads, 0, st>>>(S, E, P, D, R, r->qctr + 13);
+        const int walk = path_walk(r, S);
+        const unsigned grid = (unsigned)path_grid(r->np, r->scene->ctx->device, walk, false);
+        const auto regen = [&](auto kernel) {
+            kernel<<<grid, kTraceThreads, 0, st>>>(S, E, P, D, R, r->qctr + 13, path_chunk(r->np, grid));
+        };
+        if (walk == kStack)
+            S.attr ? regen(k_photon_regen<kStack, true, false>) : regen(k_photon_regen<kStack, false, false>);
+        else if (walk == kWide)
+            S.attr ? regen(k_photon_regen<kWide, true, false>) : regen(k_photon_regen<kWide, false, false>);
+        else if (P.work)
+            S.attr ? regen(k_photon_regen<kLinks, true, true>) : regen(k_photon_regen<kLinks, false, true>);
         else
-            S.attr ? k_photon_regen<false, true, false><<<grid, kTraceThreads, 0, st>>>(S, E, P, D, R, r->qctr + 13)
-                   : k_photon_regen<false, false, false><<<grid, kTraceThreads, 0, st>>>(S, E, P, D, R, r->qctr + 13);
+            S.attr ? regen(k_photon_regen<kLinks, true, false>) : regen(k_photon_regen<kLinks, false, false>);
     }
     return GSP_OK;
 }
@@ -576,17 +589,21 @@ static gsp_status stage_paths(gsp_sppm* r, const PassDev& P, const EyeOut& O, co
     gsp_status e = paths_front(r, P, O, D, st, J);
     if (e != GSP_OK) return e;
     if (J.nchunks > 0) {
-        const bool stack = r->traversal == GSP_TRAVERSAL_STACK;
-        const unsigned grid = (unsigned)path_grid((int64_t)J.nchunks * kMultiChunk, r->scene->ctx->device, stack, J.S.attr != nullptr);
-        if (stack)
-            J.S.attr ? k_paths<true, true, false><<<grid, kTraceThreads, 0, st>>>(J.S, P, J.qe, O, J.ne_ptr, J.qp, D, J.np_ptr, r->qctr + 12)
-                     : k_paths<true, false, false><<<grid, kTraceThreads, 0, st>>>(J.S, P, J.qe, O, J.ne_ptr, J.qp, D, J.np_ptr, r->qctr + 12);
-        else if (P.work)  // counting the work (never with the stack walk)
-            J.S.attr ? k_paths<false, true, true><<<grid, kTraceThreads, 0, st>>>(J.S, P, J.qe, O, J.ne_ptr, J.qp, D, J.np_ptr, r->qctr + 12)
-                     : k_paths<false, false, true><<<grid, kTraceThreads, 0, st>>>(J.S, P, J.qe, O, J.ne_ptr, J.qp, D, J.np_ptr, r->qctr + 12);
+        const int walk = path_walk(r, J.S);
+        const int64_t items = (J.ne_ptr ? r->npix : 0) + (J.np_ptr ? r->np : 0);
+        const unsigned grid = (unsigned)path_grid(items, r->scene->ctx->device, walk, J.S.attr != nullptr);
+        const auto paths = [&](auto kernel) {
+            kernel<<<grid, kTraceThreads, 0, st>>>(J.S, P, J.qe, O, J.ne_ptr, J.qp, D, J.np_ptr, r->qctr + 12,
+                                                   path_chunk(items, grid));
+        };
+        if (walk == kStack)
+            J.S.attr ? paths(k_paths<kStack, true, false>) : paths(k_paths<kStack, false, false>);
+        else if (walk == kWide)
+            J.S.attr ? paths(k_paths<kWide, true, false>) : paths(k_paths<kWide, false, false>);
+        else if (P.work)
+            J.S.attr ? paths(k_paths<kLinks, true, true>) : paths(k_paths<kLinks, false, true>);
         else
-            J.S.attr ? k_paths<false, true, false><<<grid, kTraceThreads, 0, st>>>(J.S, P, J.qe, O, J.ne_ptr, J.qp, D, J.np_ptr, r->qctr + 12)
-                     : k_paths<false, false, false><<<grid, kTraceThreads, 0, st>>>(J.S, P, J.qe, O, J.ne_ptr, J.qp, D, J.np_ptr, r->qctr + 12);
+            J.S.attr ? paths(k_paths<kLinks, true, false>) : paths(k_paths<kLinks, false, false>);
     }
     GSP_CUDA_TRY(cudaGetLastError());
     return GSP_OK;
@@ -960,7 +977,7 @@ static bool batch_scenes_unchanged(const gsp_batch* b) {
     if (b->captured.size() != b->rs.size()) return false;
     for (size_t i = 0; i < b->rs.size(); ++i) {
         const DevScene x = gsp_dev_scene(b->rs[i]->scene), &y = b->captured[i];
-        if (x.nodes != y.nodes || x.tris != y.tris || x.shade != y.shade || x.nlo != y.nlo || x.mats != y.mats ||
+        if (x.nodes != y.nodes || x.wide != y.wide || x.tris != y.tris || x.shade != y.shade || x.nlo != y.nlo || x.mats != y.mats ||
             x.bin != y.bin || x.attr != y.attr || x.texels != y.texels || x.mtex != y.mtex || x.nnodes != y.nnodes ||
             x.stride != y.stride || x.link_sets != y.link_sets || x.bin_root != y.bin_root ||
             x.step_limit != y.step_limit || x.status != y.status)
@@ -1022,9 +1039,12 @@ static gsp_status batch_capture_fused(gsp_batch* b, cudaStream_t st, int K, cuda
             gsp_status se = ensure_second_buffer(r);
             if (se != GSP_OK) return se;
         }
-    bool stack = true, shade = false;  // one launch for all: shading code if any scene has shading data
+    // one launch for all: shading code if any scene has shading data, the walk all renderers share
+    // (every scene has its links)
+    bool shade = false;
+    int walk = path_walk(b->rs[0], gsp_dev_scene(b->rs[0]->scene));
     for (gsp_sppm* r : b->rs) {
-        stack = stack && r->traversal == GSP_TRAVERSAL_STACK;
+        if (path_walk(r, gsp_dev_scene(r->scene)) != walk) walk = kLinks;
         shade = shade || r->scene->d_attr != nullptr;
     }
     const size_t base = K == 2 ? (size_t)n : 0;  // job tables and counters of this graph
@@ -1064,14 +1084,15 @@ static gsp_status batch_capture_fused(gsp_batch* b, cudaStream_t st, int K, cuda
         const PathJob* jt = b->d_jobs + base + (size_t)k * n;
         if (ce == cudaSuccess && total[k] > 0) {
             ce = cudaMemsetAsync(ctr, 0, sizeof(uint32_t), ps);
-            const unsigned grid = (unsigned)path_grid((int64_t)total[k] * kMultiChunk, b->device, stack, shade, true);
+            const unsigned grid = (unsigned)path_grid((int64_t)total[k] * kMultiChunk, b->device, walk, shade, true);
             if (ce == cudaSuccess) {
-                if (stack)
-                    shade ? k_paths_multi<true, true><<<grid, kTraceThreads, 0, ps>>>(jt, n, total[k], ctr)
-                          : k_paths_multi<true, false><<<grid, kTraceThreads, 0, ps>>>(jt, n, total[k], ctr);
+                const auto multi = [&](auto kernel) { kernel<<<grid, kTraceThreads, 0, ps>>>(jt, n, total[k], ctr); };
+                if (walk == kStack)
+                    shade ? multi(k_paths_multi<kStack, true>) : multi(k_paths_multi<kStack, false>);
+                else if (walk == kWide)
+                    shade ? multi(k_paths_multi<kWide, true>) : multi(k_paths_multi<kWide, false>);
                 else
-                    shade ? k_paths_multi<false, true><<<grid, kTraceThreads, 0, ps>>>(jt, n, total[k], ctr)
-                          : k_paths_multi<false, false><<<grid, kTraceThreads, 0, ps>>>(jt, n, total[k], ctr);
+                    shade ? multi(k_paths_multi<kLinks, true>) : multi(k_paths_multi<kLinks, false>);
                 ce = cudaGetLastError();
             }
         }

@@ -8,6 +8,7 @@
 #include "gsp_internal.h"
 #include "launch.h"
 #include "persist.cuh"
+#include "wide.cuh"
 
 // resident blocks per SM of the path kernels beside GSP_PATH_MIN_BLOCKS (launch.h)
 #ifndef GSP_PATH_SHADE_MIN_BLOCKS  // path kernels of scenes with shading data (72 registers)
@@ -179,8 +180,8 @@ __device__ __forceinline__ int32_t slot_refine(const DevScene& S, float3 o, floa
     return id;
 }
 
-// Closest hit of a finished walk (trav_steps), t refined as above.
-__device__ __forceinline__ Hit walk_hit(const DevScene& S, const Trav& st) {
+// Closest hit of a finished walk, t refined as above.
+__device__ __forceinline__ Hit walk_hit(const DevScene& S, const RayHit& st) {
     Hit h;
     h.id = st.best;
     h.t = st.tbest;
@@ -270,6 +271,81 @@ __device__ __forceinline__ Surf surface(const DevScene& S, const Hit& h, float3 
     sf.smooth = false;
     return sf;
 }
+
+// One lane's walk in a persistent path kernel, by one of the tree's forms: the hit/miss links, the
+// child pairs with a stack, or the four-wide nodes.
+enum { kLinks, kStack, kWide };
+
+template <int WALK>
+struct PathWalk;
+
+template <>
+struct PathWalk<kLinks> {
+    Trav st;
+    int32_t pend;
+    __device__ __forceinline__ PathWalk() {
+        st.node = st.slot = -1;
+        pend = -1;
+    }
+    __device__ __forceinline__ void start(const DevScene& S, float3 o, float3 d, float tmin) {
+        trav_init(S, o, d, tmin, __int_as_float(0x7f800000), st);
+    }
+    __device__ __forceinline__ void steps(const DevScene& S, bool active, int32_t cap, uint32_t& ntri) {
+        trav_steps(S, st, pend, active, cap, ntri);
+    }
+    __device__ __forceinline__ bool done() const { return st.node < 0 && pend < 0; }
+    // Every lane calls it; lane `owner` is the only one with a path.
+    __device__ __forceinline__ void finish(const DevScene& S, int owner, int32_t cap, CoopScratch*, uint32_t& ntri) {
+        const CoopWalk r = coop_walk(S.tris, S.nnodes, S.status, st, pend, owner, cap);
+        st = r.st;
+        pend = -1;
+        if ((threadIdx.x & 31) == owner) ntri += r.ntri;
+    }
+};
+
+template <>
+struct PathWalk<kStack> {
+    Trav st;
+    StackWalk sw;
+    __device__ __forceinline__ PathWalk() {
+        st.slot = -1;
+        sw.node = kWalkDone;
+        sw.sp = 0;
+    }
+    __device__ __forceinline__ void start(const DevScene& S, float3 o, float3 d, float tmin) {
+        trav_init(S, o, d, tmin, __int_as_float(0x7f800000), st);
+        stack_init(S, sw);
+    }
+    __device__ __forceinline__ void steps(const DevScene& S, bool active, int32_t cap, uint32_t&) {
+        stack_steps(S, st, sw, active, cap);
+    }
+    __device__ __forceinline__ bool done() const { return sw.node == kWalkDone; }
+};
+
+template <>
+struct PathWalk<kWide> {
+    WideRay st;
+    WideWalk w;
+    int2 stk[kWideStack];
+    __device__ __forceinline__ PathWalk() {
+        st.slot = -1;
+        w.cur = kWalkDone;
+        w.sp = 0;
+    }
+    __device__ __forceinline__ void start(const DevScene&, float3 o, float3 d, float tmin) {
+        wide_ray(o, d, tmin, __int_as_float(0x7f800000), st);
+        st.pad = 0.0f;  // tmin >= 0
+        wide_init(w);
+    }
+    __device__ __forceinline__ void steps(const DevScene& S, bool active, int32_t, uint32_t&) {
+        wide_steps<GSP_WIDE_KEEP>(S.wide, S.tris, st, w, stk, active);
+    }
+    __device__ __forceinline__ bool done() const { return w.cur == kWalkDone; }
+    __device__ __forceinline__ void finish(const DevScene& S, int owner, int32_t, CoopScratch* sc, uint32_t&) {
+        st = coop_wide(S.wide, S.tris, st, w, stk, owner, sc);
+        w.cur = kWalkDone;
+    }
+};
 
 // Appends the lanes with `keep` set to queue Q (warp-aggregated: one atomic per warp).
 __device__ __forceinline__ void queue_push(const PathQ& Q, uint32_t* count, bool keep, float3 o, float tmin, float3 d,
@@ -594,27 +670,23 @@ k_photon_shade(DevScene S, PassDev P, DepositDev D, PathQ cur, PathQ nxt, uint32
 // have depth <= max_eye, photon entries depth < max_photon (the host launches accordingly).
 // Once nothing is left to take, a path left alone in its warp has its walks done by all lanes
 // (coop_walk).
-// STACK: walk the child-pair layout with a stack (StackWalk) instead of the hit/miss links.
-// COUNT: add the work of the launch to P.work (the instantiation used only while counting, so
-// that the counters take no registers in the others).
-template <bool STACK, bool SHADE, bool COUNT>
+// WALK: the form of the tree that is walked (PathWalk). COUNT: add the work of the launch to P.work
+// (links only; the instantiation used only while counting, so that the counters take no registers
+// in the others). chunk: paths a warp takes at once.
+template <int WALK, bool SHADE, bool COUNT>
 __global__ void __launch_bounds__(kTraceThreads, SHADE ? GSP_PATH_SHADE_MIN_BLOCKS : GSP_PATH_MIN_BLOCKS)
 k_paths(DevScene S, PassDev P, PathQ qe, EyeOut O, const uint32_t* __restrict__ ne_ptr, PathQ qp, DepositDev D,
-        const uint32_t* __restrict__ np_ptr, uint32_t* __restrict__ ctr) {
+        const uint32_t* __restrict__ np_ptr, uint32_t* __restrict__ ctr, int32_t chunk) {
+    __shared__ CoopScratch scratch[WALK == kWide ? kTraceThreads / 32 : 1];
     const int32_t cap = trav_cap(S);
     const int32_t ne = ne_ptr ? (int32_t)*ne_ptr : 0;
     const int32_t nph = np_ptr ? (int32_t)*np_ptr : 0;
-    WarpQueue<kPathChunk> wq;
-    wq.init(ne + nph);
-    Trav st;
-    st.node = -1;
-    st.slot = -1;
-    int32_t i = -1, pend = -1, id = 0, depth = 0;
+    WarpQueue wq;
+    wq.init(ne + nph, chunk);
+    PathWalk<WALK> pw;
+    int32_t i = -1, id = 0, depth = 0;
     uint32_t ndep = 0;
     bool eye = false;
-    StackWalk sw;
-    sw.node = kWalkDone;
-    sw.sp = 0;
     float3 w = make_float3(0.0f, 0.0f, 0.0f);  // eye: throughput; photon: flux
     Rng rng;
     uint32_t c_eye = 0, c_ph = 0, c_nodes = 0, c_tris = 0;  // work of this lane
@@ -632,21 +704,24 @@ k_paths(DevScene S, PassDev P, PathQ qe, EyeOut O, const uint32_t* __restrict__ 
             rng = rng_from(Q.rng[j]);
             depth = eye ? meta : (meta & 0xff);
             ndep = eye ? 0u : (uint32_t)(meta >> 8);
-            trav_init(S, f3(a), f3(c), eye ? a.w : P.eps, __int_as_float(0x7f800000), st);
-            if (STACK) stack_init(S, sw);
+            pw.start(S, f3(a), f3(c), eye ? a.w : P.eps);
         }
-        if (__ballot_sync(0xffffffffu, i >= 0) == 0) break;
-        if (STACK)
-            stack_steps(S, st, sw, i >= 0, cap);
-        else
-            trav_steps(S, st, pend, i >= 0, cap, c_tris);
-        const bool walked = STACK ? sw.node == kWalkDone : (st.node < 0 && pend < 0);
-        if (i >= 0 && walked) {
-            const Hit h = walk_hit(S, st);
-            float3 o = st.o, d = st.d;
+        const uint32_t act = __ballot_sync(0xffffffffu, i >= 0);
+        if (act == 0) break;
+        bool lone = false;  // nothing left to take: a path left alone in the warp walks with all lanes
+        if constexpr (WALK != kStack) {
+            if (wq.done && !(act & (act - 1))) {
+                pw.finish(S, __ffs(act) - 1, cap, &scratch[WALK == kWide ? threadIdx.x >> 5 : 0], c_tris);
+                lone = true;
+            }
+        }
+        if (!lone) pw.steps(S, i >= 0, cap, c_tris);
+        if (i >= 0 && pw.done()) {
+            const Hit h = walk_hit(S, pw.st);
+            float3 o = pw.st.o, d = pw.st.d;
             bool more = false;
             if (COUNT) {
-                c_nodes += (uint32_t)st.steps;
+                if constexpr (WALK != kWide) c_nodes += (uint32_t)pw.st.steps;
                 c_eye += eye ? 1u : 0u;
                 c_ph += eye ? 0u : 1u;
             }
@@ -660,22 +735,10 @@ k_paths(DevScene S, PassDev P, PathQ qe, EyeOut O, const uint32_t* __restrict__ 
                 }
                 if (!more) D.pcount[id] = ndep;
             }
-            if (more) {
-                trav_init(S, o, d, P.eps, __int_as_float(0x7f800000), st);
-                if (STACK) stack_init(S, sw);
-            } else {
+            if (more)
+                pw.start(S, o, d, P.eps);
+            else
                 i = -1;
-            }
-        }
-        if (!STACK && wq.done) {  // nothing left to take: a path left alone in the warp walks with all lanes
-            const uint32_t act = __ballot_sync(0xffffffffu, i >= 0);
-            if (act && !(act & (act - 1)) && __shfl_sync(0xffffffffu, max(st.node, pend), __ffs(act) - 1) >= 0) {
-                const int owner = __ffs(act) - 1;
-                const CoopWalk r = coop_walk(S.tris, S.nnodes, S.status, st, pend, owner, cap);
-                st = r.st;
-                pend = -1;
-                if (COUNT && (threadIdx.x & 31) == owner) c_tris += r.ntri;
-            }
         }
     }
     if (COUNT) {  // the whole warp leaves the loop together
@@ -770,18 +833,13 @@ struct MultiQueue {
     }
 };
 
-template <bool STACK, bool SHADE>
+template <int WALK, bool SHADE>
 __global__ void __launch_bounds__(kTraceThreads, SHADE ? GSP_PATH_SHADE_MIN_BLOCKS : GSP_PATH_MULTI_MIN_BLOCKS)
 k_paths_multi(const PathJob* __restrict__ jobs, int32_t njobs, int32_t total_chunks, uint32_t* __restrict__ ctr) {
     MultiQueue mq;
     mq.init(jobs, njobs, total_chunks);
-    Trav st;
-    st.node = -1;
-    st.slot = -1;
-    StackWalk sw;
-    sw.node = kWalkDone;
-    sw.sp = 0;
-    int32_t i = -1, jb = 0, pend = -1, id = 0, depth = 0, cap = 0;
+    PathWalk<WALK> pw;
+    int32_t i = -1, jb = 0, id = 0, depth = 0, cap = 0;
     uint32_t ndep = 0;
     bool eye = false;
     float3 w = make_float3(0.0f, 0.0f, 0.0f);  // eye: throughput; photon: flux
@@ -803,20 +861,15 @@ k_paths_multi(const PathJob* __restrict__ jobs, int32_t njobs, int32_t total_chu
             depth = eye ? meta : (meta & 0xff);
             ndep = eye ? 0u : (uint32_t)(meta >> 8);
             cap = trav_cap(J.S);
-            trav_init(J.S, f3(a), f3(c), eye ? a.w : J.P.eps, __int_as_float(0x7f800000), st);
-            if (STACK) stack_init(J.S, sw);
+            pw.start(J.S, f3(a), f3(c), eye ? a.w : J.P.eps);
         }
         if (__ballot_sync(0xffffffffu, i >= 0) == 0) break;
         const PathJob& J = jobs[jb];
         uint32_t ntri = 0;  // work is not counted in batched passes
-        if (STACK)
-            stack_steps(J.S, st, sw, i >= 0, cap);
-        else
-            trav_steps(J.S, st, pend, i >= 0, cap, ntri);
-        const bool walked = STACK ? sw.node == kWalkDone : (st.node < 0 && pend < 0);
-        if (i >= 0 && walked) {
-            const Hit h = walk_hit(J.S, st);
-            float3 o = st.o, d = st.d;
+        pw.steps(J.S, i >= 0, cap, ntri);
+        if (i >= 0 && pw.done()) {
+            const Hit h = walk_hit(J.S, pw.st);
+            float3 o = pw.st.o, d = pw.st.d;
             bool more = false;
             if (eye) {
                 more = h.id >= 0 && eye_interact<SHADE>(J.S, J.P, J.O, id, h, o, d, w, rng) && ++depth <= J.P.max_eye;
@@ -828,12 +881,10 @@ k_paths_multi(const PathJob* __restrict__ jobs, int32_t njobs, int32_t total_chu
                 }
                 if (!more) J.D.pcount[id] = ndep;
             }
-            if (more) {
-                trav_init(J.S, o, d, J.P.eps, __int_as_float(0x7f800000), st);
-                if (STACK) stack_init(J.S, sw);
-            } else {
+            if (more)
+                pw.start(J.S, o, d, J.P.eps);
+            else
                 i = -1;
-            }
         }
     }
 }
@@ -848,20 +899,16 @@ struct RegenDev {
 // One bounce per thread and pass (Sec. 3.3): thread j continues its stored path, or starts a new
 // one when the stored path has ended (N_e counts the starts), traces exactly one ray, deposits at
 // a diffuse hit and stores the path state for the next pass. Persistent, with per-lane refill
-// over the threads (counter *ctr) as the path kernel; STACK and COUNT as in k_paths.
-template <bool STACK, bool SHADE, bool COUNT>
+// over the threads (counter *ctr) as the path kernel; WALK, COUNT and chunk as in k_paths.
+template <int WALK, bool SHADE, bool COUNT>
 __global__ void __launch_bounds__(kTraceThreads, GSP_PATH_MIN_BLOCKS)
-k_photon_regen(DevScene S, EmitDev E, PassDev P, DepositDev D, RegenDev R, uint32_t* __restrict__ ctr) {
+k_photon_regen(DevScene S, EmitDev E, PassDev P, DepositDev D, RegenDev R, uint32_t* __restrict__ ctr,
+               int32_t chunk) {
     const int32_t cap = trav_cap(S);
-    WarpQueue<kPathChunk> wq;
-    wq.init((int32_t)P.np);
-    Trav st;
-    st.node = -1;
-    st.slot = -1;
-    StackWalk sw;
-    sw.node = kWalkDone;
-    sw.sp = 0;
-    int32_t j = -1, pend = -1, depth = 0;
+    WarpQueue wq;
+    wq.init((int32_t)P.np, chunk);
+    PathWalk<WALK> pw;
+    int32_t j = -1, depth = 0;
     uint32_t starts = 0;
     uint32_t c_ph = 0, c_nodes = 0, c_tris = 0;  // work of this lane
     float3 phi = make_float3(0.0f, 0.0f, 0.0f);
@@ -880,22 +927,17 @@ k_photon_regen(DevScene S, EmitDev E, PassDev P, DepositDev D, RegenDev R, uint3
                 depth = 0;
                 ++starts;
             }
-            trav_init(S, o, d, P.eps, __int_as_float(0x7f800000), st);
-            if (STACK) stack_init(S, sw);
+            pw.start(S, o, d, P.eps);
         }
         if (__ballot_sync(0xffffffffu, j >= 0) == 0) break;
-        if (STACK)
-            stack_steps(S, st, sw, j >= 0, cap);
-        else
-            trav_steps(S, st, pend, j >= 0, cap, c_tris);
-        const bool walked = STACK ? sw.node == kWalkDone : (st.node < 0 && pend < 0);
-        if (j >= 0 && walked) {
+        pw.steps(S, j >= 0, cap, c_tris);
+        if (j >= 0 && pw.done()) {
             if (COUNT) {
                 c_ph += 1;
-                c_nodes += (uint32_t)st.steps;
+                if constexpr (WALK != kWide) c_nodes += (uint32_t)pw.st.steps;
             }
-            const Hit h = walk_hit(S, st);
-            float3 o = st.o, d = st.d;
+            const Hit h = walk_hit(S, pw.st);
+            float3 o = pw.st.o, d = pw.st.d;
             uint32_t ndep = 0;
             bool alive = h.id >= 0 && photon_bounce<SHADE>(S, P, D, rng, h, o, d, phi, (uint32_t)j, (uint32_t)j, ndep) &&
                          ++depth < P.max_photon;

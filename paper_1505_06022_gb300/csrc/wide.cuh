@@ -1,0 +1,264 @@
+// wide.cuh -- traversal of the tree's four-wide form: the walk that answers closest-hit queries
+// wherever nothing asks for the hit/miss links themselves (gsp_dev_scene decides).
+//
+// A wide node stands for a binary node of even depth and holds its up to four grandchildren (a
+// child that is a leaf stands for itself): their boxes as centres and half extents, plane by
+// plane, and a reference per child -- eight float4, 128 bytes, one cache line:
+//   {c.x}x4 {h.x}x4 | {c.y}x4 {h.y}x4 | {c.z}x4 {h.z}x4 | {ref}x4, unused
+// ref >= 0 is a wide node, < 0 is ~(leaf word), kWalkDone no child. Leaves are the binary tree's,
+// and the hit is the lexicographic (t, index) minimum of the same triangle tests, so the result
+// does not depend on the form walked.
+//
+// What bounds a walk is the chain of dependent node fetches and the instructions per box. The links
+// visit 53 boxes for a bounce ray of the 247,234-triangle scene (two per fetch at best) and need six
+// copies of the nodes; the wide form makes 13 node fetches for the same ray from one copy (20 MB
+// instead of 123 MB for a million triangles, so that it stays in L2). Four children rather than
+// eight: eight would make 9 fetches but test 72 boxes for 52, and the trees fill 3.1 of 4 slots but
+// 3.4 of 8. Measured against the links: 4,194,304 rays over 1,003,520 triangles 815 -> 596 us,
+// 262,147 rays over 247,234 triangles 138 -> 86 us, 1,021 rays 64 -> 24 us (with the last ray of a
+// warp walked by all lanes, below), a 512x512 pass 1.30 -> 1.00 ms, a 131x97 one 752 -> 430 us.
+#pragma once
+
+#include "launch.h"
+#include "persist.cuh"
+
+#ifndef GSP_WIDE_KEEP
+#define GSP_WIDE_KEEP 1
+#endif
+#ifndef GSP_WIDE_KEEP_TRACE
+#define GSP_WIDE_KEEP_TRACE 2
+#endif
+#ifndef GSP_WIDE_LEAF_BATCH
+#define GSP_WIDE_LEAF_BATCH 12
+#endif
+
+namespace gspd {
+
+constexpr int kWideLeafBatch = GSP_WIDE_LEAF_BATCH;  // lanes at a leaf that trigger a warp-wide leaf test
+
+// Slab interval of the box c +- h along one axis: tc = (c - o) inv, tc -+ h |inv|. With unit
+// roundoff u and an inverse good to 2u, either end is off by at most 5u |tc| + 3u h |inv|. Where
+// |tc| <= 2 h |inv| that is below the 32u h |inv| by which the builders widen h (kWideGrow); else
+// both ends have the sign of tc and a relative error of at most 13u, which the far end's factor
+// kWideFar = 1 + 32u covers. The test is conservative then, for t >= 0; for a negative tmin the
+// pad adds 64u |tmin|, more than the factor takes off a negative far end. Two operations of the
+// half-rate min/max pipe fewer per axis and box than min and max over the two planes: that pipe
+// was the busiest at 57-61 % of its cycles.
+constexpr float kWideFar = 1.0f + 0x1p-19f;
+
+struct WideRay : RayHit {
+    float pad;
+};
+
+// 1 / d to 1 ulp (2u): all that the slab test needs.
+__device__ __forceinline__ float wide_inv(float d) {
+    float r;
+    asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(fabsf(d) < 1e-30f ? copysignf(1e-30f, d) : d));
+    return r;
+}
+
+__device__ __forceinline__ void wide_ray(float3 o, float3 d, float tmin, float tmax, WideRay& st) {
+    st.o = o;
+    st.d = d;
+    st.inv = make_float3(wide_inv(d.x), wide_inv(d.y), wide_inv(d.z));
+    st.tmin = tmin;
+    st.tbest = tmax;
+    st.best = -1;
+    st.slot = -1;
+    st.pad = fmaxf(-tmin, 0.0f) * 0x1p-18f;
+}
+
+// One ray's walk: the node or leaf it is at (kWalkDone: the walk is over) and the children still
+// to visit, each with its key (entry distance; the two low bits hold the child number).
+// The stack is an array beside it, so that passing its address on does not hold these in memory.
+struct WideWalk {
+    int32_t cur, sp;
+};
+
+__device__ __forceinline__ void wide_init(WideWalk& w) {
+    w.cur = 0;
+    w.sp = 0;
+}
+
+constexpr int32_t kWideMiss = 0x7fffffff;  // sorts behind every key
+
+// Whether a child with this key may still hold a closer hit. Dropping the low bits rounds a
+// distance down unless it is negative (negative tmin, origin inside the box): never culled then.
+__device__ __forceinline__ bool wide_keep(int32_t key, float tbest) {
+    return key < 0 || __int_as_float(key & ~3) <= tbest;
+}
+
+__device__ __forceinline__ int32_t wide_pop(const RayHit& st, WideWalk& w, const int2* stk) {
+    while (w.sp > 0) {
+        const int2 e = stk[--w.sp];
+        if (wide_keep(e.x, st.tbest)) return e.y;
+    }
+    return kWalkDone;
+}
+
+// Key of child i: the bits of its entry distance with the child number in the two low bits, or
+// kWideMiss. Signed order is the order of the distances where they are not negative.
+__device__ __forceinline__ int32_t wide_key(const WideRay& st, float cx, float hx, float cy, float hy, float cz,
+                                            float hz, int i) {
+    const float tx = __fmul_rn(cx - st.o.x, st.inv.x), ty = __fmul_rn(cy - st.o.y, st.inv.y),
+                tz = __fmul_rn(cz - st.o.z, st.inv.z);
+    const float ax = fabsf(st.inv.x), ay = fabsf(st.inv.y), az = fabsf(st.inv.z);
+    const float tn = max3f(__fmaf_rn(-hx, ax, tx), __fmaf_rn(-hy, ay, ty), fmaxf(__fmaf_rn(-hz, az, tz), st.tmin));
+    const float tf = min3f(__fmaf_rn(hx, ax, tx), __fmaf_rn(hy, ay, ty), __fmaf_rn(hz, az, tz));
+    return tn <= __fmaf_rn(fminf(st.tbest, tf), kWideFar, st.pad) ? ((__float_as_int(tn) & ~3) | i) : kWideMiss;
+}
+
+__device__ __forceinline__ void wide_push(WideWalk& w, int2* stk, int32_t key, int32_t nearest, int32_t ref) {
+    if (key != kWideMiss && key != nearest) stk[w.sp++] = make_int2(key, ref);
+}
+
+// Tests the four children of node w.cur and moves to the nearest hit one; the others go on the
+// stack as they come (sorting them too saves under 1 % of the visits and costs more).
+__device__ __forceinline__ void wide_node(const float4* __restrict__ nodes, const WideRay& st, WideWalk& w, int2* stk) {
+    const float4* p = nodes + 8 * (int64_t)w.cur;
+    float4 cx, hx, cy, hy, cz, hz;
+    ldg32(p, cx, hx);
+    ldg32(p + 2, cy, hy);
+    ldg32(p + 4, cz, hz);
+    const int4 ref = __ldg((const int4*)(p + 6));
+    const int32_t k0 = wide_key(st, cx.x, hx.x, cy.x, hy.x, cz.x, hz.x, 0);
+    const int32_t k1 = wide_key(st, cx.y, hx.y, cy.y, hy.y, cz.y, hz.y, 1);
+    const int32_t k2 = wide_key(st, cx.z, hx.z, cy.z, hy.z, cz.z, hz.z, 2);
+    const int32_t k3 = wide_key(st, cx.w, hx.w, cy.w, hy.w, cz.w, hz.w, 3);
+    const int32_t k = min(min(k0, k1), min(k2, k3));
+    if (k == kWideMiss) {
+        w.cur = wide_pop(st, w, stk);
+        return;
+    }
+    wide_push(w, stk, k0, k, ref.x);
+    wide_push(w, stk, k1, k, ref.y);
+    wide_push(w, stk, k2, k, ref.z);
+    wide_push(w, stk, k3, k, ref.w);
+    const int32_t a = k & 1 ? ref.y : ref.x, b = k & 1 ? ref.w : ref.z;
+    w.cur = k & 2 ? b : a;
+}
+
+// Walks the warp's active lanes until no more than KEEP quarters of them still walk: what follows a
+// walk then runs for many lanes at once. A path kernel's shading is long (1 of 4; 8.0 ms per eight
+// 512x512 passes, against 8.07 with 2 and 8.33 with 3), a ray's end in the closest-hit kernel short
+// (2; 3 costs 1 %, 1 costs 8 %). Lanes at a leaf wait until kWideLeafBatch of them are, or no lane
+// has a node left to test, and test their leaves together (12; 8 costs 1-2 %, 4 costs 5 %).
+template <int KEEP>
+__device__ __forceinline__ void wide_steps(const float4* __restrict__ wide, const float4* __restrict__ tris, WideRay& st,
+                                           WideWalk& w, int2* stk, bool active) {
+    const int stop = (__popc(__ballot_sync(0xffffffffu, active)) * KEEP) >> 2;
+    uint32_t nm, lm;
+    do {
+        if (active && w.cur >= 0) wide_node(wide, st, w, stk);
+        const bool leaf = active && w.cur < 0 && w.cur != kWalkDone;
+        lm = __ballot_sync(0xffffffffu, leaf);
+        nm = __ballot_sync(0xffffffffu, active && w.cur >= 0);
+        if (lm && (!nm || __popc(lm) >= kWideLeafBatch)) {
+            if (leaf) {
+                trav_leaf(tris, st, (~w.cur) >> 3, (~w.cur) & 7);
+                w.cur = wide_pop(st, w, stk);
+            }
+            lm = __ballot_sync(0xffffffffu, active && w.cur != kWalkDone);
+        }
+    } while (__popc(lm | nm) > stop);
+}
+
+// ---- the last ray of a warp, walked by all 32 lanes ----------------------------------------
+// Once a warp's queue is exhausted and one lane still walks, the launch waits for a chain of
+// dependent fetches. The whole warp then takes up to eight nodes off that ray's stack at a time,
+// four lanes to a node and a child to a lane, and tests the leaves that were hit eight at a time,
+// a triangle to a lane. More boxes are tested than by one lane, in fewer rounds.
+constexpr int kCoopStack = 128;  // entries per warp: at most eight nodes' children are added while 40 fit above
+                                 // them (up to kCoopNarrow), then one node's at a time, three more per wide level
+constexpr int kCoopNarrow = 40;
+
+struct CoopScratch {
+    int2 stk[kCoopStack];
+    int32_t leaf[32];
+};
+static_assert(kCoopNarrow + 24 + 3 * (kWideMaxDepth / 2 + 1) < kCoopStack && kWideStack < kCoopStack - 3, "warp stack");
+
+// Walks lane owner's ray (st, w and stk are that lane's) to its end; every lane calls it and
+// receives the ray with its final best hit. Not inlined: the callers' loops keep their registers.
+static __device__ __noinline__ WideRay coop_wide(const float4* __restrict__ wide, const float4* __restrict__ tris,
+                                                 WideRay st, WideWalk w, const int2* stk, int owner, CoopScratch* sc) {
+    const uint32_t F = 0xffffffffu;
+    const int lane = threadIdx.x & 31, slot = lane >> 2, c = lane & 3;
+    const uint32_t lt = lanemask_lt();
+    st.o = make_float3(__shfl_sync(F, st.o.x, owner), __shfl_sync(F, st.o.y, owner), __shfl_sync(F, st.o.z, owner));
+    st.d = make_float3(__shfl_sync(F, st.d.x, owner), __shfl_sync(F, st.d.y, owner), __shfl_sync(F, st.d.z, owner));
+    st.inv = make_float3(__shfl_sync(F, st.inv.x, owner), __shfl_sync(F, st.inv.y, owner), __shfl_sync(F, st.inv.z, owner));
+    st.tmin = __shfl_sync(F, st.tmin, owner);
+    st.tbest = __shfl_sync(F, st.tbest, owner);
+    st.best = __shfl_sync(F, st.best, owner);
+    st.slot = __shfl_sync(F, st.slot, owner);
+    st.pad = __shfl_sync(F, st.pad, owner);
+    int n = __shfl_sync(F, w.sp, owner) + 1;
+    if (lane == owner) {
+        for (int i = 0; i < n - 1; ++i) sc->stk[i] = stk[i];
+        sc->stk[n - 1] = make_int2(-1, w.cur);  // a negative key: not culled
+    }
+    __syncwarp();
+    while (n > 0) {
+        const int take = n > kCoopNarrow ? 1 : min(n, 8);
+        int2 e = make_int2(0, kWalkDone);
+        if (slot < take) e = sc->stk[n - 1 - slot];
+        n -= take;
+        int32_t key = kWideMiss, ref = kWalkDone;
+        if (e.y != kWalkDone && wide_keep(e.x, st.tbest)) {
+            if (e.y >= 0) {
+                const float* q = (const float*)(wide + 8 * (int64_t)e.y) + c;
+                key = wide_key(st, __ldg(q), __ldg(q + 4), __ldg(q + 8), __ldg(q + 12), __ldg(q + 16), __ldg(q + 20), c);
+                ref = __ldg((const int32_t*)q + 24);
+            } else if (c == 0) {
+                key = e.x & ~3;
+                ref = e.y;
+            }
+        }
+        const bool hit = key != kWideMiss && ref != kWalkDone;
+        const uint32_t nm = __ballot_sync(F, hit && ref >= 0), lm = __ballot_sync(F, hit && ref < 0);
+        __syncwarp();  // every lane has read its entry
+        if (hit && ref >= 0) sc->stk[n + __popc(nm & lt)] = make_int2(key, ref);
+        if (hit && ref < 0) sc->leaf[__popc(lm & lt)] = ~ref;
+        n += __popc(nm);
+        __syncwarp();
+        const int nl = __popc(lm);
+        for (int l0 = 0; l0 < nl; l0 += 8) {
+            const int32_t word = l0 + slot < nl ? sc->leaf[l0 + slot] : 0;  // 0 triangles
+            float t = 0.0f;
+            int32_t id = 0, ts = -1;
+            bool ok = false;
+            for (int k = c; k < (word & 7); k += 4) {  // a lane's second triangle, if any, after its first
+                const float4* tp = tris + 3 * (int64_t)((word >> 3) + k);
+                const float4 P = __ldg(tp), V1 = __ldg(tp + 1), V2 = __ldg(tp + 2);
+                float tt;
+                const int32_t ti = __float_as_int(P.w);
+                if (tri_hit(st.o, st.d, P, V1, V2, tt) && tt > st.tmin &&
+                    (tt < st.tbest || (tt == st.tbest && st.best >= 0 && ti < st.best)) &&
+                    (!ok || tt < t || (tt == t && ti < id))) {
+                    ok = true;
+                    t = tt;
+                    id = ti;
+                    ts = (word >> 3) + k;
+                }
+            }
+            if (__ballot_sync(F, ok) == 0) continue;
+            uint32_t tk = 0xffffffffu;  // t as an unsigned key in float order (-0 and +0 alike)
+            if (ok) {
+                const uint32_t b = __float_as_uint(t + 0.0f);
+                tk = (b & 0x80000000u) ? ~b : (b | 0x80000000u);
+            }
+            const uint32_t kmin = __reduce_min_sync(F, tk);
+            const bool tie = ok && tk == kmin;
+            const uint32_t imin = __reduce_min_sync(F, tie ? (uint32_t)id : 0xffffffffu);
+            const int win = __ffs(__ballot_sync(F, tie && (uint32_t)id == imin)) - 1;
+            st.tbest = __shfl_sync(F, t, win);
+            st.best = (int32_t)imin;
+            st.slot = __shfl_sync(F, ts, win);
+        }
+    }
+    __syncwarp();  // the scratch may be reused
+    return st;
+}
+
+}  // namespace gspd
