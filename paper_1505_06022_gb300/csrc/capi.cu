@@ -163,25 +163,33 @@ k_trace_wide(DevScene S, const float4* __restrict__ rays, int64_t n, const uint3
     w.cur = kWalkDone;
     w.sp = 0;
     int32_t ray = -1;
+    bool quad = false;  // the last rays, four lanes to a ray
     while (true) {
-        const int32_t got = wq.take(ray < 0, ctr);
+        const int32_t got = quad ? -1 : wq.take(ray < 0, ctr);
         if (got >= 0) {
             ray = got;
             const float4 a = __ldcs(rays + 2 * (int64_t)ray), b = __ldcs(rays + 2 * (int64_t)ray + 1);
             wide_ray(f3(a), f3(b), a.w, b.w, st);
             wide_init(w);
         }
-        if (__ballot_sync(0xffffffffu, ray >= 0) == 0) break;
         const uint32_t act = __ballot_sync(0xffffffffu, ray >= 0);
-        if (wq.done && !(act & (act - 1))) {  // no rays left to take and one lane walks: all lanes walk its ray
+        if (act == 0) break;
+        if (wq.done && __popc(act) == (quad ? 4 : 1)) {
             st = coop_wide(S.wide, S.tris, st, w, stk, __ffs(act) - 1, &scratch[threadIdx.x >> 5]);
             w.cur = kWalkDone;
-        } else {
+        } else if (!quad && wq.done && __popc(act) <= kQuadRays) {
+            quad = true;
+            const int src = quad_source(act);
+            quad_take(st, w, stk, src < 0 ? lane : src);
+            ray = __shfl_sync(0xffffffffu, ray, src < 0 ? lane : src);
+            if (src < 0) ray = -1;
+        } else if (quad)
+            quad_steps<GSP_WIDE_KEEP_TRACE>(S.wide, S.tris, st, w, stk, ray >= 0);
+        else
             wide_steps<GSP_WIDE_KEEP_TRACE>(S.wide, S.tris, st, w, stk, ray >= 0);
-        }
         const bool fin = ray >= 0 && w.cur == kWalkDone;
         bool flag = false;
-        if (fin) {
+        if (fin && (!quad || (lane & 3) == 0)) {
             float u = 0.0f, v = 0.0f;
             if (st.slot >= 0)
                 flag = hit_needs_refine(S.tris + 3 * st.slot, st.o, st.d, st.tbest, refine_factor, uv != nullptr, u, v);

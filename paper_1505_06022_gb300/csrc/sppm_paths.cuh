@@ -295,7 +295,7 @@ struct PathWalk<kLinks> {
     }
     __device__ __forceinline__ bool done() const { return st.node < 0 && pend < 0; }
     // Every lane calls it; lane `owner` is the only one with a path.
-    __device__ __forceinline__ void finish(const DevScene& S, int owner, int32_t cap, CoopScratch*, uint32_t& ntri) {
+    __device__ __forceinline__ void finish(const DevScene& S, int owner, int32_t cap, uint32_t& ntri) {
         const CoopWalk r = coop_walk(S.tris, S.nnodes, S.status, st, pend, owner, cap);
         st = r.st;
         pend = -1;
@@ -340,12 +340,23 @@ struct PathWalk<kWide> {
     __device__ __forceinline__ void steps(const DevScene& S, bool active, int32_t, uint32_t&) {
         wide_steps<GSP_WIDE_KEEP>(S.wide, S.tris, st, w, stk, active);
     }
-    __device__ __forceinline__ bool done() const { return w.cur == kWalkDone; }
-    __device__ __forceinline__ void finish(const DevScene& S, int owner, int32_t, CoopScratch* sc, uint32_t&) {
+    __device__ __forceinline__ void finish(const DevScene& S, int owner, CoopScratch* sc) {
         st = coop_wide(S.wide, S.tris, st, w, stk, owner, sc);
         w.cur = kWalkDone;
     }
+    __device__ __forceinline__ void quad_steps(const DevScene& S, bool active) {
+        gspd::quad_steps<GSP_WIDE_KEEP>(S.wide, S.tris, st, w, stk, active);
+    }
+    __device__ __forceinline__ bool done() const { return w.cur == kWalkDone; }
 };
+
+// The path state beside a walk, handed from lane src to this one with it (every lane calls these).
+__device__ __forceinline__ Rng shfl_rng(const Rng& r, int src) {
+    Rng g;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) g.s[k] = __shfl_sync(0xffffffffu, r.s[k], src);
+    return g;
+}
 
 // Appends the lanes with `keep` set to queue Q (warp-aggregated: one atomic per warp).
 __device__ __forceinline__ void queue_push(const PathQ& Q, uint32_t* count, bool keep, float3 o, float tmin, float3 d,
@@ -388,16 +399,17 @@ struct EyeOut {
 // One eye-path interaction at a hit. Emission seen from the front is added to the pixel's
 // direct term of this pass (one path per pixel, so no atomics);
 // a diffuse hit records the hit point and ends the path; a mirror or dielectric bends the ray
-// (returns true: the path continues from x along the new d).
+// (returns true: the path continues from x along the new d). Of lanes that hold the same path, the
+// one with `lead` writes.
 template <bool SHADE>
 __device__ __forceinline__ bool eye_interact(const DevScene& S, const PassDev& P, const EyeOut& O, int64_t p,
-                                             const Hit& h, float3& o, float3& d, float3& w, Rng& rng) {
+                                             const Hit& h, float3& o, float3& d, float3& w, Rng& rng, bool lead = true) {
     const float4 sh = __ldg(S.shade + h.id);
     const float3 n = f3(sh);
     const int32_t mid = __float_as_int(sh.w);
     const Material m = load_mat(S, mid);
     const bool front = dot3(d, n) < 0.0f;
-    if (front && emits(m)) {
+    if (lead && front && emits(m)) {
         float4 v = O.hd[p];
         v.x += w.x * m.emission.x;
         v.y += w.y * m.emission.y;
@@ -411,10 +423,12 @@ __device__ __forceinline__ bool eye_interact(const DevScene& S, const PassDev& P
         const float3 ns = front ? n : n * -1.0f;
         const float3 wt = mul3(w, sf.tex);  // the hit point's weight without its albedo
         const float3 f = mul3(wt, m.albedo) * (1.0f / kPi);
-        O.hx[p] = make_float4(x.x, x.y, x.z, __int_as_float(mid));
-        O.hn[p] = make_float4(ns.x, ns.y, ns.z, 0.0f);
-        O.hf[p] = make_float4(f.x, f.y, f.z, 0.0f);
-        if (O.hw) O.hw[p] = make_float4(wt.x, wt.y, wt.z, 0.0f);
+        if (lead) {
+            O.hx[p] = make_float4(x.x, x.y, x.z, __int_as_float(mid));
+            O.hn[p] = make_float4(ns.x, ns.y, ns.z, 0.0f);
+            O.hf[p] = make_float4(f.x, f.y, f.z, 0.0f);
+            if (O.hw) O.hw[p] = make_float4(wt.x, wt.y, wt.z, 0.0f);
+        }
         return false;
     }
     if (m.type == GSP_MIRROR) {
@@ -550,11 +564,11 @@ struct DepositDev {
     int32_t* __restrict__ smat;          // optional: material of each deposit's surface (gradient replay)
 };
 
-// One photon interaction at a hit. Returns false when the path ends.
+// One photon interaction at a hit. Returns false when the path ends. lead as in eye_interact.
 template <bool SHADE>
 __device__ __forceinline__ bool photon_bounce(const DevScene& S, const PassDev& P, const DepositDev& D,
                                               Rng& rng, const Hit& h, float3& o, float3& d, float3& phi,
-                                              uint32_t id, uint32_t slot, uint32_t& ndep) {
+                                              uint32_t id, uint32_t slot, uint32_t& ndep, bool lead = true) {
     const float4 sh = __ldg(S.shade + h.id);
     const float3 n = f3(sh);
     const Material m = load_mat(S, __float_as_int(sh.w));
@@ -562,17 +576,21 @@ __device__ __forceinline__ bool photon_bounce(const DevScene& S, const PassDev& 
     const float3 x = madd3(d, h.t, o);
     const Surf sf = surface<SHADE>(S, h, o, d, n, m, __float_as_int(sh.w));
     if (m.type == GSP_DIFFUSE) {
-        if (D.smat) D.smat[slot] = __float_as_int(sh.w);
-        float4* rec = D.slots + 2 * (size_t)slot;
-        rec[0] = make_float4(x.x, x.y, x.z, __uint_as_float(id));
-        rec[1] = make_float4(phi.x, phi.y, phi.z, __uint_as_float(oct_encode(d)));
+        if (lead) {
+            if (D.smat) D.smat[slot] = __float_as_int(sh.w);
+            float4* rec = D.slots + 2 * (size_t)slot;
+            rec[0] = make_float4(x.x, x.y, x.z, __uint_as_float(id));
+            rec[1] = make_float4(phi.x, phi.y, phi.z, __uint_as_float(oct_encode(d)));
+        }
         ++ndep;
         if (D.stochastic) {
             const float z = rng_next(rng);
-            const uint32_t b = bucket_of(x, P.inv_h, P.tmask);
-            const unsigned long long key = ((unsigned long long)__float_as_uint(z) << 32) | slot;
-            atomicMin(D.entry + b, key);
-            atomicAdd(D.ecount + b, 1u);
+            if (lead) {
+                const uint32_t b = bucket_of(x, P.inv_h, P.tmask);
+                const unsigned long long key = ((unsigned long long)__float_as_uint(z) << 32) | slot;
+                atomicMin(D.entry + b, key);
+                atomicAdd(D.ecount + b, 1u);
+            }
         }
         const float urr = rng_next(rng);
         if (!(urr < P.rr)) return false;
@@ -690,8 +708,9 @@ k_paths(DevScene S, PassDev P, PathQ qe, EyeOut O, const uint32_t* __restrict__ 
     float3 w = make_float3(0.0f, 0.0f, 0.0f);  // eye: throughput; photon: flux
     Rng rng;
     uint32_t c_eye = 0, c_ph = 0, c_nodes = 0, c_tris = 0;  // work of this lane
+    bool quad = false;  // the last paths, four lanes to a path
     while (true) {
-        const int32_t got = wq.take(i < 0, ctr);
+        const int32_t got = quad ? -1 : wq.take(i < 0, ctr);
         if (got >= 0) {
             i = got;
             eye = got < ne;
@@ -706,16 +725,39 @@ k_paths(DevScene S, PassDev P, PathQ qe, EyeOut O, const uint32_t* __restrict__ 
             ndep = eye ? 0u : (uint32_t)(meta >> 8);
             pw.start(S, f3(a), f3(c), eye ? a.w : P.eps);
         }
-        const uint32_t act = __ballot_sync(0xffffffffu, i >= 0);
+        uint32_t act = __ballot_sync(0xffffffffu, i >= 0);
         if (act == 0) break;
-        bool lone = false;  // nothing left to take: a path left alone in the warp walks with all lanes
-        if constexpr (WALK != kStack) {
+        bool walked = false;
+        if constexpr (WALK == kLinks) {  // nothing left to take: a path left alone in the warp walks with all lanes
             if (wq.done && !(act & (act - 1))) {
-                pw.finish(S, __ffs(act) - 1, cap, &scratch[WALK == kWide ? threadIdx.x >> 5 : 0], c_tris);
-                lone = true;
+                pw.finish(S, __ffs(act) - 1, cap, c_tris);
+                walked = true;
             }
         }
-        if (!lone) pw.steps(S, i >= 0, cap, c_tris);
+        if constexpr (WALK == kWide) {
+            if (!quad && wq.done && __popc(act) <= kQuadRays && __popc(act) > 1) {
+                quad = true;
+                const int own = threadIdx.x & 31, from = quad_source(act), src = from < 0 ? own : from;
+                quad_take(pw.st, pw.w, pw.stk, src);
+                i = from < 0 ? -1 : 0;
+                id = __shfl_sync(0xffffffffu, id, src);
+                depth = __shfl_sync(0xffffffffu, depth, src);
+                ndep = __shfl_sync(0xffffffffu, ndep, src);
+                eye = __shfl_sync(0xffffffffu, (int)eye, src) != 0;
+                w = shfl3(w, src);
+                rng = shfl_rng(rng, src);
+                act = __ballot_sync(0xffffffffu, i >= 0);
+            }
+            if (wq.done && __popc(act) == (quad ? 4 : 1)) {
+                pw.finish(S, __ffs(act) - 1, &scratch[threadIdx.x >> 5]);
+                walked = true;
+            } else if (quad) {
+                pw.quad_steps(S, i >= 0);
+                walked = true;
+            }
+        }
+        const bool lead = !quad || (threadIdx.x & 3) == 0;
+        if (!walked) pw.steps(S, i >= 0, cap, c_tris);
         if (i >= 0 && pw.done()) {
             const Hit h = walk_hit(S, pw.st);
             float3 o = pw.st.o, d = pw.st.d;
@@ -726,14 +768,14 @@ k_paths(DevScene S, PassDev P, PathQ qe, EyeOut O, const uint32_t* __restrict__ 
                 c_ph += eye ? 0u : 1u;
             }
             if (eye) {
-                more = h.id >= 0 && eye_interact<SHADE>(S, P, O, id, h, o, d, w, rng) && ++depth <= P.max_eye;
+                more = h.id >= 0 && eye_interact<SHADE>(S, P, O, id, h, o, d, w, rng, lead) && ++depth <= P.max_eye;
             } else {
                 if (h.id >= 0) {
                     const uint32_t pid = (uint32_t)id * kSlotsPerPath + depth;
                     const uint32_t slot = (uint32_t)id * kSlotsPerPath + ndep;
-                    more = photon_bounce<SHADE>(S, P, D, rng, h, o, d, w, pid, slot, ndep) && ++depth < P.max_photon;
+                    more = photon_bounce<SHADE>(S, P, D, rng, h, o, d, w, pid, slot, ndep, lead) && ++depth < P.max_photon;
                 }
-                if (!more) D.pcount[id] = ndep;
+                if (!more && lead) D.pcount[id] = ndep;
             }
             if (more)
                 pw.start(S, o, d, P.eps);
@@ -844,8 +886,9 @@ k_paths_multi(const PathJob* __restrict__ jobs, int32_t njobs, int32_t total_chu
     bool eye = false;
     float3 w = make_float3(0.0f, 0.0f, 0.0f);  // eye: throughput; photon: flux
     Rng rng;
+    bool quad = false;  // the last paths, four lanes to a path
     while (true) {
-        const int32_t got = mq.take(i < 0, jobs, njobs, ctr, jb);
+        const int32_t got = quad ? -1 : mq.take(i < 0, jobs, njobs, ctr, jb);
         if (got >= 0) {
             const PathJob& J = jobs[jb];
             const int32_t ne = J.ne_ptr ? (int32_t)*J.ne_ptr : 0;
@@ -863,23 +906,43 @@ k_paths_multi(const PathJob* __restrict__ jobs, int32_t njobs, int32_t total_chu
             cap = trav_cap(J.S);
             pw.start(J.S, f3(a), f3(c), eye ? a.w : J.P.eps);
         }
-        if (__ballot_sync(0xffffffffu, i >= 0) == 0) break;
+        const uint32_t act = __ballot_sync(0xffffffffu, i >= 0);
+        if (act == 0) break;
+        if constexpr (WALK == kWide) {
+            if (!quad && mq.done && __popc(act) <= kQuadRays) {
+                quad = true;
+                const int own = threadIdx.x & 31, from = quad_source(act), src = from < 0 ? own : from;
+                quad_take(pw.st, pw.w, pw.stk, src);
+                i = from < 0 ? -1 : 0;
+                jb = __shfl_sync(0xffffffffu, jb, src);
+                id = __shfl_sync(0xffffffffu, id, src);
+                depth = __shfl_sync(0xffffffffu, depth, src);
+                ndep = __shfl_sync(0xffffffffu, ndep, src);
+                eye = __shfl_sync(0xffffffffu, (int)eye, src) != 0;
+                w = shfl3(w, src);
+                rng = shfl_rng(rng, src);
+            }
+        }
         const PathJob& J = jobs[jb];
         uint32_t ntri = 0;  // work is not counted in batched passes
-        pw.steps(J.S, i >= 0, cap, ntri);
+        const bool lead = !quad || (threadIdx.x & 3) == 0;
+        if constexpr (WALK == kWide) {
+            if (quad) pw.quad_steps(J.S, i >= 0);
+        }
+        if (!quad) pw.steps(J.S, i >= 0, cap, ntri);
         if (i >= 0 && pw.done()) {
             const Hit h = walk_hit(J.S, pw.st);
             float3 o = pw.st.o, d = pw.st.d;
             bool more = false;
             if (eye) {
-                more = h.id >= 0 && eye_interact<SHADE>(J.S, J.P, J.O, id, h, o, d, w, rng) && ++depth <= J.P.max_eye;
+                more = h.id >= 0 && eye_interact<SHADE>(J.S, J.P, J.O, id, h, o, d, w, rng, lead) && ++depth <= J.P.max_eye;
             } else {
                 if (h.id >= 0) {
                     const uint32_t pid = (uint32_t)id * kSlotsPerPath + depth;
                     const uint32_t slot = (uint32_t)id * kSlotsPerPath + ndep;
-                    more = photon_bounce<SHADE>(J.S, J.P, J.D, rng, h, o, d, w, pid, slot, ndep) && ++depth < J.P.max_photon;
+                    more = photon_bounce<SHADE>(J.S, J.P, J.D, rng, h, o, d, w, pid, slot, ndep, lead) && ++depth < J.P.max_photon;
                 }
-                if (!more) J.D.pcount[id] = ndep;
+                if (!more && lead) J.D.pcount[id] = ndep;
             }
             if (more)
                 pw.start(J.S, o, d, J.P.eps);
@@ -913,8 +976,9 @@ k_photon_regen(DevScene S, EmitDev E, PassDev P, DepositDev D, RegenDev R, uint3
     uint32_t c_ph = 0, c_nodes = 0, c_tris = 0;  // work of this lane
     float3 phi = make_float3(0.0f, 0.0f, 0.0f);
     Rng rng;
+    bool quad = false;  // the last paths, four lanes to a path
     while (true) {
-        const int32_t got = wq.take(j < 0, ctr);
+        const int32_t got = quad ? -1 : wq.take(j < 0, ctr);
         if (got >= 0) {
             j = got;
             rng = rng_seed(P.seed, P.scene_id, 1u, pass_index(P), (uint64_t)j);
@@ -929,8 +993,23 @@ k_photon_regen(DevScene S, EmitDev E, PassDev P, DepositDev D, RegenDev R, uint3
             }
             pw.start(S, o, d, P.eps);
         }
-        if (__ballot_sync(0xffffffffu, j >= 0) == 0) break;
-        pw.steps(S, j >= 0, cap, c_tris);
+        const uint32_t act = __ballot_sync(0xffffffffu, j >= 0);
+        if (act == 0) break;
+        if constexpr (WALK == kWide) {
+            if (!quad && wq.done && __popc(act) <= kQuadRays) {
+                quad = true;
+                const int own = threadIdx.x & 31, from = quad_source(act), src = from < 0 ? own : from;
+                quad_take(pw.st, pw.w, pw.stk, src);
+                j = __shfl_sync(0xffffffffu, j, src);
+                if (from < 0) j = -1;
+                depth = __shfl_sync(0xffffffffu, depth, src);
+                phi = shfl3(phi, src);
+                rng = shfl_rng(rng, src);
+            }
+            if (quad) pw.quad_steps(S, j >= 0);
+        }
+        const bool lead = !quad || (threadIdx.x & 3) == 0;
+        if (!quad) pw.steps(S, j >= 0, cap, c_tris);
         if (j >= 0 && pw.done()) {
             if (COUNT) {
                 c_ph += 1;
@@ -939,12 +1018,14 @@ k_photon_regen(DevScene S, EmitDev E, PassDev P, DepositDev D, RegenDev R, uint3
             const Hit h = walk_hit(S, pw.st);
             float3 o = pw.st.o, d = pw.st.d;
             uint32_t ndep = 0;
-            bool alive = h.id >= 0 && photon_bounce<SHADE>(S, P, D, rng, h, o, d, phi, (uint32_t)j, (uint32_t)j, ndep) &&
+            bool alive = h.id >= 0 && photon_bounce<SHADE>(S, P, D, rng, h, o, d, phi, (uint32_t)j, (uint32_t)j, ndep, lead) &&
                          ++depth < P.max_photon;
-            D.pcount[j] = ndep;
-            R.ro[j] = make_float4(o.x, o.y, o.z, __int_as_float(depth));
-            R.rd[j] = make_float4(d.x, d.y, d.z, __int_as_float(alive ? 1 : 0));
-            R.rphi[j] = make_float4(phi.x, phi.y, phi.z, 0.0f);
+            if (lead) {
+                D.pcount[j] = ndep;
+                R.ro[j] = make_float4(o.x, o.y, o.z, __int_as_float(depth));
+                R.rd[j] = make_float4(d.x, d.y, d.z, __int_as_float(alive ? 1 : 0));
+                R.rphi[j] = make_float4(phi.x, phi.y, phi.z, 0.0f);
+            }
             j = -1;
         }
     }
