@@ -20,7 +20,7 @@
 //                 path k owns slots [k*32, k*32+32) (one slot per thread in REGEN mode)
 //     queues      eye and photon wavefront queues, two of each (ping-pong), their lengths,
 //                 the path kernel's work counter, the wavefront steps' trace counters
-//   exact grid    bucket-sorted SoA copies spos[], spay[] + bucket starts bstart[T+1]
+//   exact grid    bucket-sorted SoA copies spos[], spay[] + bucket starts bstart[T+1] (hash_grid.cuh)
 //   stochastic    entry[T] = min(random depth bits << 32 | slot), ecount[T], one table per trace set
 #include <algorithm>
 #include <cmath>
@@ -31,6 +31,7 @@
 
 #include "devcommon.cuh"
 #include "gsp_internal.h"
+#include "hash_grid.cuh"
 #include "launch.h"
 #include "persist.cuh"
 #include "scan_sort.h"
@@ -101,7 +102,6 @@ struct gsp_sppm {
     uint32_t* ecount = nullptr;
     float4 *ro = nullptr, *rd = nullptr, *rphi = nullptr;
     unsigned long long* started = nullptr;
-    uint32_t* last_order = nullptr;  // sorted slot order of the last exact pass
     uint32_t* heavy = nullptr;  // exact gather: hit points with long queries (k_gather_heavy), npix entries
     unsigned long long* work = nullptr;  // work counters (kWorkCounts), see gsp_sppm_count_work
     bool count_work = false;
@@ -325,20 +325,21 @@ gsp_status gsp_sppm_create(gsp_scene* s, const gsp_sppm_params* params, gsp_sppm
     A(&r->tb[0].slots, 2 * r->slot_cap);
     A(&r->tb[0].pcount, r->np);
     use_buf(r, 0);
-    A(&r->poff, r->np);
     A(&r->counters, 16);
     A(&r->started, 1);
     A(&r->work, kWorkCounts);
-    const int64_t scan_tmp = std::max({gsp_scan_temp_elems(r->np), gsp_scan_temp_elems(r->T),
-                                       gsp_scan_temp_elems(gsp_sort_hist_elems())});
-    A(&r->scan_tmp, scan_tmp);
     if (P.hash_mode == GSP_EXACT) {
-        for (int b = 0; b < 2; ++b) {
-            A(&r->keys[b], r->slot_cap);
-            A(&r->vals[b], r->slot_cap);
-        }
+        A(&r->keys[0], r->slot_cap);
+        A(&r->vals[0], r->slot_cap);
+        A(&r->keys[1], 2 * r->slot_cap);  // the parts' {bucket, slot} pairs, or the radix sort's second pair
+        r->vals[1] = r->keys[1] ? r->keys[1] + r->slot_cap : nullptr;
         A(&r->hist, gsp_sort_hist_elems());
-        A(&r->bcount, r->T);
+        if (r->tbits > kGridMaxBits) {  // the radix sort's buffers
+            A(&r->poff, r->np);
+            A(&r->bcount, r->T);
+            A(&r->scan_tmp, std::max({gsp_scan_temp_elems(r->np), gsp_scan_temp_elems(r->T),
+                                      gsp_scan_temp_elems(gsp_sort_hist_elems())}));
+        }
         A(&r->bstart, r->T + 1);
         A(&r->spos, r->slot_cap);
         A(&r->spay, r->slot_cap);
@@ -609,10 +610,39 @@ static gsp_status stage_paths(gsp_sppm* r, const PassDev& P, const EyeOut& O, co
     return GSP_OK;
 }
 
-// Exact hash grid of the pass's deposits: compaction in id order, stable sort by bucket,
-// bucket starts, sorted SoA copies.
+// The launches of a hash grid of at most 2^kGridMaxBits buckets (hash_grid.cuh). `hist` has
+// gsp_sort_hist_elems() words: the aux words at its end and, where they fit before them, the tiles'
+// counts, which else go to bstart (there are at most 2^low tiles then, so they fit).
+static_assert((int64_t)kGridMaxTiles * 256 + kGridAux <= kGspSortHistElems && kGridMaxTiles <= kGridMaxLow &&
+                  512 + 2 * kGridMaxParts + 1 <= kGridAux && kGridMaxLow <= 4 * kGridThreads && kGridSegment < 65536,
+              "the counts of 256 parts fit beside the aux words, those of more parts in the bucket starts");
+static cudaError_t grid_launch(const GridIn& in, int bits, uint32_t* keys, uint32_t* vals, uint2* pairs, uint32_t* hist,
+                               uint32_t* order, float4* spos, float4* spay, uint32_t* bstart, uint32_t* d_total,
+                               uint32_t* clear, cudaStream_t st) {
+    const GridPlan plan = grid_plan(in.items, bits);
+    const bool beside = (int64_t)plan.tiles * plan.parts <= kGspSortHistElems - kGridAux;
+    const GridBuf buf{keys, vals, pairs, beside ? hist : bstart, hist + kGspSortHistElems - kGridAux};
+    if (plan.tiles) k_grid_tiles<<<plan.tiles, kGridThreads, 0, st>>>(in, plan, buf);
+    k_grid_scan<<<(plan.parts + 31) / 32, kScanThreads, 0, st>>>(plan, buf);
+    k_grid_split<<<std::max(1, plan.tiles), kGridThreads, 0, st>>>(in, plan, buf, d_total, clear);
+    k_grid_parts<<<plan.parts, kGridThreads, 0, st>>>(in, plan, buf, order, spos, spay, bstart);
+    return cudaGetLastError();
+}
+
+static GridIn deposits_in(const gsp_sppm* r, float inv_h, uint32_t mask) {
+    return GridIn{r->slots, r->pcount, r->np, r->slots_per_path, 0, inv_h, mask};
+}
+
+// Exact hash grid of the pass's deposits, in id order within a bucket: bucket starts and sorted SoA
+// copies. Tables of more than 2^kGridMaxBits buckets (more than 2^20 photons a pass by default) are
+// sorted by radix passes.
 static gsp_status stage_deposit(gsp_sppm* r, const PassDev& P, cudaStream_t st) {
     uint32_t* d_total = r->counters;  // deposits this pass
+    if (r->tbits <= kGridMaxBits) {
+        GSP_CUDA_TRY(grid_launch(deposits_in(r, r->inv_h, P.tmask), r->tbits, r->keys[0], r->vals[0], (uint2*)r->keys[1], r->hist,
+                                 nullptr, r->spos, r->spay, r->bstart, d_total, r->counters + 10, st));
+        return GSP_OK;
+    }
     GSP_CUDA_TRY(gsp_scan_u32(r->pcount, r->poff, r->np, d_total, r->scan_tmp, st));
     GSP_CUDA_TRY(cudaMemsetAsync(r->bcount, 0, r->T * sizeof(uint32_t), st));
     k_compact<<<blocks(r->np, 256), 256, 0, st>>>(r->slots, r->pcount, r->poff, r->np, r->slots_per_path, r->inv_h,
@@ -621,21 +651,8 @@ static gsp_status stage_deposit(gsp_sppm* r, const PassDev& P, cudaStream_t st) 
     uint32_t *ko = nullptr, *vo = nullptr;
     GSP_CUDA_TRY(gsp_radix_sort_u32(r->keys[0], r->vals[0], r->keys[1], r->vals[1], d_total, r->tbits, r->hist,
                                     r->scan_tmp, st, &ko, &vo));
-    r->last_order = vo;
     k_permute<<<1024, 256, 0, st>>>(r->slots, vo, d_total, r->spos, r->spay);
-    GSP_CUDA_TRY(cudaGetLastError());
-    return GSP_OK;
-}
-
-// The pass's deposits in path order, without the hash grid: the list the adjoint's photon loop
-// walks (a grid would only order it).
-static gsp_status stage_deposit_list(gsp_sppm* r, cudaStream_t st) {
-    uint32_t* d_total = r->counters;
-    GSP_CUDA_TRY(gsp_scan_u32(r->pcount, r->poff, r->np, d_total, r->scan_tmp, st));
-    k_compact<<<blocks(r->np, 256), 256, 0, st>>>(r->slots, r->pcount, r->poff, r->np, r->slots_per_path, 0.0f, 0u,
-                                                  nullptr, r->vals[0], nullptr);
-    r->last_order = r->vals[0];
-    k_permute<<<1024, 256, 0, st>>>(r->slots, r->vals[0], d_total, r->spos, r->spay);
+    GSP_CUDA_TRY(cudaMemsetAsync(r->counters + 10, 0, sizeof(uint32_t), st));
     GSP_CUDA_TRY(cudaGetLastError());
     return GSP_OK;
 }
@@ -667,8 +684,9 @@ static gsp_status gather_half(gsp_sppm* r, const PassDev& P, cudaStream_t st) {
         G.slots = r->slots;
         G.entry = r->entry;
         G.ecount = r->ecount;
-        // deposit count for diagnostics
-        GSP_CUDA_TRY(gsp_scan_u32(r->pcount, r->poff, r->np, r->counters, r->scan_tmp, st));
+        G.pcount = r->pcount;
+        G.total = r->counters;  // deposit count for diagnostics
+        GSP_CUDA_TRY(cudaMemsetAsync(G.total, 0, sizeof(uint32_t), st));
         k_gather_stoch<<<blocks(r->npix, 128), 128, 0, st>>>(G, P);
     } else {
         gsp_status e = stage_deposit(r, P, st);
@@ -679,8 +697,7 @@ static gsp_status gather_half(gsp_sppm* r, const PassDev& P, cudaStream_t st) {
         // long queries are listed by k_gather_exact and served by whole blocks (counters[10] counts them)
         if (r->heavy) {
             G.heavy = r->heavy;
-            G.nheavy = r->counters + 10;
-            GSP_CUDA_TRY(cudaMemsetAsync(G.nheavy, 0, sizeof(uint32_t), st));
+            G.nheavy = r->counters + 10;  // cleared by the deposit
         }
         launch_gather_exact(r->gather_lanes, G, P, r->npix, st);
         if (r->heavy) k_gather_heavy<<<2 * sm_count(r->scene->ctx->device), kHeavyThreads, 0, st>>>(G, P);
@@ -692,6 +709,9 @@ static gsp_status gather_half(gsp_sppm* r, const PassDev& P, cudaStream_t st) {
 
 #ifndef GSP_ADJ_LANES
 #define GSP_ADJ_LANES 8
+#endif
+#ifndef GSP_ADJ_COLUMNS  // blocks that share a tile's deposits
+#define GSP_ADJ_COLUMNS 16
 #endif
 
 static gsp_status check_grad_room(gsp_sppm* r, int64_t npasses) {
@@ -909,8 +929,11 @@ gsp_status gsp_render_grad(gsp_sppm* r, const float* d_dloss_dimg, float* d_grad
         if (e != GSP_OK) return e;
         GSP_CUDA_TRY(cudaEventRecord(r->ev_traced[j], r->tstream[j]));
         GSP_CUDA_TRY(cudaStreamWaitEvent(st, r->ev_traced[j], 0));
-        e = stage_deposit_list(r, st);
-        if (e != GSP_OK) return e;
+        // the pass's deposits in path order, tile by tile (a grid would only order the adjoint's loop)
+        GridPlan list = grid_plan(r->np, 0);
+        list.parts = 0;
+        const GridBuf lbuf{r->keys[0], r->vals[0], nullptr, nullptr, r->hist};
+        k_grid_tiles<<<list.tiles, kGridThreads, 0, st>>>(deposits_in(r, 0.0f, 0u), list, lbuf);
         e = gsp_grid_build_with(r->hx, r->npix, hp_cell, r->hp_T, r->hp_order, r->hp_bstart, r->hp_scratch, st, true);
         if (e != GSP_OK) return e;
         AdjDev A;
@@ -925,16 +948,16 @@ gsp_status gsp_render_grad(gsp_sppm* r, const float* d_dloss_dimg, float* d_grad
         A.hp_mask = (uint32_t)(r->hp_T - 1);
         A.inv_hp = 1.0f / hp_cell;
         A.rmax = r->P.r0;
-        A.spos = r->spos;
-        A.spay = r->spay;
-        A.order = r->last_order;
-        A.d_total = r->counters;
+        A.slots = r->slots;
+        A.list = r->vals[0];
+        A.tile_count = r->hist;
+        A.tile_stride = (int64_t)list.per_tile * r->slots_per_path;
         A.badj = r->badj;
         A.work = r->count_work ? r->work : nullptr;
         A.hp_rec = r->hp_rec;
-        if (A.work) k_work_add<<<1, 1, 0, st>>>(A.work + kWorkDeposits, r->counters);
+        if (A.work) k_work_sum<<<1, 256, 0, st>>>(A.work + kWorkDeposits, A.tile_count, list.tiles);
         k_adj_hp_records<<<blocks(r->npix, 256), 256, 0, st>>>(A, r->npix, r->hp_rec);
-        k_adj_photons<GSP_ADJ_LANES><<<grid * GSP_ADJ_LANES, 128, 0, st>>>(A);
+        k_adj_photons<GSP_ADJ_LANES><<<dim3(list.tiles, GSP_ADJ_COLUMNS), 128, 0, st>>>(A);
         k_adj_pixels<<<grid, 256, 0, st>>>(r->hx, r->hw, A.rhist, r->shist + (size_t)i * r->npix, d_dloss_dimg,
                                            r->npix, r->gacc, nmat);
         k_adj_paths<<<grid, 128, 0, st>>>(r->slots, r->pcount, r->smat, r->badj, r->scene->d_mats, r->np, r->gacc,
@@ -1685,7 +1708,9 @@ int64_t gsp_sppm_last_deposits(gsp_sppm* r, uint32_t* h_ids, int64_t capacity) {
 // ping-pong buffers, the radix histogram, scan partials and the device copy of n.
 int64_t gsp_grid_scratch_words(int64_t n, int64_t T) { return gsp_grid_scratch_words_c(n, T); }
 
-// Exact hash grid of n points: keys -> counts -> in-place bucket scan -> stable radix sort.
+// Exact hash grid of n points (hash_grid.cuh), or for more than 2^kGridMaxBits buckets: keys ->
+// counts -> in-place bucket scan -> stable radix sort. With skip_invalid, points whose w holds a
+// negative integer are in no bucket; the order of the others ends at bstart[T].
 gsp_status gsp_grid_build_with(const float4* pos, int64_t n, float cell_h, int64_t T, uint32_t* order,
                                uint32_t* bstart, uint32_t* scratch, cudaStream_t st, bool skip_invalid) {
     int tbits = 0;
@@ -1698,6 +1723,12 @@ gsp_status gsp_grid_build_with(const float4* pos, int64_t n, float cell_h, int64
     uint32_t* hist = vb + n;
     uint32_t* nbuf = hist + gsp_sort_hist_elems();
     uint32_t* tmp = nbuf + 64;
+    if (tbits - (skip_invalid ? 1 : 0) <= kGridMaxBits) {
+        GSP_CUDA_TRY(grid_launch(GridIn{pos, nullptr, n, 1, skip_invalid ? 1 : 0, 1.0f / cell_h, (uint32_t)(T - 1)},
+                                 tbits - (skip_invalid ? 1 : 0), ka, va, (uint2*)kb, hist, order, nullptr, nullptr, bstart, nullptr,
+                                 nullptr, st));
+        return GSP_OK;
+    }
     GSP_CUDA_TRY(cudaMemsetAsync(bstart, 0, (size_t)T * sizeof(uint32_t), st));
     k_store_u32<<<1, 1, 0, st>>>(nbuf, (uint32_t)n);
     if (n > 0)

@@ -11,7 +11,6 @@ namespace gspd {
 // ------------------------------------------------------------------------------------------
 // exact hash-grid deposit: compaction in id order, bucket keys, bucket counts
 // ------------------------------------------------------------------------------------------
-// keys == nullptr: the compaction alone (slot of each deposit in path order, no buckets).
 __global__ void __launch_bounds__(256)
 k_compact(const float4* __restrict__ slots, const uint32_t* __restrict__ pcount,
           const uint32_t* __restrict__ poff, int64_t np, int32_t slots_per_path, float inv_h,
@@ -23,7 +22,6 @@ k_compact(const float4* __restrict__ slots, const uint32_t* __restrict__ pcount,
     for (uint32_t i = 0; i < c; ++i) {
         const uint32_t slot = (uint32_t)k * slots_per_path + i;
         vals[off + i] = slot;
-        if (!keys) continue;
         const float4 a = slots[2 * (size_t)slot];
         const uint32_t b = bucket_of(f3(a), inv_h, tmask);
         keys[off + i] = b;
@@ -62,6 +60,8 @@ struct GatherDev {
     const float4* __restrict__ slots;
     const unsigned long long* __restrict__ entry;
     const uint32_t* __restrict__ ecount;
+    const uint32_t* __restrict__ pcount;  // deposits per path, summed into *total (zeroed before) for diagnostics
+    uint32_t* __restrict__ total;
     int64_t npix;
     float* __restrict__ rhist;  // optional: [pass][npix] radius each pixel gathered with (gradient)
     float4* __restrict__ shist; // optional: [pass][npix] sum of the gathered photons' flux (gradient)
@@ -133,6 +133,10 @@ __device__ __forceinline__ void cell_range(float x, float R, float inv_h, int32_
 // cell edge is >= 2 r0 in this mode).
 __global__ void __launch_bounds__(128) k_gather_stoch(GatherDev G, PassDev P) {
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    uint32_t deposits = 0;
+    for (int64_t k = p; k < P.np; k += (int64_t)gridDim.x * blockDim.x) deposits += G.pcount[k];
+    deposits = __reduce_add_sync(0xffffffffu, deposits);
+    if ((threadIdx.x & 31) == 0 && deposits) atomicAdd(G.total, deposits);
     if (p >= G.npix) return;
     const float4 hxp = G.hx[p];
     float4 s1 = G.st1[p];
@@ -396,10 +400,10 @@ struct AdjDev {
     uint32_t hp_mask;
     float inv_hp;                       // 1 / hit-point cell size
     float rmax;                         // largest gather radius (r0)
-    const float4* __restrict__ spos;    // deposits of the pass, bucket-sorted
-    const float4* __restrict__ spay;
-    const uint32_t* __restrict__ order; // sorted deposit -> photon slot
-    const uint32_t* __restrict__ d_total;
+    const float4* __restrict__ slots;   // deposits of the pass
+    const uint32_t* __restrict__ list;  // their slots, per tile of paths (k_grid_tiles)
+    const uint32_t* __restrict__ tile_count;
+    int64_t tile_stride;                // list words per tile
     float4* __restrict__ badj;          // per slot: B_k, the weight of Phi_k in the loss
     unsigned long long* work;           // work counters, or null
 };
@@ -411,7 +415,7 @@ struct AdjDev {
 // forming it per photon).
 __global__ void __launch_bounds__(256) k_adj_hp_records(AdjDev A, int64_t npix, float4* __restrict__ rec) {
     const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= npix) return;
+    if (j >= npix || j >= A.hp_bstart[(size_t)A.hp_mask + 1]) return;  // pixels without a hit point are in no bucket
     const uint32_t p = A.hp_order[j];
     const float R = A.rhist[p];
     const float3 gp = make_float3(A.g[3 * p], A.g[3 * p + 1], A.g[3 * p + 2]);
@@ -427,15 +431,18 @@ __global__ void __launch_bounds__(256) k_adj_hp_records(AdjDev A, int64_t npix, 
 // of Phi_k in the loss. A group of L lanes serves one deposit: it visits the hit-point grid's cells
 // overlapping xk +- r0 (no radius exceeds r0), its lanes split each bucket's hit points, and a hit
 // point counts only in its own cell. Group sums combine by a fixed butterfly; nothing is atomic.
+// blockIdx.x is the tile of paths whose deposits the block serves, with the blocks of its column.
 template <int L>
 __global__ void __launch_bounds__(128) k_adj_photons(AdjDev A) {
-    const int nd = (int)*A.d_total;
+    const int nd = (int)A.tile_count[blockIdx.x];
+    const uint32_t* list = A.list + blockIdx.x * A.tile_stride;
     const int gl = threadIdx.x & (L - 1);
     const int lane = threadIdx.x & 31;
     const uint32_t gmask = (L == 32 ? 0xffffffffu : ((1u << L) - 1u)) << (lane & ~(L - 1));
-    const int groups = (int)(((int64_t)gridDim.x * blockDim.x) / L);
-    for (int i = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / L); i < nd; i += groups) {
-        const float4 a = A.spos[i], c = A.spay[i];
+    const int groups = (int)(gridDim.y * blockDim.x) / L;
+    for (int i = (int)(blockIdx.y * blockDim.x + threadIdx.x) / L; i < nd; i += groups) {
+        const uint32_t slot = list[i];
+        const float4 a = A.slots[2 * (size_t)slot], c = A.slots[2 * (size_t)slot + 1];
         const float3 xk = f3(a);
         const uint32_t dir = __float_as_uint(c.w);
         int32_t lx, hx, ly, hy, lz, hz;
@@ -467,7 +474,7 @@ __global__ void __launch_bounds__(128) k_adj_photons(AdjDev A) {
             B.y += __shfl_xor_sync(gmask, B.y, off, L);
             B.z += __shfl_xor_sync(gmask, B.z, off, L);
         }
-        if (gl == 0) A.badj[A.order[i]] = make_float4(B.x, B.y, B.z, 0.0f);
+        if (gl == 0) A.badj[slot] = make_float4(B.x, B.y, B.z, 0.0f);
         if (A.work) atomicAdd(A.work + kWorkHitsScanned, (unsigned long long)scanned);
     }
 }
@@ -637,6 +644,13 @@ __global__ void k_store_u32(uint32_t* p, uint32_t v) { *p = v; }
 __global__ void k_add_u32(uint32_t* p, uint32_t v) { *p += v; }
 
 __global__ void k_work_add(unsigned long long* p, const uint32_t* v) { *p += *v; }
+
+// Adds the n words of v to *p (one block).
+__global__ void k_work_sum(unsigned long long* p, const uint32_t* __restrict__ v, int32_t n) {
+    unsigned long long s = 0;
+    for (int32_t i = threadIdx.x; i < n; i += blockDim.x) s += v[i];
+    if (s) atomicAdd(p, s);
+}
 
 __global__ void k_fill_u64(unsigned long long* p, int64_t n, unsigned long long v) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) p[i] = v;

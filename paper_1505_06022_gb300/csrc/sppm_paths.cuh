@@ -6,6 +6,7 @@
 
 #include "devcommon.cuh"
 #include "gsp_internal.h"
+#include "hash_grid.cuh"
 #include "launch.h"
 #include "persist.cuh"
 #include "wide.cuh"
@@ -140,23 +141,6 @@ __device__ __forceinline__ float3 oct_decode(uint32_t e) {
     v.x += v.x >= 0.0f ? -t : t;
     v.y += v.y >= 0.0f ? -t : t;
     return normalize3(v);
-}
-
-// Teschner et al. 2003 spatial hash of an integer cell, 32-bit wraparound.
-__device__ __forceinline__ uint32_t cell_hash(int32_t ix, int32_t iy, int32_t iz, uint32_t mask) {
-    return (((uint32_t)ix * 73856093u) ^ ((uint32_t)iy * 19349663u) ^ ((uint32_t)iz * 83492791u)) & mask;
-}
-
-// Cell lattice shifted by 0.381966 of a cell so that axis-aligned walls at multiples of the
-// cell size (e.g. a floor at 0) do not lie on cell boundaries.
-constexpr float kCellOffset = 0.381966f;
-
-__device__ __forceinline__ int32_t cell_of(float x, float inv_h) {
-    return (int32_t)floorf(fmaf(x, inv_h, kCellOffset));
-}
-
-__device__ __forceinline__ uint32_t bucket_of(float3 x, float inv_h, uint32_t mask) {
-    return cell_hash(cell_of(x.x, inv_h), cell_of(x.y, inv_h), cell_of(x.z, inv_h), mask);
 }
 
 // ------------------------------------------------------------------------------------------
