@@ -69,7 +69,7 @@ struct gsp_sppm {
     // The tracing of a pass: its path queues and counters, and the outputs its deposit and gather
     // read. Two sets, so that the tracing of pass i + 1 runs while pass i is gathered and while
     // the longest paths of pass i are still being traced (gsp_sppm_pass with several passes);
-    // both sets are made at creation in exact mode (else on first use). hx .. rlist alias the set
+    // both are made at creation. hx .. rlist alias the set
     // in use.
     struct TraceBuf {
         float4 *hx = nullptr, *hn = nullptr, *hf = nullptr, *hd = nullptr, *slots = nullptr;
@@ -129,14 +129,35 @@ struct gsp_sppm {
 
 namespace {
 
-template <class T>
-cudaError_t alloc(gsp_sppm* r, T** p, int64_t count) {
-    *p = nullptr;
-    if (count <= 0) return cudaSuccess;
-    cudaError_t e = cudaMalloc((void**)p, (size_t)count * sizeof(T));
-    if (e == cudaSuccess) r->allocs.push_back((void*)*p);
-    return e;
-}
+// Several device arrays from one allocation: their sizes are noted, then make() allocates their sum
+// and sets the pointers (all null and nothing allocated on failure). A renderer has about 70 arrays; one
+// cudaMalloc and cudaFree each took 3.8 of the 4.4 ms that making and freeing a 256x256 renderer of
+// 262,144 photons with gradients takes, one for all of them ALLOCMS ms (the driver maps the same GB).
+struct Arena {
+    struct Item {
+        void** p;
+        size_t offset;
+    };
+    std::vector<Item> items;
+    size_t total = 0;
+
+    template <class T>
+    void add(T** p, int64_t count) {
+        *p = nullptr;
+        if (count <= 0) return;
+        items.push_back({(void**)p, total});
+        total += ((size_t)count * sizeof(T) + 255) / 256 * 256;  // as aligned as cudaMalloc's own
+    }
+    cudaError_t make(gsp_sppm* r) {
+        if (!total) return cudaSuccess;
+        char* base = nullptr;
+        const cudaError_t e = cudaMalloc((void**)&base, total);
+        if (e != cudaSuccess) return e;
+        r->allocs.push_back(base);
+        for (const Item& i : items) *i.p = base + i.offset;
+        return cudaSuccess;
+    }
+};
 
 void free_all(gsp_sppm* r) {
     for (void* p : r->allocs) cudaFree(p);
@@ -162,11 +183,21 @@ void use_buf(gsp_sppm* r, int j) {
     r->ecount = r->tb[j].ecount;
 }
 
-// The path queues and counters of trace set j.
-template <class AllocF>
-void alloc_trace_queues(gsp_sppm* r, int j, AllocF&& A) {
+// Trace set j: its outputs, path queues and counters.
+void add_trace_set(gsp_sppm* r, int j, Arena& arena) {
     const int64_t nq = r->P.photon_mode == GSP_FULL_PATH ? r->np : 0;
     auto& t = r->tb[j];
+    const auto A = [&](auto** p, int64_t n) { arena.add(p, n); };
+    A(&t.hx, r->npix);
+    A(&t.hn, r->npix);
+    A(&t.hf, r->npix);
+    A(&t.hd, r->npix);
+    A(&t.slots, 2 * r->slot_cap);
+    A(&t.pcount, r->np);
+    if (r->P.hash_mode == GSP_STOCHASTIC) {  // a table per trace set, so that passes overlap
+        A(&t.entry, r->T);
+        A(&t.ecount, r->T);
+    }
     for (int b = 0; b < 2; ++b) {
         A(&t.q[b].ray, 2 * nq);
         A(&t.q[b].w, nq);
@@ -191,8 +222,6 @@ inline unsigned blocks(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
 }  // namespace
 
 extern "C" {
-
-static gsp_status ensure_second_buffer(gsp_sppm* r);
 
 gsp_status gsp_sppm_create(gsp_scene* s, const gsp_sppm_params* params, gsp_sppm** out) {
     if (!s || !params || !out) return GSP_ERR_INVALID_ARG;
@@ -312,19 +341,12 @@ gsp_status gsp_sppm_create(gsp_scene* s, const gsp_sppm_params* params, gsp_sppm
         r->cam.w = c.width;
         r->cam.h = c.height;
     }
-    cudaError_t e = cudaSuccess;
-    auto A = [&](auto** p, int64_t n) { if (e == cudaSuccess) e = alloc(r, p, n); };
+    Arena arena;
+    const auto A = [&](auto** p, int64_t n) { arena.add(p, n); };
     A(&r->d_emit, 5 * (int64_t)ne);
     A(&r->d_cdf, ne);
     A(&r->st0, r->npix);
     A(&r->st1, r->npix);
-    A(&r->tb[0].hx, r->npix);
-    A(&r->tb[0].hn, r->npix);
-    A(&r->tb[0].hf, r->npix);
-    A(&r->tb[0].hd, r->npix);
-    A(&r->tb[0].slots, 2 * r->slot_cap);
-    A(&r->tb[0].pcount, r->np);
-    use_buf(r, 0);
     A(&r->counters, 16);
     A(&r->started, 1);
     A(&r->work, kWorkCounts);
@@ -332,7 +354,6 @@ gsp_status gsp_sppm_create(gsp_scene* s, const gsp_sppm_params* params, gsp_sppm
         A(&r->keys[0], r->slot_cap);
         A(&r->vals[0], r->slot_cap);
         A(&r->keys[1], 2 * r->slot_cap);  // the parts' {bucket, slot} pairs, or the radix sort's second pair
-        r->vals[1] = r->keys[1] ? r->keys[1] + r->slot_cap : nullptr;
         A(&r->hist, gsp_sort_hist_elems());
         if (r->tbits > kGridMaxBits) {  // the radix sort's buffers
             A(&r->poff, r->np);
@@ -345,9 +366,6 @@ gsp_status gsp_sppm_create(gsp_scene* s, const gsp_sppm_params* params, gsp_sppm
         A(&r->spay, r->slot_cap);
         // the heavy-query split pays on large images; on small ones its extra launch costs more
         if (r->npix >= kHeavyMinPixels) A(&r->heavy, r->npix);
-    } else {
-        A(&r->tb[0].entry, r->T);  // one table per trace set, so that passes overlap
-        A(&r->tb[0].ecount, r->T);
     }
     r->qcap = std::max(r->npix, P.photon_mode == GSP_FULL_PATH ? r->np : (int64_t)0);
     // gather lanes per hit point: a small image's gather has too few hit points to fill the GPU
@@ -356,13 +374,19 @@ gsp_status gsp_sppm_create(gsp_scene* s, const gsp_sppm_params* params, gsp_sppm
     r->eye_steps = 0;     // no wavefront steps: the persistent path kernel (per-lane refill)
     r->photon_steps = 0;  // traces every bounce; a step costs a closest-hit launch over the whole
                           // queue plus a shade launch, and waits for its slowest ray
-    alloc_trace_queues(r, 0, A);
-    use_buf(r, 0);
+    for (int j = 0; j < 2; ++j) add_trace_set(r, j, arena);  // several passes are traced into both
     if (P.photon_mode == GSP_REGEN) {
         A(&r->ro, r->np);
         A(&r->rd, r->np);
         A(&r->rphi, r->np);
     }
+    cudaError_t e = arena.make(r);
+    if (r->keys[1]) r->vals[1] = r->keys[1] + r->slot_cap;
+    use_buf(r, 0);
+    for (cudaStream_t& t : r->tstream)
+        if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&t, cudaStreamNonBlocking);
+    for (cudaEvent_t* ev : {&r->ev_start, &r->ev_traced[0], &r->ev_traced[1], &r->ev_free[0], &r->ev_free[1]})
+        if (e == cudaSuccess) e = cudaEventCreateWithFlags(ev, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaMemcpy(r->d_emit, emit.data(), emit.size() * sizeof(float4), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(r->d_cdf, cdff.data(), cdff.size() * sizeof(float), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) {
@@ -376,20 +400,11 @@ gsp_status gsp_sppm_create(gsp_scene* s, const gsp_sppm_params* params, gsp_sppm
         if (e == cudaSuccess) e = cudaMemset(r->rd, 0, r->np * sizeof(float4));
         if (e == cudaSuccess) e = cudaMemset(r->rphi, 0, r->np * sizeof(float4));
     }
-    // several passes are traced into both trace sets: the second one is made now, so that no
-    // pass allocates
-    if (e == cudaSuccess) {
-        const gsp_status se = ensure_second_buffer(r);
-        if (se != GSP_OK) {
-            gsp_sppm_destroy(r);
-            return se;
-        }
-    }
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e != cudaSuccess) {
-        free_all(r);
-        delete r;
-        return gsp_cuda_fail(e);
+        const gsp_status se = gsp_cuda_fail(e);
+        gsp_sppm_destroy(r);
+        return se;
     }
     *out = r;
     return GSP_OK;
@@ -738,40 +753,6 @@ static gsp_status sppm_one_pass(gsp_sppm* r, cudaStream_t st, bool graph = false
     return GSP_OK;
 }
 
-// The second set of trace buffers, the tracing streams and their events (at creation in exact
-// mode, else on first use).
-static gsp_status ensure_second_buffer(gsp_sppm* r) {
-    if (r->tb[1].hx && r->tb[1].qctr && (!r->grad || r->tb[1].hw) &&
-        (r->P.hash_mode != GSP_STOCHASTIC || r->tb[1].entry))
-        return GSP_OK;
-    cudaError_t e = cudaSuccess;
-    auto A = [&](auto** p, int64_t n) {
-        if (e == cudaSuccess && !*p) e = alloc(r, p, n);
-    };
-    A(&r->tb[1].hx, r->npix);
-    A(&r->tb[1].hn, r->npix);
-    A(&r->tb[1].hf, r->npix);
-    A(&r->tb[1].hd, r->npix);
-    A(&r->tb[1].slots, 2 * r->slot_cap);
-    A(&r->tb[1].pcount, r->np);
-    if (r->grad) {
-        A(&r->tb[1].hw, r->npix);
-        A(&r->tb[1].smat, r->slot_cap);
-    }
-    if (r->P.hash_mode == GSP_STOCHASTIC) {
-        A(&r->tb[1].entry, r->T);
-        A(&r->tb[1].ecount, r->T);
-    }
-    if (!r->tb[1].qctr) alloc_trace_queues(r, 1, A);
-    for (cudaStream_t& t : r->tstream)
-        if (e == cudaSuccess && !t) e = cudaStreamCreateWithFlags(&t, cudaStreamNonBlocking);
-    for (cudaEvent_t* ev : {&r->ev_start, &r->ev_traced[0], &r->ev_traced[1], &r->ev_free[0], &r->ev_free[1]})
-        if (e == cudaSuccess && !*ev) e = cudaEventCreateWithFlags(ev, cudaEventDisableTiming);
-    if (e != cudaSuccess) return gsp_cuda_fail(e);
-    use_buf(r, r->cur);
-    return GSP_OK;
-}
-
 // Several passes, pass i traced on tracing stream i % 2 into trace set i % 2 while the caller's
 // stream deposits and gathers the pass before: the tracing of pass i + 1 starts as soon as its
 // set has been gathered (pass i - 1), so it runs beside the long tail of pass i's path kernel,
@@ -780,8 +761,6 @@ static gsp_status ensure_second_buffer(gsp_sppm* r) {
 // those of one pass after the other. Exact hashing only (stochastic hashing shares its table
 // between the two halves).
 static gsp_status passes_overlapped(gsp_sppm* r, int32_t npasses, cudaStream_t st) {
-    gsp_status se = ensure_second_buffer(r);
-    if (se != GSP_OK) return se;
     // the tracing streams start after everything the caller queued before
     GSP_CUDA_TRY(cudaEventRecord(r->ev_start, st));
     for (cudaStream_t t : r->tstream) GSP_CUDA_TRY(cudaStreamWaitEvent(t, r->ev_start, 0));
@@ -876,21 +855,21 @@ gsp_status gsp_sppm_enable_grad(gsp_sppm* r, int32_t max_passes) {
     GSP_CUDA_TRY(cudaSetDevice(r->scene->ctx->device));
     r->hp_T = 1;
     while (r->hp_T < 2 * r->npix) r->hp_T *= 2;
-    cudaError_t e = cudaSuccess;
-    auto A = [&](auto** p, int64_t n) { if (e == cudaSuccess) e = alloc(r, p, n); };
+    Arena arena;
+    const auto A = [&](auto** p, int64_t n) { arena.add(p, n); };
     A(&r->rhist, (int64_t)max_passes * r->npix);
     A(&r->shist, (int64_t)max_passes * r->npix);
-    for (int j = 0; j < 2; ++j)
-        if (r->tb[j].hx) {
-            A(&r->tb[j].hw, r->npix);
-            A(&r->tb[j].smat, r->slot_cap);
-        }
+    for (auto& t : r->tb) {
+        A(&t.hw, r->npix);
+        A(&t.smat, r->slot_cap);
+    }
     A(&r->badj, r->slot_cap);
     A(&r->gacc, (int64_t)kMaxGradMats * 3 + 3);
     A(&r->hp_order, r->npix);
     A(&r->hp_bstart, r->hp_T + 1);
     A(&r->hp_scratch, gsp_grid_scratch_words(r->npix, r->hp_T));
     A(&r->hp_rec, 3 * r->npix);
+    const cudaError_t e = arena.make(r);
     if (e != cudaSuccess) return gsp_cuda_fail(e);
     r->grad = true;
     r->grad_max_passes = max_passes;
@@ -912,8 +891,7 @@ gsp_status gsp_render_grad(gsp_sppm* r, const float* d_dloss_dimg, float* d_grad
     const int grid = 4 * sm_count(r->scene->ctx->device);
     // Pass i + 1 is replayed on the other tracing stream into the other trace set while the adjoint
     // kernels of pass i run on the caller's stream (the same double buffering as gsp_sppm_pass).
-    gsp_status e = ensure_second_buffer(r);
-    if (e != GSP_OK) return e;
+    gsp_status e = GSP_OK;
     GSP_CUDA_TRY(cudaEventRecord(r->ev_start, st));
     for (cudaStream_t t : r->tstream) GSP_CUDA_TRY(cudaStreamWaitEvent(t, r->ev_start, 0));
     for (int64_t i = 0; i < r->passes; ++i) {
@@ -1057,11 +1035,6 @@ static gsp_status batch_capture_fused(gsp_batch* b, cudaStream_t st, int K, cuda
         GSP_CUDA_TRY(cudaMalloc(&b->d_jobs, 3 * (size_t)n * sizeof(PathJob)));
         GSP_CUDA_TRY(cudaMalloc(&b->d_ctr, 3 * sizeof(uint32_t)));
     }
-    if (K == 2)
-        for (gsp_sppm* r : b->rs) {  // both trace sets (made outside the capture)
-            gsp_status se = ensure_second_buffer(r);
-            if (se != GSP_OK) return se;
-        }
     // one launch for all: shading code if any scene has shading data, the walk all renderers share
     // (every scene has its links)
     bool shade = false;
@@ -1416,7 +1389,6 @@ gsp_status gsp_sppm_autotune(gsp_sppm* r, int32_t trial_passes, gsp_tune_result*
     // way gsp_sppm_pass runs them (overlapped), which changes which settings win:
     // the overlap hides the path kernel's tail.
     const bool overlap = trial_passes >= 2;
-    if (overlap) e = ensure_second_buffer(t);
     auto trial = [&](const Cand& c) {
         if (ce != cudaSuccess || e != GSP_OK) return;
         t->eye_steps = c.es;
