@@ -186,7 +186,7 @@ k_trace_wide(DevScene S, const float4* __restrict__ rays, int64_t n, const uint3
         } else if (quad)
             quad_steps<GSP_WIDE_KEEP_TRACE>(S.wide, S.tris, st, w, stk, ray >= 0);
         else
-            wide_steps<GSP_WIDE_KEEP_TRACE>(S.wide, S.tris, st, w, stk, ray >= 0);
+            wide_steps(S.wide, S.tris, st, w, stk, ray >= 0, GSP_WIDE_KEEP_TRACE);
         const bool fin = ray >= 0 && w.cur == kWalkDone;
         bool flag = false;
         if (fin && (!quad || (lane & 3) == 0)) {

@@ -7,8 +7,8 @@
 // the pass's direct term), photon pass (whole paths, or one bounce per thread with path
 // regeneration), hash-grid deposit, and the fused range query + progressive update (which also
 // folds the pass's direct term into the pixel state). The eye and photon passes are emission
-// kernels, optional wavefront steps, and one persistent path kernel (k_paths; k_paths_multi for
-// a batch of renderers); several passes overlap on three streams (passes_overlapped: two
+// kernels, optional wavefront steps, and one persistent path kernel (k_paths_pool over the four-wide
+// tree, else k_paths, or k_paths_multi for a batch of renderers); several passes overlap on three streams (passes_overlapped: two
 // tracing streams, one per trace set, and the caller's stream for the deposits and gathers).
 //
 // Device layout (all library-owned, sized at creation):
@@ -33,6 +33,7 @@
 #include "gsp_internal.h"
 #include "hash_grid.cuh"
 #include "launch.h"
+#include "path_pool.cuh"
 #include "persist.cuh"
 #include "scan_sort.h"
 #include "sppm_gather.cuh"
@@ -132,7 +133,8 @@ namespace {
 // Several device arrays from one allocation: their sizes are noted, then make() allocates their sum
 // and sets the pointers (all null and nothing allocated on failure). A renderer has about 70 arrays; one
 // cudaMalloc and cudaFree each took 3.8 of the 4.4 ms that making and freeing a 256x256 renderer of
-// 262,144 photons with gradients takes, one for all of them ALLOCMS ms (the driver maps the same GB).
+// 262,144 photons with gradients takes; with one for all of them it takes 1.3 ms (the driver still maps
+// the same GB), and a gradient step of eight passes 6.1 instead of 9.3 ms.
 struct Arena {
     struct Item {
         void** p;
@@ -488,10 +490,10 @@ static int path_grid(int64_t items, int device, int walk, bool shade, bool multi
         const void* const kernels[2][3][2] = {
             {{(const void*)k_paths<kLinks, false, false>, (const void*)k_paths<kLinks, true, false>},
              {(const void*)k_paths<kStack, false, false>, (const void*)k_paths<kStack, true, false>},
-             {(const void*)k_paths<kWide, false, false>, (const void*)k_paths<kWide, true, false>}},
+             {(const void*)k_paths_pool<false, false, false>, (const void*)k_paths_pool<false, true, false>}},
             {{(const void*)k_paths_multi<kLinks, false>, (const void*)k_paths_multi<kLinks, true>},
              {(const void*)k_paths_multi<kStack, false>, (const void*)k_paths_multi<kStack, true>},
-             {(const void*)k_paths_multi<kWide, false>, (const void*)k_paths_multi<kWide, true>}}};
+             {(const void*)k_paths_pool<true, false, false>, (const void*)k_paths_pool<true, true, false>}}};
         int b = 0;
         cudaDeviceGetAttribute(&sms[device], cudaDevAttrMultiProcessorCount, device);
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, kernels[multi][walk][shade], kTraceThreads, 0);
@@ -504,6 +506,12 @@ static int path_grid(int64_t items, int device, int walk, bool shade, bool multi
 
 // Paths a warp of k_paths / k_photon_regen takes at once.
 static int path_chunk(int64_t items, unsigned grid) { return gsp_chunk(items, (int64_t)grid * (kTraceThreads / 32), kPathChunk); }
+
+// Paths a warp of k_paths_pool keeps: half of its share, so that the other half goes to whoever is
+// ahead, within 32 and kPool.
+static int pool_size(int64_t items, unsigned grid) {
+    return (int)std::max<int64_t>(32, std::min<int64_t>(kPool, items / ((int64_t)grid * (kTraceThreads / 32) * 2)));
+}
 
 // Eye pass up to the persistent kernel: primary rays, then eye_steps wavefront steps. Returns in
 // b the queue holding the paths still going (none if b > max_eye_depth).
@@ -531,7 +539,7 @@ static gsp_status eye_front(gsp_sppm* r, const PassDev& P, const EyeOut& O, cuda
 // Photon pass up to the persistent kernel: emission and photon_steps wavefront steps of whole
 // paths (b = the queue still going; none if b >= max_photon_depth), or the one-bounce-per-thread
 // pass of Sec. 3.3 (b = -1).
-static gsp_status photon_front(gsp_sppm* r, const PassDev& P, const DepositDev& D, cudaStream_t st, int& b) {
+static gsp_status photon_front(gsp_sppm* r, const PassDev& P, const DepositDev& D, cudaStream_t st, int& b, bool merged) {
     gsp_scene* s = r->scene;
     const DevScene S = gsp_dev_scene(s);
     uint32_t* qn = r->qctr + 8;
@@ -554,7 +562,7 @@ static gsp_status photon_front(gsp_sppm* r, const PassDev& P, const DepositDev& 
             else
                 k_photon_shade<false><<<shade_blocks(r->np, s->ctx->device), 256, 0, st>>>(S, P, D, cur, r->q[(b + 1) & 1], qn, b, tctr);
         }
-    } else {
+    } else if (!merged) {
         RegenDev R{r->ro, r->rd, r->rphi, r->started};
         GSP_CUDA_TRY(cudaMemsetAsync(r->qctr + 13, 0, sizeof(uint32_t), st));
         const int walk = path_walk(r, S);
@@ -576,12 +584,14 @@ static gsp_status photon_front(gsp_sppm* r, const PassDev& P, const DepositDev& 
 
 // Eye and photon passes of one pass (Sec. 2): both fronts, then one persistent kernel finishes
 // the eye and photon paths still going.
-// Both fronts of a pass; J describes the paths still going (J.nchunks == 0: none).
+// Both fronts of a pass; J describes the paths still going (J.nchunks == 0: none). merge_regen: the
+// one-bounce photon pass may be left to k_paths_pool too (J.nregen), beside the eye paths' tail.
 static gsp_status paths_front(gsp_sppm* r, const PassDev& P, const EyeOut& O, const DepositDev& D, cudaStream_t st,
-                              PathJob& J) {
+                              PathJob& J, bool merge_regen = false) {
     int be = 0, bp = -1;
     gsp_status e = eye_front(r, P, O, st, be);
-    if (e == GSP_OK) e = photon_front(r, P, D, st, bp);
+    const bool merged = merge_regen && r->P.photon_mode == GSP_REGEN && path_walk(r, gsp_dev_scene(r->scene)) == kWide;
+    if (e == GSP_OK) e = photon_front(r, P, D, st, bp, merged);
     if (e != GSP_OK) return e;
     const bool eye_left = be <= r->P.max_eye_depth;
     const bool ph_left = bp >= 0 && bp < r->P.max_photon_depth;
@@ -594,7 +604,10 @@ static gsp_status paths_front(gsp_sppm* r, const PassDev& P, const EyeOut& O, co
     J.ne_ptr = eye_left ? r->qctr + 4 + be % 3 : nullptr;
     J.np_ptr = ph_left ? r->qctr + 8 + bp % 3 : nullptr;
     J.first_chunk = 0;
-    const int64_t items = (eye_left ? r->npix : 0) + (ph_left ? r->np : 0);
+    J.nregen = merged ? (int32_t)r->np : 0;
+    J.E = EmitDev{r->d_emit, r->d_cdf, r->nemit};
+    J.R = RegenDev{r->ro, r->rd, r->rphi, r->started};
+    const int64_t items = (eye_left ? r->npix : 0) + (ph_left ? r->np : 0) + J.nregen;
     J.nchunks = (int32_t)((items + kMultiChunk - 1) / kMultiChunk);
     return GSP_OK;
 }
@@ -602,11 +615,11 @@ static gsp_status paths_front(gsp_sppm* r, const PassDev& P, const EyeOut& O, co
 static gsp_status stage_paths(gsp_sppm* r, const PassDev& P, const EyeOut& O, const DepositDev& D, cudaStream_t st) {
     NvtxRange nvtx("gsp: eye + photon paths");
     PathJob J;
-    gsp_status e = paths_front(r, P, O, D, st, J);
+    gsp_status e = paths_front(r, P, O, D, st, J, true);
     if (e != GSP_OK) return e;
     if (J.nchunks > 0) {
         const int walk = path_walk(r, J.S);
-        const int64_t items = (J.ne_ptr ? r->npix : 0) + (J.np_ptr ? r->np : 0);
+        const int64_t items = (J.ne_ptr ? r->npix : 0) + (J.np_ptr ? r->np : 0) + J.nregen;
         const unsigned grid = (unsigned)path_grid(items, r->scene->ctx->device, walk, J.S.attr != nullptr);
         const auto paths = [&](auto kernel) {
             kernel<<<grid, kTraceThreads, 0, st>>>(J.S, P, J.qe, O, J.ne_ptr, J.qp, D, J.np_ptr, r->qctr + 12,
@@ -615,7 +628,16 @@ static gsp_status stage_paths(gsp_sppm* r, const PassDev& P, const EyeOut& O, co
         if (walk == kStack)
             J.S.attr ? paths(k_paths<kStack, true, false>) : paths(k_paths<kStack, false, false>);
         else if (walk == kWide)
-            J.S.attr ? paths(k_paths<kWide, true, false>) : paths(k_paths<kWide, false, false>);
+        {
+            const auto pooled = [&](auto kernel) {
+                kernel<<<grid, kTraceThreads, 0, st>>>(J, nullptr, 0, 0, r->qctr + 12, path_chunk(items, grid),
+                                                       pool_size(items, grid));
+            };
+            if (J.nregen)
+                J.S.attr ? pooled(k_paths_pool<false, true, true>) : pooled(k_paths_pool<false, false, true>);
+            else
+                J.S.attr ? pooled(k_paths_pool<false, true, false>) : pooled(k_paths_pool<false, false, false>);
+        }
         else if (P.work)
             J.S.attr ? paths(k_paths<kLinks, true, true>) : paths(k_paths<kLinks, false, true>);
         else
@@ -1086,7 +1108,13 @@ static gsp_status batch_capture_fused(gsp_batch* b, cudaStream_t st, int K, cuda
                 if (walk == kStack)
                     shade ? multi(k_paths_multi<kStack, true>) : multi(k_paths_multi<kStack, false>);
                 else if (walk == kWide)
-                    shade ? multi(k_paths_multi<kWide, true>) : multi(k_paths_multi<kWide, false>);
+                {
+                    const auto pooled = [&](auto kernel) {
+                        kernel<<<grid, kTraceThreads, 0, ps>>>(PathJob{}, jt, n, total[k], ctr, 0,
+                                                               pool_size((int64_t)total[k] * kMultiChunk, grid));
+                    };
+                    shade ? pooled(k_paths_pool<true, true, false>) : pooled(k_paths_pool<true, false, false>);
+                }
                 else
                     shade ? multi(k_paths_multi<kLinks, true>) : multi(k_paths_multi<kLinks, false>);
                 ce = cudaGetLastError();

@@ -322,11 +322,7 @@ struct PathWalk<kWide> {
         wide_init(w);
     }
     __device__ __forceinline__ void steps(const DevScene& S, bool active, int32_t, uint32_t&) {
-        wide_steps<GSP_WIDE_KEEP>(S.wide, S.tris, st, w, stk, active);
-    }
-    __device__ __forceinline__ void finish(const DevScene& S, int owner, CoopScratch* sc) {
-        st = coop_wide(S.wide, S.tris, st, w, stk, owner, sc);
-        w.cur = kWalkDone;
+        wide_steps(S.wide, S.tris, st, w, stk, active, GSP_WIDE_KEEP);
     }
     __device__ __forceinline__ void quad_steps(const DevScene& S, bool active) {
         gspd::quad_steps<GSP_WIDE_KEEP>(S.wide, S.tris, st, w, stk, active);
@@ -380,42 +376,86 @@ struct EyeOut {
     float4* __restrict__ hw;  // optional: eye throughput w of each hit point (gradient replay)
 };
 
-// One eye-path interaction at a hit. Emission seen from the front is added to the pixel's
-// direct term of this pass (one path per pixel, so no atomics);
-// a diffuse hit records the hit point and ends the path; a mirror or dielectric bends the ray
-// (returns true: the path continues from x along the new d). Of lanes that hold the same path, the
-// one with `lead` writes.
+struct DepositDev {
+    float4* __restrict__ slots;          // 2 float4 per slot
+    uint32_t* __restrict__ pcount;       // deposits per path / thread
+    unsigned long long* __restrict__ entry;  // stochastic: min key per bucket
+    uint32_t* __restrict__ ecount;       // stochastic: photons per bucket
+    int32_t stochastic;
+    int32_t* __restrict__ smat;          // optional: material of each deposit's surface (gradient replay)
+};
+
+// One interaction of an eye or photon path at hit h. Eye path of pixel `id`: emission seen from the
+// front is added to the pixel's direct term of this pass (one path per pixel, so no atomics), and a
+// diffuse hit records the hit point and ends the path. Photon path: a diffuse hit deposits (record `rec`,
+// slot `slot`; ndep counts), survives with probability rr and leaves along a cosine-distributed
+// direction. A mirror or dielectric bends either. False when the path ends, else it goes on from o
+// along d with w updated. Of lanes that hold the same path, the one with `lead` writes. The two
+// kinds share the code (a path kernel's instruction fetches grow with every copy of it): the three
+// draws of a diffuse bounce are a loop, and are all made before the roulette decides, which changes
+// nothing (a path that ends draws no more).
 template <bool SHADE>
-__device__ __forceinline__ bool eye_interact(const DevScene& S, const PassDev& P, const EyeOut& O, int64_t p,
-                                             const Hit& h, float3& o, float3& d, float3& w, Rng& rng, bool lead = true) {
+__device__ __forceinline__ bool path_interact(const DevScene& S, const PassDev& P, const EyeOut& O, const DepositDev& D,
+                                              bool eye, int32_t id, const Hit& h, float3& o, float3& d, float3& w, Rng& rng,
+                                              uint32_t rec, uint32_t slot, uint32_t& ndep, bool lead = true) {
     const float4 sh = __ldg(S.shade + h.id);
     const float3 n = f3(sh);
     const int32_t mid = __float_as_int(sh.w);
     const Material m = load_mat(S, mid);
     const bool front = dot3(d, n) < 0.0f;
-    if (lead && front && emits(m)) {
-        float4 v = O.hd[p];
+    if (eye && lead && front && emits(m)) {
+        float4 v = O.hd[id];
         v.x += w.x * m.emission.x;
         v.y += w.y * m.emission.y;
         v.z += w.z * m.emission.z;
-        O.hd[p] = v;
+        O.hd[id] = v;
     }
     if (m.type == GSP_EMITTER) return false;
     const float3 x = madd3(d, h.t, o);
     const Surf sf = surface<SHADE>(S, h, o, d, n, m, mid);
     if (m.type == GSP_DIFFUSE) {
-        const float3 ns = front ? n : n * -1.0f;
-        const float3 wt = mul3(w, sf.tex);  // the hit point's weight without its albedo
-        const float3 f = mul3(wt, m.albedo) * (1.0f / kPi);
-        if (lead) {
-            O.hx[p] = make_float4(x.x, x.y, x.z, __int_as_float(mid));
-            O.hn[p] = make_float4(ns.x, ns.y, ns.z, 0.0f);
-            O.hf[p] = make_float4(f.x, f.y, f.z, 0.0f);
-            if (O.hw) O.hw[p] = make_float4(wt.x, wt.y, wt.z, 0.0f);
+        if (eye) {
+            if (lead) {
+                const float3 ns = front ? n : n * -1.0f;
+                const float3 wt = mul3(w, sf.tex);  // the hit point's weight without its albedo
+                const float3 f = mul3(wt, m.albedo) * (1.0f / kPi);
+                O.hx[id] = make_float4(x.x, x.y, x.z, __int_as_float(mid));
+                O.hn[id] = make_float4(ns.x, ns.y, ns.z, 0.0f);
+                O.hf[id] = make_float4(f.x, f.y, f.z, 0.0f);
+                if (O.hw) O.hw[id] = make_float4(wt.x, wt.y, wt.z, 0.0f);
+            }
+            return false;
         }
-        return false;
-    }
-    if (m.type == GSP_MIRROR) {
+        if (lead) {
+            if (D.smat) D.smat[slot] = mid;
+            float4* p = D.slots + 2 * (size_t)slot;
+            p[0] = make_float4(x.x, x.y, x.z, __uint_as_float(rec));
+            p[1] = make_float4(w.x, w.y, w.z, __uint_as_float(oct_encode(d)));
+        }
+        ++ndep;
+        if (D.stochastic) {
+            const float z = rng_next(rng);
+            if (lead) {
+                const uint32_t b = bucket_of(x, P.inv_h, P.tmask);
+                const unsigned long long key = ((unsigned long long)__float_as_uint(z) << 32) | slot;
+                atomicMin(D.entry + b, key);
+                atomicAdd(D.ecount + b, 1u);
+            }
+        }
+        float urr = 0.0f, ua = 0.0f, ub = 0.0f;
+#pragma unroll 1
+        for (int k = 0; k < 3; ++k) {
+            urr = ua;
+            ua = ub;
+            ub = rng_next(rng);
+        }
+        if (!(urr < P.rr)) return false;
+        w = mul3(mul3(w, m.albedo), sf.tex) * (1.0f / P.rr);
+        const float3 ns = front ? sf.ns : sf.ns * -1.0f;
+        d = cosine_dir(ns, ua, ub);
+        // about a shading normal the direction can point into the surface: the path ends there
+        if (sf.smooth && !(dot3(d, front ? n : n * -1.0f) > 0.0f)) return false;
+    } else if (m.type == GSP_MIRROR) {
         w = mul3(w, m.albedo);
         d = reflect3(d, sf.ns);
     } else {
@@ -502,7 +542,8 @@ k_eye_shade(DevScene S, PassDev P, PathQ cur, PathQ nxt, EyeOut O, uint32_t* __r
             h.slot = -1;
             if (h.id >= 0 && !P.tri_is_id) h.id = slot_refine(S, o, d, h);
             if (h.id >= 0) {
-                keep = eye_interact<SHADE>(S, P, O, p, h, o, d, w, rng) && depth + 1 <= P.max_eye;
+                uint32_t none = 0;
+                keep = path_interact<SHADE>(S, P, O, DepositDev{}, true, p, h, o, d, w, rng, 0, 0, none) && depth + 1 <= P.max_eye;
             }
         }
         queue_push(nxt, qn + (b + 1) % 3, keep, o, P.eps, d, w, p, rng, depth + 1);
@@ -537,62 +578,6 @@ __device__ __forceinline__ void emit_photon(const EmitDev& E, Rng& rng, float3& 
     o = make_float3(coord(v0.x, e1.x, e2.x), coord(v0.y, e1.y, e2.y), coord(v0.z, e1.z, e2.z));
     const float u3 = rng_next(rng), u4 = rng_next(rng);
     d = cosine_dir(n, u3, u4);
-}
-
-struct DepositDev {
-    float4* __restrict__ slots;          // 2 float4 per slot
-    uint32_t* __restrict__ pcount;       // deposits per path / thread
-    unsigned long long* __restrict__ entry;  // stochastic: min key per bucket
-    uint32_t* __restrict__ ecount;       // stochastic: photons per bucket
-    int32_t stochastic;
-    int32_t* __restrict__ smat;          // optional: material of each deposit's surface (gradient replay)
-};
-
-// One photon interaction at a hit. Returns false when the path ends. lead as in eye_interact.
-template <bool SHADE>
-__device__ __forceinline__ bool photon_bounce(const DevScene& S, const PassDev& P, const DepositDev& D,
-                                              Rng& rng, const Hit& h, float3& o, float3& d, float3& phi,
-                                              uint32_t id, uint32_t slot, uint32_t& ndep, bool lead = true) {
-    const float4 sh = __ldg(S.shade + h.id);
-    const float3 n = f3(sh);
-    const Material m = load_mat(S, __float_as_int(sh.w));
-    if (m.type == GSP_EMITTER) return false;
-    const float3 x = madd3(d, h.t, o);
-    const Surf sf = surface<SHADE>(S, h, o, d, n, m, __float_as_int(sh.w));
-    if (m.type == GSP_DIFFUSE) {
-        if (lead) {
-            if (D.smat) D.smat[slot] = __float_as_int(sh.w);
-            float4* rec = D.slots + 2 * (size_t)slot;
-            rec[0] = make_float4(x.x, x.y, x.z, __uint_as_float(id));
-            rec[1] = make_float4(phi.x, phi.y, phi.z, __uint_as_float(oct_encode(d)));
-        }
-        ++ndep;
-        if (D.stochastic) {
-            const float z = rng_next(rng);
-            if (lead) {
-                const uint32_t b = bucket_of(x, P.inv_h, P.tmask);
-                const unsigned long long key = ((unsigned long long)__float_as_uint(z) << 32) | slot;
-                atomicMin(D.entry + b, key);
-                atomicAdd(D.ecount + b, 1u);
-            }
-        }
-        const float urr = rng_next(rng);
-        if (!(urr < P.rr)) return false;
-        phi = mul3(mul3(phi, m.albedo), sf.tex) * (1.0f / P.rr);
-        const bool fr = dot3(d, n) < 0.0f;
-        const float3 ns = fr ? sf.ns : sf.ns * -1.0f;
-        const float ua = rng_next(rng), ub = rng_next(rng);
-        d = cosine_dir(ns, ua, ub);
-        // about a shading normal the direction can point into the surface: the path ends there
-        if (sf.smooth && !(dot3(d, fr ? n : n * -1.0f) > 0.0f)) return false;
-    } else if (m.type == GSP_MIRROR) {
-        phi = mul3(phi, m.albedo);
-        d = reflect3(d, sf.ns);
-    } else {
-        d = dielectric(d, sf.ns, m.ior, rng_next(rng));
-    }
-    o = x;
-    return true;
 }
 
 // Photon paths: emission into the queue in path order (whole paths per pass).
@@ -656,7 +641,7 @@ k_photon_shade(DevScene S, PassDev P, DepositDev D, PathQ cur, PathQ nxt, uint32
                 const uint32_t id = (uint32_t)k * kSlotsPerPath + depth;
                 const uint32_t slot = (uint32_t)k * kSlotsPerPath + ndep;
                 const uint32_t before = ndep;
-                keep = photon_bounce<SHADE>(S, P, D, rng, h, o, d, phi, id, slot, ndep) && depth + 1 < P.max_photon;
+                keep = path_interact<SHADE>(S, P, EyeOut{}, D, false, k, h, o, d, phi, rng, id, slot, ndep) && depth + 1 < P.max_photon;
                 if (ndep != before) D.pcount[k] = ndep;
             }
         }
@@ -679,7 +664,6 @@ template <int WALK, bool SHADE, bool COUNT>
 __global__ void __launch_bounds__(kTraceThreads, SHADE ? GSP_PATH_SHADE_MIN_BLOCKS : GSP_PATH_MIN_BLOCKS)
 k_paths(DevScene S, PassDev P, PathQ qe, EyeOut O, const uint32_t* __restrict__ ne_ptr, PathQ qp, DepositDev D,
         const uint32_t* __restrict__ np_ptr, uint32_t* __restrict__ ctr, int32_t chunk) {
-    __shared__ CoopScratch scratch[WALK == kWide ? kTraceThreads / 32 : 1];
     const int32_t cap = trav_cap(S);
     const int32_t ne = ne_ptr ? (int32_t)*ne_ptr : 0;
     const int32_t nph = np_ptr ? (int32_t)*np_ptr : 0;
@@ -692,9 +676,8 @@ k_paths(DevScene S, PassDev P, PathQ qe, EyeOut O, const uint32_t* __restrict__ 
     float3 w = make_float3(0.0f, 0.0f, 0.0f);  // eye: throughput; photon: flux
     Rng rng;
     uint32_t c_eye = 0, c_ph = 0, c_nodes = 0, c_tris = 0;  // work of this lane
-    bool quad = false;  // the last paths, four lanes to a path
     while (true) {
-        const int32_t got = quad ? -1 : wq.take(i < 0, ctr);
+        const int32_t got = wq.take(i < 0, ctr);
         if (got >= 0) {
             i = got;
             eye = got < ne;
@@ -709,7 +692,7 @@ k_paths(DevScene S, PassDev P, PathQ qe, EyeOut O, const uint32_t* __restrict__ 
             ndep = eye ? 0u : (uint32_t)(meta >> 8);
             pw.start(S, f3(a), f3(c), eye ? a.w : P.eps);
         }
-        uint32_t act = __ballot_sync(0xffffffffu, i >= 0);
+        const uint32_t act = __ballot_sync(0xffffffffu, i >= 0);
         if (act == 0) break;
         bool walked = false;
         if constexpr (WALK == kLinks) {  // nothing left to take: a path left alone in the warp walks with all lanes
@@ -718,49 +701,25 @@ k_paths(DevScene S, PassDev P, PathQ qe, EyeOut O, const uint32_t* __restrict__ 
                 walked = true;
             }
         }
-        if constexpr (WALK == kWide) {
-            if (!quad && wq.done && __popc(act) <= kQuadRays && __popc(act) > 1) {
-                quad = true;
-                const int own = threadIdx.x & 31, from = quad_source(act), src = from < 0 ? own : from;
-                quad_take(pw.st, pw.w, pw.stk, src);
-                i = from < 0 ? -1 : 0;
-                id = __shfl_sync(0xffffffffu, id, src);
-                depth = __shfl_sync(0xffffffffu, depth, src);
-                ndep = __shfl_sync(0xffffffffu, ndep, src);
-                eye = __shfl_sync(0xffffffffu, (int)eye, src) != 0;
-                w = shfl3(w, src);
-                rng = shfl_rng(rng, src);
-                act = __ballot_sync(0xffffffffu, i >= 0);
-            }
-            if (wq.done && __popc(act) == (quad ? 4 : 1)) {
-                pw.finish(S, __ffs(act) - 1, &scratch[threadIdx.x >> 5]);
-                walked = true;
-            } else if (quad) {
-                pw.quad_steps(S, i >= 0);
-                walked = true;
-            }
-        }
-        const bool lead = !quad || (threadIdx.x & 3) == 0;
         if (!walked) pw.steps(S, i >= 0, cap, c_tris);
         if (i >= 0 && pw.done()) {
             const Hit h = walk_hit(S, pw.st);
             float3 o = pw.st.o, d = pw.st.d;
             bool more = false;
             if (COUNT) {
-                if constexpr (WALK != kWide) c_nodes += (uint32_t)pw.st.steps;
+                c_nodes += (uint32_t)pw.st.steps;
                 c_eye += eye ? 1u : 0u;
                 c_ph += eye ? 0u : 1u;
             }
-            if (eye) {
-                more = h.id >= 0 && eye_interact<SHADE>(S, P, O, id, h, o, d, w, rng, lead) && ++depth <= P.max_eye;
-            } else {
-                if (h.id >= 0) {
-                    const uint32_t pid = (uint32_t)id * kSlotsPerPath + depth;
-                    const uint32_t slot = (uint32_t)id * kSlotsPerPath + ndep;
-                    more = photon_bounce<SHADE>(S, P, D, rng, h, o, d, w, pid, slot, ndep, lead) && ++depth < P.max_photon;
+            if (h.id >= 0) {
+                const uint32_t base = (uint32_t)id * kSlotsPerPath;
+                more = path_interact<SHADE>(S, P, O, D, eye, id, h, o, d, w, rng, base + depth, base + ndep, ndep);
+                if (more) {
+                    ++depth;
+                    more = eye ? depth <= P.max_eye : depth < P.max_photon;
                 }
-                if (!more && lead) D.pcount[id] = ndep;
             }
+            if (!more && !eye) D.pcount[id] = ndep;
             if (more)
                 pw.start(S, o, d, P.eps);
             else
@@ -778,6 +737,14 @@ k_paths(DevScene S, PassDev P, PathQ qe, EyeOut O, const uint32_t* __restrict__ 
 // ------------------------------------------------------------------------------------------
 // the eye and photon paths of many renderers in one persistent launch (batched passes)
 // ------------------------------------------------------------------------------------------
+// One bounce per pass (Sec. 3.3): the stored path of each thread, and the paths started.
+struct RegenDev {
+    float4* __restrict__ ro;    // {o.xyz, depth bits}
+    float4* __restrict__ rd;    // {d.xyz, alive bits}
+    float4* __restrict__ rphi;  // {flux.rgb, 0}
+    unsigned long long* __restrict__ started;
+};
+
 // One renderer's share of a fused launch: its scene, pass, queues and outputs, where its item
 // counts live on the device, and its range of 64-item chunks in the launch's chunk sequence
 // (sized by capacity; chunks past the pass's actual counts are skipped).
@@ -790,6 +757,9 @@ struct PathJob {
     const uint32_t* ne_ptr;  // null: no eye items
     const uint32_t* np_ptr;  // null: no photon items
     int32_t first_chunk, nchunks;
+    int32_t nregen;  // k_paths_pool<.., REGEN>: threads of the one-bounce photon pass, which follow the eye items
+    EmitDev E;
+    RegenDev R;
 };
 
 // Work distribution over the chunks of all jobs: as WarpQueue, but a chunk also names its job
@@ -870,9 +840,8 @@ k_paths_multi(const PathJob* __restrict__ jobs, int32_t njobs, int32_t total_chu
     bool eye = false;
     float3 w = make_float3(0.0f, 0.0f, 0.0f);  // eye: throughput; photon: flux
     Rng rng;
-    bool quad = false;  // the last paths, four lanes to a path
     while (true) {
-        const int32_t got = quad ? -1 : mq.take(i < 0, jobs, njobs, ctr, jb);
+        const int32_t got = mq.take(i < 0, jobs, njobs, ctr, jb);
         if (got >= 0) {
             const PathJob& J = jobs[jb];
             const int32_t ne = J.ne_ptr ? (int32_t)*J.ne_ptr : 0;
@@ -890,44 +859,23 @@ k_paths_multi(const PathJob* __restrict__ jobs, int32_t njobs, int32_t total_chu
             cap = trav_cap(J.S);
             pw.start(J.S, f3(a), f3(c), eye ? a.w : J.P.eps);
         }
-        const uint32_t act = __ballot_sync(0xffffffffu, i >= 0);
-        if (act == 0) break;
-        if constexpr (WALK == kWide) {
-            if (!quad && mq.done && __popc(act) <= kQuadRays) {
-                quad = true;
-                const int own = threadIdx.x & 31, from = quad_source(act), src = from < 0 ? own : from;
-                quad_take(pw.st, pw.w, pw.stk, src);
-                i = from < 0 ? -1 : 0;
-                jb = __shfl_sync(0xffffffffu, jb, src);
-                id = __shfl_sync(0xffffffffu, id, src);
-                depth = __shfl_sync(0xffffffffu, depth, src);
-                ndep = __shfl_sync(0xffffffffu, ndep, src);
-                eye = __shfl_sync(0xffffffffu, (int)eye, src) != 0;
-                w = shfl3(w, src);
-                rng = shfl_rng(rng, src);
-            }
-        }
+        if (__ballot_sync(0xffffffffu, i >= 0) == 0) break;
         const PathJob& J = jobs[jb];
         uint32_t ntri = 0;  // work is not counted in batched passes
-        const bool lead = !quad || (threadIdx.x & 3) == 0;
-        if constexpr (WALK == kWide) {
-            if (quad) pw.quad_steps(J.S, i >= 0);
-        }
-        if (!quad) pw.steps(J.S, i >= 0, cap, ntri);
+        pw.steps(J.S, i >= 0, cap, ntri);
         if (i >= 0 && pw.done()) {
             const Hit h = walk_hit(J.S, pw.st);
             float3 o = pw.st.o, d = pw.st.d;
             bool more = false;
-            if (eye) {
-                more = h.id >= 0 && eye_interact<SHADE>(J.S, J.P, J.O, id, h, o, d, w, rng, lead) && ++depth <= J.P.max_eye;
-            } else {
-                if (h.id >= 0) {
-                    const uint32_t pid = (uint32_t)id * kSlotsPerPath + depth;
-                    const uint32_t slot = (uint32_t)id * kSlotsPerPath + ndep;
-                    more = photon_bounce<SHADE>(J.S, J.P, J.D, rng, h, o, d, w, pid, slot, ndep, lead) && ++depth < J.P.max_photon;
+            if (h.id >= 0) {
+                const uint32_t base = (uint32_t)id * kSlotsPerPath;
+                more = path_interact<SHADE>(J.S, J.P, J.O, J.D, eye, id, h, o, d, w, rng, base + depth, base + ndep, ndep);
+                if (more) {
+                    ++depth;
+                    more = eye ? depth <= J.P.max_eye : depth < J.P.max_photon;
                 }
-                if (!more && lead) J.D.pcount[id] = ndep;
             }
+            if (!more && !eye) J.D.pcount[id] = ndep;
             if (more)
                 pw.start(J.S, o, d, J.P.eps);
             else
@@ -935,13 +883,6 @@ k_paths_multi(const PathJob* __restrict__ jobs, int32_t njobs, int32_t total_chu
         }
     }
 }
-
-struct RegenDev {
-    float4* __restrict__ ro;    // {o.xyz, depth bits}
-    float4* __restrict__ rd;    // {d.xyz, alive bits}
-    float4* __restrict__ rphi;  // {flux.rgb, 0}
-    unsigned long long* __restrict__ started;
-};
 
 // One bounce per thread and pass (Sec. 3.3): thread j continues its stored path, or starts a new
 // one when the stored path has ended (N_e counts the starts), traces exactly one ray, deposits at
@@ -1002,7 +943,7 @@ k_photon_regen(DevScene S, EmitDev E, PassDev P, DepositDev D, RegenDev R, uint3
             const Hit h = walk_hit(S, pw.st);
             float3 o = pw.st.o, d = pw.st.d;
             uint32_t ndep = 0;
-            bool alive = h.id >= 0 && photon_bounce<SHADE>(S, P, D, rng, h, o, d, phi, (uint32_t)j, (uint32_t)j, ndep, lead) &&
+            bool alive = h.id >= 0 && path_interact<SHADE>(S, P, EyeOut{}, D, false, j, h, o, d, phi, rng, (uint32_t)j, (uint32_t)j, ndep, lead) &&
                          ++depth < P.max_photon;
             if (lead) {
                 D.pcount[j] = ndep;

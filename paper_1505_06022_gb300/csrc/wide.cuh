@@ -144,15 +144,14 @@ __device__ __forceinline__ void wide_node(const float4* __restrict__ nodes, cons
     wide_next(k0, k1, k2, k3, ref, st, w, stk);
 }
 
-// Walks the warp's active lanes until no more than KEEP quarters of them still walk: what follows a
+// Walks the warp's active lanes until no more than `keep` quarters of them still walk: what follows a
 // walk then runs for many lanes at once. A path kernel's shading is long (1 of 4; 8.0 ms per eight
 // 512x512 passes, against 8.07 with 2 and 8.33 with 3), a ray's end in the closest-hit kernel short
 // (2; 3 costs 1 %, 1 costs 8 %). Lanes at a leaf wait until kWideLeafBatch of them are, or no lane
 // has a node left to test, and test their leaves together (12; 8 costs 1-2 %, 4 costs 5 %).
-template <int KEEP>
 __device__ __forceinline__ void wide_steps(const float4* __restrict__ wide, const float4* __restrict__ tris, WideRay& st,
-                                           WideWalk& w, int2* stk, bool active) {
-    const int stop = (__popc(__ballot_sync(0xffffffffu, active)) * KEEP) >> 2;
+                                           WideWalk& w, int2* stk, bool active, int keep) {
+    const int stop = (__popc(__ballot_sync(0xffffffffu, active)) * keep) >> 2;
     uint32_t nm, lm;
     do {
         if (active && w.cur >= 0) wide_node(wide, st, w, stk);

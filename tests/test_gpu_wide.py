@@ -47,7 +47,8 @@ def test_closest_hits(ctx, ntris, builder):
 
 @pytest.mark.parametrize("photon_mode", [gsp.FULL_PATH, gsp.REGEN])
 @pytest.mark.parametrize("make,w,h,photons", [(I.cornell_box, 37, 21, 700), (I.full_scene, 96, 64, 20_000),
-                                              (I.shaded_scene, 64, 48, 9_000)])
+                                              (I.shaded_scene, 64, 48, 9_000),
+                                              (I.full_scene, 300, 201, 400_000)])  # pools refilled from the queue
 def test_renders(ctx, make, w, h, photons, photon_mode):
     sc = make(width=w, height=h) if make is I.cornell_box else make(width=w, height=h, plane_quads=32, sphere_n=9)
     s = gsp.Scene(ctx, sc)
