@@ -29,6 +29,15 @@ gsp_status gsp_pending_error(const char* who, cudaError_t e) {
     return GSP_ERR_CUDA;
 }
 
+// Calls of up to this many rays per warp re-evaluate flagged hits inside the wide kernel: that saves
+// k_refine's launch and, up to 32 rays per warp, k_zero_u64x2's (1,021 rays 23.0 -> 18.1 us, 262,147 rays
+// 76.2 -> 69.1 us, 300k 116.5 -> 110.9 us). The re-evaluation in the loop costs the walk 6 % (spilled
+// registers, warps that wait for FP64), so long calls list their hits: 600k rays are level
+// (130.2 / 130.5 us), 1M 167 listed / 172 us, 4M 642 / 685 us.
+#ifndef GSP_REFINE_INLINE
+#define GSP_REFINE_INLINE 128
+#endif
+
 namespace gspd {
 
 // Closest-hit kernel (Fig. 3), persistent. A warp takes chunks of kTraceChunk consecutive rays
@@ -143,8 +152,30 @@ k_trace_stack(DevScene S, const float4* __restrict__ rays, int64_t n, int32_t* _
     }
 }
 
+// FP64 re-evaluation of listed hit e = (ray, slot).
+__device__ __forceinline__ void refine_listed(const DevScene& S, const float4* __restrict__ rays, int2 e,
+                                              float* __restrict__ tout, float2* __restrict__ uv) {
+    const float4 a = __ldg(rays + 2 * (int64_t)e.x), b = __ldg(rays + 2 * (int64_t)e.x + 1);
+    Hit h;
+    if (refine_hit(S.tris + 3 * (int64_t)e.y, f3(a), f3(b), h)) {
+        tout[e.x] = h.t;
+        if (uv) uv[e.x] = make_float2(h.u, h.v);
+    }
+}
+
+// The hits that k_trace listed (their rays are rare; full warps keep the FP64 pipe busy).
+__global__ void __launch_bounds__(256)
+k_refine(DevScene S, const float4* __restrict__ rays, const int2* __restrict__ rlist,
+         const unsigned long long* __restrict__ count, float* __restrict__ tout, float2* __restrict__ uv) {
+    const int64_t cnt = (int64_t)*count;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < cnt; i += (int64_t)gridDim.x * blockDim.x)
+        refine_listed(S, rays, rlist[i], tout, uv);
+}
+
 // Closest hit through the four-wide form of the tree (wide.cuh): the kernel of scenes that have
-// one, with k_trace's work distribution, outputs and list of hits for FP64 re-evaluation.
+// one, with k_trace's work distribution and outputs. LIST: hits for FP64 re-evaluation go to k_trace's
+// list; otherwise a warp collects its own and re-evaluates them 32 at a time.
+template <bool LIST>
 __global__ void __launch_bounds__(kTraceThreads, GSP_WIDE_MIN_BLOCKS)
 k_trace_wide(DevScene S, const float4* __restrict__ rays, int64_t n, const uint32_t* __restrict__ d_n,
              int32_t* __restrict__ tri, float* __restrict__ tout, float2* __restrict__ uv,
@@ -154,6 +185,9 @@ k_trace_wide(DevScene S, const float4* __restrict__ rays, int64_t n, const uint3
     const int lane = threadIdx.x & 31;
     const uint32_t lt = lanemask_lt();
     __shared__ CoopScratch scratch[kTraceThreads / 32];
+    __shared__ int2 lists[LIST ? 1 : kTraceThreads / 32][64];
+    int2* const list = lists[LIST ? 0 : threadIdx.x >> 5];
+    int32_t nlist = 0;  // warp-uniform, below 32 at the loop's head
     WarpQueue wq;
     wq.init((int32_t)n, chunk);
     WideRay st;
@@ -199,33 +233,26 @@ k_trace_wide(DevScene S, const float4* __restrict__ rays, int64_t n, const uint3
         }
         const uint32_t fm = __ballot_sync(0xffffffffu, flag);
         if (fm) {
-            const int leader = __ffs(fm) - 1;
-            unsigned long long b = 0;
-            if (lane == leader) b = atomicAdd(ctr + 1, (unsigned long long)__popc(fm));
-            b = __shfl_sync(0xffffffffu, b, leader);
-            if (flag) rlist[b + __popc(fm & lt)] = make_int2((int)ray, st.slot);
+            if (LIST) {
+                const int leader = __ffs(fm) - 1;
+                unsigned long long b = 0;
+                if (lane == leader) b = atomicAdd(ctr + 1, (unsigned long long)__popc(fm));
+                b = __shfl_sync(0xffffffffu, b, leader);
+                if (flag) rlist[b + __popc(fm & lt)] = make_int2(ray, st.slot);
+            } else {
+                if (flag) list[nlist + __popc(fm & lt)] = make_int2(ray, st.slot);
+                nlist += __popc(fm);
+                __syncwarp();
+                if (nlist >= 32) {
+                    nlist -= 32;
+                    refine_listed(S, rays, list[nlist + lane], tout, uv);
+                    __syncwarp();
+                }
+            }
         }
         if (fin) ray = -1;
     }
-}
-
-// FP64 re-evaluation of the listed hits (their rays are rare; full warps keep the FP64 pipe busy).
-__global__ void __launch_bounds__(256)
-k_refine(DevScene S, const float4* __restrict__ rays, const int2* __restrict__ rlist,
-         const unsigned long long* __restrict__ ctr, float* __restrict__ tout, float2* __restrict__ uv) {
-    const int64_t cnt = (int64_t)ctr[1];
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < cnt; i += (int64_t)gridDim.x * blockDim.x) {
-        const int2 e = rlist[i];
-        const float4 a = __ldg(rays + 2 * (int64_t)e.x), b = __ldg(rays + 2 * (int64_t)e.x + 1);
-        Hit h;
-        h.t = tout[e.x];
-        h.u = h.v = 0.0f;
-        h.id = 0;
-        if (refine_hit(S.tris + 3 * (int64_t)e.y, f3(a), f3(b), h)) {
-            tout[e.x] = h.t;
-            if (uv) uv[e.x] = make_float2(h.u, h.v);
-        }
-    }
+    if (!LIST && lane < nlist) refine_listed(S, rays, list[lane], tout, uv);
 }
 
 __global__ void k_zero_u64x2(unsigned long long* p) {
@@ -263,52 +290,53 @@ static int trace_wide_grid(int device) {
     if (device >= 0 && device < 64 && cached[device]) return cached[device];
     int sms = 0, per_sm = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, gspd::k_trace_wide, kTraceThreads, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, gspd::k_trace_wide<true>, kTraceThreads, 0);
     int g = std::max(1, sms) * std::max(1, per_sm);
     if (device >= 0 && device < 64) cached[device] = g;
     return g;
 }
 
-// The closest-hit kernel that S is walked with.
+// Closest hit of n rays (of the first *d_n, if given) as S is walked. `zero`: the counters are zeroed if
+// a kernel uses them; the wide kernel without a list uses none when each warp's first chunk covers n.
 static void run_trace(const gspd::DevScene& S, int device, const float4* rays, int64_t n, const uint32_t* d_n,
                       int32_t* tri, float* t, float2* uv, unsigned long long* ctr, int2* rlist, float refine_factor,
-                      int32_t out_slot, cudaStream_t st) {
+                      int32_t out_slot, bool zero, cudaStream_t st, cudaEvent_t e0 = nullptr, cudaEvent_t e1 = nullptr) {
+    const int links_grid = gsp_trace_grid(device);
+    constexpr int kWarps = kTraceThreads / 32;
+    const int64_t wide_grid = std::min<int64_t>(trace_wide_grid(device), (n + kWarps - 1) / kWarps);
+    const int chunk = gsp_chunk(n, wide_grid * kWarps, kTraceChunk);
+    const bool list = refine_factor < INFINITY && !(S.wide && n <= GSP_REFINE_INLINE * wide_grid * kWarps);
+    if (zero && (list || !S.wide || chunk * wide_grid * kWarps < n)) gspd::k_zero_u64x2<<<1, 1, 0, st>>>(ctr);
+    if (e0) cudaEventRecord(e0, st);
     if (S.wide) {
-        constexpr int kWarps = kTraceThreads / 32;
-        const int64_t grid = std::min<int64_t>(trace_wide_grid(device), (n + kWarps - 1) / kWarps);
-        gspd::k_trace_wide<<<(unsigned)grid, kTraceThreads, 0, st>>>(S, rays, n, d_n, tri, t, uv, ctr, rlist, refine_factor,
-                                                                     out_slot, gsp_chunk(n, grid * kWarps, kTraceChunk));
+        auto* const kernel = list ? gspd::k_trace_wide<true> : gspd::k_trace_wide<false>;
+        kernel<<<(unsigned)wide_grid, kTraceThreads, 0, st>>>(S, rays, n, d_n, tri, t, uv, ctr, rlist, refine_factor,
+                                                              out_slot, chunk);
     } else
-        gspd::k_trace<<<gsp_trace_grid(device), kTraceThreads, 0, st>>>(S, rays, n, d_n, tri, t, uv, ctr, rlist,
-                                                                        refine_factor, out_slot);
+        gspd::k_trace<<<links_grid, kTraceThreads, 0, st>>>(S, rays, n, d_n, tri, t, uv, ctr, rlist, refine_factor,
+                                                            out_slot);
+    if (e1) cudaEventRecord(e1, st);
+    if (list)
+        gspd::k_refine<<<(unsigned)std::min<int64_t>(std::max(1, links_grid / 2), (n + 255) / 256), 256, 0, st>>>(
+            S, rays, rlist, ctr + 1, t, uv);
 }
 
-// One closest-hit call on device buffers: counters zeroed, k_trace, FP64 refinement of the
-// flagged hits. ctr (2 u64) and rlist (n entries) belong to this call's stream.
-// With e0 and e1 (gsp_trace_time_launches), the two events bracket the k_trace launch alone.
+// One closest-hit call on device buffers: the traversal and the FP64 refinement of the flagged hits.
+// ctr (2 u64) and rlist (n entries) belong to this call's stream.
+// With e0 and e1 (gsp_trace_time_launches), the two events bracket the traversal launch alone.
 static void launch_trace(const gsp_scene* s, const float4* rays, int64_t n, int32_t* tri, float* t, float2* uv,
                          unsigned long long* ctr, int2* rlist, cudaStream_t st, cudaEvent_t e0 = nullptr,
                          cudaEvent_t e1 = nullptr) {
     NvtxRange nvtx("gsp: closest hit");
-    const gspd::DevScene S = gsp_dev_scene(s);
-    gspd::k_zero_u64x2<<<1, 1, 0, st>>>(ctr);
-    const int grid = gsp_trace_grid(s->ctx->device);
-    if (e0) cudaEventRecord(e0, st);
-    run_trace(S, s->ctx->device, rays, n, nullptr, tri, t, uv, ctr, rlist, GSP_REFINE_FACTOR, 0, st);
-    if (e1) cudaEventRecord(e1, st);
-    gspd::k_refine<<<(unsigned)std::min<int64_t>(std::max(1, grid / 2), (n + 255) / 256), 256, 0, st>>>(S, rays, rlist, ctr,
-                                                                                                    t, uv);
+    run_trace(gsp_dev_scene(s), s->ctx->device, rays, n, nullptr, tri, t, uv, ctr, rlist, GSP_REFINE_FACTOR, 0, true, st,
+              e0, e1);
 }
 
 cudaError_t gsp_trace_queue(const gsp_scene* s, const float4* rays, int64_t max_n, const uint32_t* d_n, int32_t* tri,
                             float* t, float refine_factor, bool zero_counters, bool out_slot, unsigned long long* ctr,
                             int2* rlist, cudaStream_t st) {
-    const gspd::DevScene S = gsp_dev_scene(s);
-    const int grid = gsp_trace_grid(s->ctx->device);
-    const bool list = refine_factor < INFINITY;
-    if (list || zero_counters) gspd::k_zero_u64x2<<<1, 1, 0, st>>>(ctr);
-    run_trace(S, s->ctx->device, rays, max_n, d_n, tri, t, nullptr, ctr, rlist, refine_factor, out_slot ? 1 : 0, st);
-    if (list) gspd::k_refine<<<std::max(1, grid / 2), 256, 0, st>>>(S, rays, rlist, ctr, t, nullptr);
+    run_trace(gsp_dev_scene(s), s->ctx->device, rays, max_n, d_n, tri, t, nullptr, ctr, rlist, refine_factor,
+              out_slot ? 1 : 0, refine_factor < INFINITY || zero_counters, st);
     return cudaGetLastError();
 }
 
@@ -927,7 +955,7 @@ gsp_status gsp_trace_closest_hit_stack(gsp_scene* s, const float* d_rays, int64_
     const int grid = gsp_trace_grid(s->ctx->device);
     gspd::k_trace_stack<<<grid, kTraceThreads, 0, st>>>(S, (const float4*)d_rays, n, d_tri, d_t, (float2*)d_uv,
                                                         s->d_counter, s->d_rlist, GSP_REFINE_FACTOR);
-    gspd::k_refine<<<std::max(1, grid / 2), 256, 0, st>>>(S, (const float4*)d_rays, s->d_rlist, s->d_counter, d_t,
+    gspd::k_refine<<<std::max(1, grid / 2), 256, 0, st>>>(S, (const float4*)d_rays, s->d_rlist, s->d_counter + 1, d_t,
                                                           (float2*)d_uv);
     GSP_CUDA_TRY(cudaGetLastError());
     return GSP_OK;

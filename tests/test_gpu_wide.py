@@ -45,6 +45,23 @@ def test_closest_hits(ctx, ntris, builder):
     ctx.sync()
 
 
+@pytest.mark.parametrize("per_warp", [32, 128])
+@pytest.mark.parametrize("extra", [0, 1])
+def test_long_calls_equal_their_parts(ctx, per_warp, extra):
+    """The line between static and dynamic chunks (32 rays per warp) and the line between hits
+    re-evaluated in the kernel and through a list (128) do not show in the results."""
+    n = torch.cuda.get_device_properties(0).multi_processor_count * 32 * per_warp + extra
+    sc = I.random_soup(3000, seed=2, size=0.1)
+    s = gsp.Scene(ctx, sc)
+    rays = torch.from_numpy(I.random_rays(n, seed=6)).cuda()
+    whole = s.trace(rays, with_uv=True)
+    part = 4000
+    for k in range(0, n, part):
+        for a, b in zip(whole, s.trace(rays[k:k + part].clone(), with_uv=True)):
+            assert torch.equal(a[k:k + part].view(torch.int32), b.view(torch.int32)), k
+    ctx.sync()
+
+
 @pytest.mark.parametrize("photon_mode", [gsp.FULL_PATH, gsp.REGEN])
 @pytest.mark.parametrize("make,w,h,photons", [(I.cornell_box, 37, 21, 700), (I.full_scene, 96, 64, 20_000),
                                               (I.shaded_scene, 64, 48, 9_000),
