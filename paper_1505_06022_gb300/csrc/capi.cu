@@ -193,7 +193,9 @@ k_trace_wide(DevScene S, const float4* __restrict__ rays, int64_t n, const uint3
     WideRay st;
     st.slot = -1;
     WideWalk w;
-    int2 stk[kWideStack];
+    __shared__ int2 tops[kTraceThreads / 32][GSP_WIDE_TOP_TRACE * 32];
+    int2 deep[kWideStack - GSP_WIDE_TOP_TRACE];
+    const WideStack<GSP_WIDE_TOP_TRACE> stk{deep, tops[threadIdx.x >> 5] + lane};
     w.cur = kWalkDone;
     w.sp = 0;
     int32_t ray = -1;

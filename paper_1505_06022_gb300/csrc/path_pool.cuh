@@ -153,7 +153,8 @@ k_paths_pool(const __grid_constant__ PathJob one, const PathJob* __restrict__ jo
     int nready = 0, ndone = pool;
     WideRay st;
     WideWalk w;
-    int2 stk[kWideStack];
+    int2 deep[kWideStack];
+    const WideStack<0> stk{deep, nullptr};
     uint32_t starts = 0;  // REGEN: paths started by this lane
     int at = -1;          // the slot whose ray this lane walks
     const float4 *wide = one.S.wide, *tris = one.S.tris;  // and the tree it walks (MULTI: its job's)

@@ -322,10 +322,10 @@ struct PathWalk<kWide> {
         wide_init(w);
     }
     __device__ __forceinline__ void steps(const DevScene& S, bool active, int32_t, uint32_t&) {
-        wide_steps(S.wide, S.tris, st, w, stk, active, GSP_WIDE_KEEP);
+        wide_steps(S.wide, S.tris, st, w, WideStack<0>{stk, nullptr}, active, GSP_WIDE_KEEP);
     }
     __device__ __forceinline__ void quad_steps(const DevScene& S, bool active) {
-        gspd::quad_steps<GSP_WIDE_KEEP>(S.wide, S.tris, st, w, stk, active);
+        gspd::quad_steps<GSP_WIDE_KEEP>(S.wide, S.tris, st, w, WideStack<0>{stk, nullptr}, active);
     }
     __device__ __forceinline__ bool done() const { return w.cur == kWalkDone; }
 };
@@ -924,7 +924,7 @@ k_photon_regen(DevScene S, EmitDev E, PassDev P, DepositDev D, RegenDev R, uint3
             if (!quad && wq.done && __popc(act) <= kQuadRays) {
                 quad = true;
                 const int own = threadIdx.x & 31, from = quad_source(act), src = from < 0 ? own : from;
-                quad_take(pw.st, pw.w, pw.stk, src);
+                quad_take(pw.st, pw.w, WideStack<0>{pw.stk, nullptr}, src);
                 j = __shfl_sync(0xffffffffu, j, src);
                 if (from < 0) j = -1;
                 depth = __shfl_sync(0xffffffffu, depth, src);

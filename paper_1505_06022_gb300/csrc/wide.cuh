@@ -28,6 +28,9 @@
 #ifndef GSP_WIDE_KEEP_TRACE
 #define GSP_WIDE_KEEP_TRACE 2
 #endif
+#ifndef GSP_WIDE_TOP_TRACE
+#define GSP_WIDE_TOP_TRACE 12
+#endif
 #ifndef GSP_WIDE_LEAF_BATCH
 #define GSP_WIDE_LEAF_BATCH 12
 #endif
@@ -70,9 +73,33 @@ __device__ __forceinline__ void wide_ray(float3 o, float3 d, float tmin, float t
 
 // One ray's walk: the node or leaf it is at (kWalkDone: the walk is over) and the children still
 // to visit, each with its key (entry distance; the two low bits hold the child number).
-// The stack is an array beside it, so that passing its address on does not hold these in memory.
+// The stack is beside it, so that passing its address on does not hold these in memory.
 struct WideWalk {
     int32_t cur, sp;
+};
+
+// Entries [0, K) of a lane's stack are in shared memory, an entry of the warp's lanes side by side (`top`
+// points to the lane's first), the others in the lane's local memory. The closest-hit kernel pops 1.5
+// times per node it tests, for four lanes of a warp at once; lanes at different depths make a local access
+// two L1 wavefronts a lane, beside the nodes' in a pipe that is busy 65 % of the time, but meet no bank
+// conflict in shared memory. K = 12 (the kernel's 60 KB of stacks per SM come out of the L1 cache):
+// 4,194,304 rays 643 -> 625 us, the random half alone 496 -> 474 us, 1,048,576 rays in host memory
+// 288 -> 279 us; 4 entries give 650 us, 8 628, 16 628, 20 633. The path kernels, whose path pools have
+// taken that shared memory, keep K = 0: with 4 or 8 a 512x512 pass is level and a 131x97 one 6 % slower.
+template <int K>
+struct WideStack {
+    int2 *deep, *top;
+
+    __device__ __forceinline__ int2 get(int i) const {
+        if (K > 0 && i < K) return top[32 * i];
+        return deep[i - K];
+    }
+    __device__ __forceinline__ void set(int i, int2 e) const {
+        if (K > 0 && i < K)
+            top[32 * i] = e;
+        else
+            deep[i - K] = e;
+    }
 };
 
 __device__ __forceinline__ void wide_init(WideWalk& w) {
@@ -88,9 +115,10 @@ __device__ __forceinline__ bool wide_keep(int32_t key, float tbest) {
     return key < 0 || __int_as_float(key & ~3) <= tbest;
 }
 
-__device__ __forceinline__ int32_t wide_pop(const RayHit& st, WideWalk& w, const int2* stk) {
+template <class Stack>
+__device__ __forceinline__ int32_t wide_pop(const RayHit& st, WideWalk& w, const Stack& stk) {
     while (w.sp > 0) {
-        const int2 e = stk[--w.sp];
+        const int2 e = stk.get(--w.sp);
         if (wide_keep(e.x, st.tbest)) return e.y;
     }
     return kWalkDone;
@@ -108,14 +136,16 @@ __device__ __forceinline__ int32_t wide_key(const WideRay& st, float cx, float h
     return tn <= __fmaf_rn(fminf(st.tbest, tf), kWideFar, st.pad) ? ((__float_as_int(tn) & ~3) | i) : kWideMiss;
 }
 
-__device__ __forceinline__ void wide_push(WideWalk& w, int2* stk, int32_t key, int32_t nearest, int32_t ref) {
-    if (key != kWideMiss && key != nearest) stk[w.sp++] = make_int2(key, ref);
+template <class Stack>
+__device__ __forceinline__ void wide_push(WideWalk& w, const Stack& stk, int32_t key, int32_t nearest, int32_t ref) {
+    if (key != kWideMiss && key != nearest) stk.set(w.sp++, make_int2(key, ref));
 }
 
 // Moves to the nearest of the children hit; the others go on the stack as they come (sorting them
 // too saves under 1 % of the visits and costs more).
+template <class Stack>
 __device__ __forceinline__ void wide_next(int32_t k0, int32_t k1, int32_t k2, int32_t k3, int4 ref, const RayHit& st,
-                                          WideWalk& w, int2* stk) {
+                                          WideWalk& w, const Stack& stk) {
     const int32_t k = min(min(k0, k1), min(k2, k3));
     if (k == kWideMiss) {
         w.cur = wide_pop(st, w, stk);
@@ -130,7 +160,9 @@ __device__ __forceinline__ void wide_next(int32_t k0, int32_t k1, int32_t k2, in
 }
 
 // Tests the four children of node w.cur and moves on.
-__device__ __forceinline__ void wide_node(const float4* __restrict__ nodes, const WideRay& st, WideWalk& w, int2* stk) {
+template <class Stack>
+__device__ __forceinline__ void wide_node(const float4* __restrict__ nodes, const WideRay& st, WideWalk& w,
+                                          const Stack& stk) {
     const float4* p = nodes + 8 * (int64_t)w.cur;
     float4 cx, hx, cy, hy, cz, hz;
     ldg32(p, cx, hx);
@@ -149,8 +181,9 @@ __device__ __forceinline__ void wide_node(const float4* __restrict__ nodes, cons
 // 512x512 passes, against 8.07 with 2 and 8.33 with 3), a ray's end in the closest-hit kernel short
 // (2; 3 costs 1 %, 1 costs 8 %). Lanes at a leaf wait until kWideLeafBatch of them are, or no lane
 // has a node left to test, and test their leaves together (12; 8 costs 1-2 %, 4 costs 5 %).
+template <class Stack>
 __device__ __forceinline__ void wide_steps(const float4* __restrict__ wide, const float4* __restrict__ tris, WideRay& st,
-                                           WideWalk& w, int2* stk, bool active, int keep) {
+                                           WideWalk& w, const Stack& stk, bool active, int keep) {
     const int stop = (__popc(__ballot_sync(0xffffffffu, active)) * keep) >> 2;
     uint32_t nm, lm;
     do {
@@ -190,7 +223,8 @@ __device__ __forceinline__ float3 shfl3(float3 v, int src) {
 }
 
 // Copies lane src's walk to this lane (every lane calls it; src: a lane, its own if it has no use).
-__device__ __forceinline__ void quad_take(WideRay& st, WideWalk& w, int2* stk, int src) {
+template <class Stack>
+__device__ __forceinline__ void quad_take(WideRay& st, WideWalk& w, const Stack& stk, int src) {
     const uint32_t F = 0xffffffffu;
     st.o = shfl3(st.o, src);
     st.d = shfl3(st.d, src);
@@ -205,16 +239,16 @@ __device__ __forceinline__ void quad_take(WideRay& st, WideWalk& w, int2* stk, i
     w.sp = __shfl_sync(F, old, src);
     const int most = __reduce_max_sync(F, w.sp);
     for (int e = 0; e < most; ++e) {
-        const int2 own = e < old ? stk[e] : make_int2(0, 0);
+        const int2 own = e < old ? stk.get(e) : make_int2(0, 0);
         const int2 got = make_int2(__shfl_sync(F, own.x, src), __shfl_sync(F, own.y, src));
-        if (e < w.sp) stk[e] = got;
+        if (e < w.sp) stk.set(e, got);
     }
 }
 
 // As wide_steps, for groups of four lanes; `active` is the same in the lanes of a group.
-template <int KEEP>
+template <int KEEP, class Stack>
 __device__ __forceinline__ void quad_steps(const float4* __restrict__ wide, const float4* __restrict__ tris, WideRay& st,
-                                           WideWalk& w, int2* stk, bool active) {
+                                           WideWalk& w, const Stack& stk, bool active) {
     const uint32_t F = 0xffffffffu;
     const int c = threadIdx.x & 3;
     const int stop = (__popc(__ballot_sync(F, active)) * KEEP) >> 2;
@@ -289,8 +323,9 @@ static_assert(kCoopNarrow + 24 + 3 * (kWideMaxDepth / 2 + 1) < kCoopStack && kWi
 
 // Walks lane owner's ray (st, w and stk are that lane's) to its end; every lane calls it and
 // receives the ray with its final best hit. Not inlined: the callers' loops keep their registers.
-static __device__ __noinline__ WideRay coop_wide(const float4* __restrict__ wide, const float4* __restrict__ tris,
-                                                 WideRay st, WideWalk w, const int2* stk, int owner, CoopScratch* sc) {
+template <class Stack>
+__device__ __noinline__ WideRay coop_wide(const float4* __restrict__ wide, const float4* __restrict__ tris,
+                                          WideRay st, WideWalk w, Stack stk, int owner, CoopScratch* sc) {
     const uint32_t F = 0xffffffffu;
     const int lane = threadIdx.x & 31, slot = lane >> 2, c = lane & 3;
     const uint32_t lt = lanemask_lt();
@@ -304,7 +339,7 @@ static __device__ __noinline__ WideRay coop_wide(const float4* __restrict__ wide
     st.pad = __shfl_sync(F, st.pad, owner);
     int n = __shfl_sync(F, w.sp, owner) + 1;
     if (lane == owner) {
-        for (int i = 0; i < n - 1; ++i) sc->stk[i] = stk[i];
+        for (int i = 0; i < n - 1; ++i) sc->stk[i] = stk.get(i);
         sc->stk[n - 1] = make_int2(-1, w.cur);  // a negative key: not culled
     }
     __syncwarp();
