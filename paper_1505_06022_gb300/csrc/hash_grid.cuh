@@ -212,10 +212,9 @@ __global__ void __launch_bounds__(kScanThreads) k_grid_scan(GridPlan plan, GridB
 
 // The tile's points to their parts, in order: each warp has a contiguous share of the list, counts it
 // by part, and after a sum over the warps before it walks it again, 32 points at a time, ranking equal
-// parts among the lanes. Block 0 also writes the part starts and the number of points (d_total), and
-// clears the word `clear`.
+// parts among the lanes. Block 0 also writes the part starts and clears the word `clear`.
 __global__ void __launch_bounds__(kGridThreads)
-k_grid_split(GridIn in, GridPlan plan, GridBuf buf, uint32_t* __restrict__ d_total, uint32_t* __restrict__ clear) {
+k_grid_split(GridIn in, GridPlan plan, GridBuf buf, uint32_t* __restrict__ clear) {
     __shared__ uint32_t s_base[kGridMaxParts];
     __shared__ uint16_t s_count[kGridWarps][kGridMaxParts];
     __shared__ uint32_t s_warp[kGridWarps];
@@ -234,7 +233,6 @@ k_grid_split(GridIn in, GridPlan plan, GridBuf buf, uint32_t* __restrict__ d_tot
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         buf.part_start()[plan.parts] = n;
-        if (d_total) *d_total = n;
         if (clear) *clear = 0;
     }
     __syncthreads();

@@ -55,6 +55,8 @@ static_assert(kWorkCounts == GSP_WORK_COUNTS && kWorkEyeRays == GSP_WORK_EYE_RAY
                   kWorkHitsScanned == GSP_WORK_HIT_POINTS_SCANNED,
               "the work counters of the kernels are the ones gsp.h names");
 
+constexpr int64_t kOwnGridSlots = int64_t(1) << 22;  // see gsp_sppm::TraceBuf
+
 struct gsp_sppm {
     gsp_scene* scene = nullptr;
     gsp_sppm_params P{};
@@ -71,7 +73,12 @@ struct gsp_sppm {
     // read. Two sets, so that the tracing of pass i + 1 runs while pass i is gathered and while
     // the longest paths of pass i are still being traced (gsp_sppm_pass with several passes);
     // both are made at creation. hx .. rlist alias the set
-    // in use.
+    // in use. Full-path renderers of up to kOwnGridSlots deposit slots also build a pass's hash grid on its
+    // tracing stream, in arrays of the set's own: a small pass's gather is short, and four grid
+    // launches before each one were a third of the chain that its passes wait for (four passes of
+    // 64x64 pixels and 16,384 photons 436 -> 399 us). The arrays take 48 bytes per slot; for larger renderers
+    // that costs more (a gradient step that makes a renderer of 8.4 million slots: 5.65 -> 5.90 ms,
+    // 400 MB more to map) than it gives (512x512 passes of 2^20 photons 1.4 %).
     struct TraceBuf {
         float4 *hx = nullptr, *hn = nullptr, *hf = nullptr, *hd = nullptr, *slots = nullptr;
         uint32_t* pcount = nullptr;
@@ -84,7 +91,12 @@ struct gsp_sppm {
         int2* rlist = nullptr;               // their FP64 refinement list (qcap entries)
         unsigned long long* entry = nullptr;  // stochastic hashing: the pass's table (T entries)
         uint32_t* ecount = nullptr;
+        // exact hashing: the pass's hash grid and its buffers (set 1 shares set 0's unless own_grids)
+        uint32_t *keys[2] = {nullptr, nullptr}, *vals[2] = {nullptr, nullptr}, *hist = nullptr, *bstart = nullptr;
+        float4 *spos = nullptr, *spay = nullptr;
+        uint32_t* nheavy = nullptr;  // hit points listed for k_gather_heavy, cleared by the deposit
     } tb[2];
+    bool own_grids = false;  // each trace set has its own hash grid
     int cur = 0;
     float4 *hx = nullptr, *hn = nullptr, *hf = nullptr, *hd = nullptr;
     float4* slots = nullptr;
@@ -99,6 +111,7 @@ struct gsp_sppm {
     uint32_t *keys[2] = {nullptr, nullptr}, *vals[2] = {nullptr, nullptr};
     uint32_t *hist = nullptr, *scan_tmp = nullptr, *bcount = nullptr, *bstart = nullptr;
     float4 *spos = nullptr, *spay = nullptr;
+    uint32_t* nheavy = nullptr;
     unsigned long long* entry = nullptr;
     uint32_t* ecount = nullptr;
     float4 *ro = nullptr, *rd = nullptr, *rphi = nullptr;
@@ -168,6 +181,13 @@ void free_all(gsp_sppm* r) {
 
 void use_buf(gsp_sppm* r, int j) {
     r->cur = j;
+    std::copy(r->tb[j].keys, r->tb[j].keys + 2, r->keys);
+    std::copy(r->tb[j].vals, r->tb[j].vals + 2, r->vals);
+    r->hist = r->tb[j].hist;
+    r->bstart = r->tb[j].bstart;
+    r->spos = r->tb[j].spos;
+    r->spay = r->tb[j].spay;
+    r->nheavy = r->tb[j].nheavy;
     r->hw = r->tb[j].hw;
     r->smat = r->tb[j].smat;
     r->hx = r->tb[j].hx;
@@ -217,6 +237,15 @@ void add_trace_set(gsp_sppm* r, int j, Arena& arena) {
     A(&t.qctr, 16);
     A(&t.tctr, 2);
     A(&t.rlist, r->qcap);
+    if (r->P.hash_mode == GSP_EXACT && (j == 0 || r->own_grids)) {
+        A(&t.keys[0], r->slot_cap);
+        A(&t.vals[0], r->slot_cap);
+        A(&t.keys[1], 2 * r->slot_cap);  // the parts' {bucket, slot} pairs, or the radix sort's second pair
+        A(&t.hist, gsp_sort_hist_elems());
+        A(&t.bstart, r->T + 1);
+        A(&t.spos, r->slot_cap);
+        A(&t.spay, r->slot_cap);
+    }
 }
 
 inline unsigned blocks(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
@@ -353,19 +382,13 @@ gsp_status gsp_sppm_create(gsp_scene* s, const gsp_sppm_params* params, gsp_sppm
     A(&r->started, 1);
     A(&r->work, kWorkCounts);
     if (P.hash_mode == GSP_EXACT) {
-        A(&r->keys[0], r->slot_cap);
-        A(&r->vals[0], r->slot_cap);
-        A(&r->keys[1], 2 * r->slot_cap);  // the parts' {bucket, slot} pairs, or the radix sort's second pair
-        A(&r->hist, gsp_sort_hist_elems());
         if (r->tbits > kGridMaxBits) {  // the radix sort's buffers
             A(&r->poff, r->np);
             A(&r->bcount, r->T);
             A(&r->scan_tmp, std::max({gsp_scan_temp_elems(r->np), gsp_scan_temp_elems(r->T),
                                       gsp_scan_temp_elems(gsp_sort_hist_elems())}));
         }
-        A(&r->bstart, r->T + 1);
-        A(&r->spos, r->slot_cap);
-        A(&r->spay, r->slot_cap);
+        r->own_grids = r->tbits <= kGridMaxBits && r->slot_cap <= kOwnGridSlots && P.photon_mode == GSP_FULL_PATH;
         // the heavy-query split pays on large images; on small ones its extra launch costs more
         if (r->npix >= kHeavyMinPixels) A(&r->heavy, r->npix);
     }
@@ -383,7 +406,17 @@ gsp_status gsp_sppm_create(gsp_scene* s, const gsp_sppm_params* params, gsp_sppm
         A(&r->rphi, r->np);
     }
     cudaError_t e = arena.make(r);
-    if (r->keys[1]) r->vals[1] = r->keys[1] + r->slot_cap;
+    for (int j = 0; j < 2; ++j) {
+        auto &t = r->tb[j], &grid = r->tb[r->own_grids ? j : 0];
+        if (grid.keys[1]) grid.vals[1] = grid.keys[1] + r->slot_cap;
+        std::copy(grid.keys, grid.keys + 2, t.keys);
+        std::copy(grid.vals, grid.vals + 2, t.vals);
+        t.hist = grid.hist;
+        t.bstart = grid.bstart;
+        t.spos = grid.spos;
+        t.spay = grid.spay;
+        t.nheavy = r->counters + 9 + (r->own_grids ? j : 0);
+    }
     use_buf(r, 0);
     for (cudaStream_t& t : r->tstream)
         if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&t, cudaStreamNonBlocking);
@@ -443,8 +476,8 @@ static PassDev pass_params(const gsp_sppm* r, int64_t pass) {
 }
 
 // Renderer counters (uint32): [0] deposits of the pass, [7] first pass index of a replayed graph,
-// [10] hit points listed for k_gather_heavy, [11] out-of-range pixels of a state given to
-// gsp_sppm_set_state.
+// [9..10] hit points listed for k_gather_heavy (per trace set, if each has its own grid), [11]
+// out-of-range pixels of a state given to gsp_sppm_set_state.
 // Per trace set (qctr): [4..6] eye queue lengths, [8..10] photon queue lengths (three each, used
 // in rotation), [12] work counter of k_paths, [13] work counter of k_photon_regen.
 static int sm_count(int device) {
@@ -654,14 +687,14 @@ static_assert((int64_t)kGridMaxTiles * 256 + kGridAux <= kGspSortHistElems && kG
                   512 + 2 * kGridMaxParts + 1 <= kGridAux && kGridMaxLow <= 4 * kGridThreads && kGridSegment < 65536,
               "the counts of 256 parts fit beside the aux words, those of more parts in the bucket starts");
 static cudaError_t grid_launch(const GridIn& in, int bits, uint32_t* keys, uint32_t* vals, uint2* pairs, uint32_t* hist,
-                               uint32_t* order, float4* spos, float4* spay, uint32_t* bstart, uint32_t* d_total,
-                               uint32_t* clear, cudaStream_t st) {
+                               uint32_t* order, float4* spos, float4* spay, uint32_t* bstart, uint32_t* clear,
+                               cudaStream_t st) {
     const GridPlan plan = grid_plan(in.items, bits);
     const bool beside = (int64_t)plan.tiles * plan.parts <= kGspSortHistElems - kGridAux;
     const GridBuf buf{keys, vals, pairs, beside ? hist : bstart, hist + kGspSortHistElems - kGridAux};
     if (plan.tiles) k_grid_tiles<<<plan.tiles, kGridThreads, 0, st>>>(in, plan, buf);
     k_grid_scan<<<(plan.parts + 31) / 32, kScanThreads, 0, st>>>(plan, buf);
-    k_grid_split<<<std::max(1, plan.tiles), kGridThreads, 0, st>>>(in, plan, buf, d_total, clear);
+    k_grid_split<<<std::max(1, plan.tiles), kGridThreads, 0, st>>>(in, plan, buf, clear);
     k_grid_parts<<<plan.parts, kGridThreads, 0, st>>>(in, plan, buf, order, spos, spay, bstart);
     return cudaGetLastError();
 }
@@ -674,12 +707,12 @@ static GridIn deposits_in(const gsp_sppm* r, float inv_h, uint32_t mask) {
 // copies. Tables of more than 2^kGridMaxBits buckets (more than 2^20 photons a pass by default) are
 // sorted by radix passes.
 static gsp_status stage_deposit(gsp_sppm* r, const PassDev& P, cudaStream_t st) {
-    uint32_t* d_total = r->counters;  // deposits this pass
     if (r->tbits <= kGridMaxBits) {
         GSP_CUDA_TRY(grid_launch(deposits_in(r, r->inv_h, P.tmask), r->tbits, r->keys[0], r->vals[0], (uint2*)r->keys[1], r->hist,
-                                 nullptr, r->spos, r->spay, r->bstart, d_total, r->counters + 10, st));
+                                 nullptr, r->spos, r->spay, r->bstart, r->nheavy, st));
         return GSP_OK;
     }
+    uint32_t* d_total = r->counters;
     GSP_CUDA_TRY(gsp_scan_u32(r->pcount, r->poff, r->np, d_total, r->scan_tmp, st));
     GSP_CUDA_TRY(cudaMemsetAsync(r->bcount, 0, r->T * sizeof(uint32_t), st));
     k_compact<<<blocks(r->np, 256), 256, 0, st>>>(r->slots, r->pcount, r->poff, r->np, r->slots_per_path, r->inv_h,
@@ -689,7 +722,7 @@ static gsp_status stage_deposit(gsp_sppm* r, const PassDev& P, cudaStream_t st) 
     GSP_CUDA_TRY(gsp_radix_sort_u32(r->keys[0], r->vals[0], r->keys[1], r->vals[1], d_total, r->tbits, r->hist,
                                     r->scan_tmp, st, &ko, &vo));
     k_permute<<<1024, 256, 0, st>>>(r->slots, vo, d_total, r->spos, r->spay);
-    GSP_CUDA_TRY(cudaMemsetAsync(r->counters + 10, 0, sizeof(uint32_t), st));
+    GSP_CUDA_TRY(cudaMemsetAsync(r->nheavy, 0, sizeof(uint32_t), st));
     GSP_CUDA_TRY(cudaGetLastError());
     return GSP_OK;
 }
@@ -704,8 +737,8 @@ static gsp_status trace_half(gsp_sppm* r, const PassDev& P, cudaStream_t st) {
     return stage_paths(r, P, O, D, st);
 }
 
-// Gather half of a pass: deposit (exact mode) and the fused range query + progressive update.
-static gsp_status gather_half(gsp_sppm* r, const PassDev& P, cudaStream_t st) {
+// Gather half of a pass: deposit (exact mode, unless done) and the fused range query + progressive update.
+static gsp_status gather_half(gsp_sppm* r, const PassDev& P, cudaStream_t st, bool deposited = false) {
     NvtxRange nvtx("gsp: deposit + gather");
     GatherDev G{};
     G.hx = r->hx;
@@ -726,15 +759,16 @@ static gsp_status gather_half(gsp_sppm* r, const PassDev& P, cudaStream_t st) {
         GSP_CUDA_TRY(cudaMemsetAsync(G.total, 0, sizeof(uint32_t), st));
         k_gather_stoch<<<blocks(r->npix, 128), 128, 0, st>>>(G, P);
     } else {
-        gsp_status e = stage_deposit(r, P, st);
+        const gsp_status e = deposited ? GSP_OK : stage_deposit(r, P, st);
         if (e != GSP_OK) return e;
+        G.total = r->counters;
         G.spos = r->spos;
         G.spay = r->spay;
         G.bstart = r->bstart;
-        // long queries are listed by k_gather_exact and served by whole blocks (counters[10] counts them)
+        // long queries are listed by k_gather_exact and served by whole blocks (*nheavy counts them)
         if (r->heavy) {
             G.heavy = r->heavy;
-            G.nheavy = r->counters + 10;  // cleared by the deposit
+            G.nheavy = r->nheavy;  // cleared by the deposit
         }
         launch_gather_exact(r->gather_lanes, G, P, r->npix, st);
         if (r->heavy) k_gather_heavy<<<2 * sm_count(r->scene->ctx->device), kHeavyThreads, 0, st>>>(G, P);
@@ -778,7 +812,8 @@ static gsp_status sppm_one_pass(gsp_sppm* r, cudaStream_t st, bool graph = false
 // Several passes, pass i traced on tracing stream i % 2 into trace set i % 2 while the caller's
 // stream deposits and gathers the pass before: the tracing of pass i + 1 starts as soon as its
 // set has been gathered (pass i - 1), so it runs beside the long tail of pass i's path kernel,
-// when only the longest paths are still going, and beside pass i's sort and gather. Events order
+// when only the longest paths are still going, and beside pass i's sort and gather (the sort goes to
+// the tracing stream where the set has a grid of its own). Events order
 // each set's reuse (and, with paths carried from pass to pass, the tracing itself); results are
 // those of one pass after the other. Exact hashing only (stochastic hashing shares its table
 // between the two halves).
@@ -787,6 +822,7 @@ static gsp_status passes_overlapped(gsp_sppm* r, int32_t npasses, cudaStream_t s
     GSP_CUDA_TRY(cudaEventRecord(r->ev_start, st));
     for (cudaStream_t t : r->tstream) GSP_CUDA_TRY(cudaStreamWaitEvent(t, r->ev_start, 0));
     const bool chained = r->P.photon_mode == GSP_REGEN;  // photon paths continue into the next pass
+    const bool deposit = r->own_grids;
     for (int32_t i = 0; i < npasses; ++i) {
         const int j = i & 1;
         use_buf(r, j);
@@ -794,10 +830,11 @@ static gsp_status passes_overlapped(gsp_sppm* r, int32_t npasses, cudaStream_t s
         if (i >= 2) GSP_CUDA_TRY(cudaStreamWaitEvent(r->tstream[j], r->ev_free[j], 0));  // pass i - 2 gathered
         if (chained && i >= 1) GSP_CUDA_TRY(cudaStreamWaitEvent(r->tstream[j], r->ev_traced[j ^ 1], 0));
         gsp_status e = trace_half(r, P, r->tstream[j]);
+        if (e == GSP_OK && deposit) e = stage_deposit(r, P, r->tstream[j]);
         if (e != GSP_OK) return e;
         GSP_CUDA_TRY(cudaEventRecord(r->ev_traced[j], r->tstream[j]));
         GSP_CUDA_TRY(cudaStreamWaitEvent(st, r->ev_traced[j], 0));
-        e = gather_half(r, P, st);
+        e = gather_half(r, P, st, deposit);
         if (e != GSP_OK) return e;
         GSP_CUDA_TRY(cudaEventRecord(r->ev_free[j], st));
         r->passes += 1;
@@ -1726,7 +1763,7 @@ gsp_status gsp_grid_build_with(const float4* pos, int64_t n, float cell_h, int64
     if (tbits - (skip_invalid ? 1 : 0) <= kGridMaxBits) {
         GSP_CUDA_TRY(grid_launch(GridIn{pos, nullptr, n, 1, skip_invalid ? 1 : 0, 1.0f / cell_h, (uint32_t)(T - 1)},
                                  tbits - (skip_invalid ? 1 : 0), ka, va, (uint2*)kb, hist, order, nullptr, nullptr, bstart, nullptr,
-                                 nullptr, st));
+                                 st));
         return GSP_OK;
     }
     GSP_CUDA_TRY(cudaMemsetAsync(bstart, 0, (size_t)T * sizeof(uint32_t), st));

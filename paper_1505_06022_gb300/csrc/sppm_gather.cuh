@@ -61,7 +61,7 @@ struct GatherDev {
     const unsigned long long* __restrict__ entry;
     const uint32_t* __restrict__ ecount;
     const uint32_t* __restrict__ pcount;  // deposits per path, summed into *total (zeroed before) for diagnostics
-    uint32_t* __restrict__ total;
+    uint32_t* __restrict__ total;           // (exact: set to the grid's count, if given)
     int64_t npix;
     float* __restrict__ rhist;  // optional: [pass][npix] radius each pixel gathered with (gradient)
     float4* __restrict__ shist; // optional: [pass][npix] sum of the gathered photons' flux (gradient)
@@ -290,6 +290,7 @@ __global__ void __launch_bounds__(128) k_gather_exact(GatherDev G, PassDev P) {
     static_assert(L >= 1 && L <= 32 && (L & (L - 1)) == 0, "group size");
     const int gl = threadIdx.x & (L - 1);
     const int64_t p = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / L;
+    if (G.total && blockIdx.x == 0 && threadIdx.x == 0) *G.total = G.bstart[(size_t)P.tmask + 1];
     if (p >= G.npix) return;
     const float4 hxp = G.hx[p];
     if (__float_as_int(hxp.w) < 0) {  // the whole group leaves together
