@@ -997,8 +997,10 @@ gsp_status gsp_render_grad(gsp_sppm* r, const float* d_dloss_dimg, float* d_grad
         k_adj_photons<GSP_ADJ_LANES><<<dim3(list.tiles, GSP_ADJ_COLUMNS), 128, 0, st>>>(A);
         k_adj_pixels<<<grid, 256, 0, st>>>(r->hx, r->hw, A.rhist, r->shist + (size_t)i * r->npix, d_dloss_dimg,
                                            r->npix, r->gacc, nmat);
-        k_adj_paths<<<grid, 128, 0, st>>>(r->slots, r->pcount, r->smat, r->badj, r->scene->d_mats, r->np, r->gacc,
-                                          nmat);
+        // a path per thread hides its loads best; past 16 blocks per SM their sums in global memory cost more
+        // (262,144 paths: 4 blocks per SM 28 us, 8 25, 16 24)
+        k_adj_paths<<<(unsigned)std::min<int64_t>(blocks(r->np, 128), 4 * grid), 128, 0, st>>>(
+            r->slots, r->pcount, r->smat, r->badj, r->scene->d_mats, r->np, r->gacc, nmat);
         GSP_CUDA_TRY(cudaEventRecord(r->ev_free[j], st));
     }
     const double ne = (double)r->passes * (double)r->np;
