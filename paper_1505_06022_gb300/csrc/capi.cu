@@ -467,7 +467,7 @@ static void scene_free_bvh(gsp_scene* s) {
 void gsp_scene_destroy(gsp_scene* s) {
     if (!s) return;
     if (s->ctx) {
-        cudaSetDevice(s->ctx->device);
+        cudaSetDevice(s->device);
         scene_free_bvh(s);
         trace_events_free(s);
         cudaFree(s->d_shade);
@@ -512,6 +512,7 @@ gsp_status gsp_scene_upload(gsp_context* ctx, const float* verts, int64_t nv, co
     gsp_scene* s = new (std::nothrow) gsp_scene;
     if (!s) return GSP_ERR_OOM;
     s->ctx = ctx;
+    s->device = ctx ? ctx->device : 0;
     s->nv = nv;
     s->nt = nt;
     s->nmat = nmat;

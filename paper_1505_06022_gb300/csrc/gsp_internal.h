@@ -62,6 +62,7 @@ struct gsp_context {
 
 struct gsp_scene {
     gsp_context* ctx = nullptr;
+    int32_t device = 0;  // the context's: destroying a scene does not read the context, which may be gone
     int64_t nv = 0, nt = 0;
     int32_t nmat = 0;
     std::vector<float> verts;

@@ -59,6 +59,7 @@ constexpr int64_t kOwnGridSlots = int64_t(1) << 22;  // see gsp_sppm::TraceBuf
 
 struct gsp_sppm {
     gsp_scene* scene = nullptr;
+    int32_t device = 0;  // the scene's: destroying a renderer does not read the scene, which may be gone
     gsp_sppm_params P{};
     int32_t w = 0, h = 0;
     int64_t npix = 0, np = 0, T = 0, slot_cap = 0;
@@ -329,6 +330,7 @@ gsp_status gsp_sppm_create(gsp_scene* s, const gsp_sppm_params* params, gsp_sppm
     gsp_sppm* r = new (std::nothrow) gsp_sppm;
     if (!r) return GSP_ERR_OOM;
     r->scene = s;
+    r->device = s->ctx->device;
     r->P = P;
     r->w = s->cam.width;
     r->h = s->cam.height;
@@ -447,7 +449,7 @@ gsp_status gsp_sppm_create(gsp_scene* s, const gsp_sppm_params* params, gsp_sppm
 
 void gsp_sppm_destroy(gsp_sppm* r) {
     if (!r) return;
-    cudaSetDevice(r->scene->ctx->device);
+    cudaSetDevice(r->device);
     for (cudaStream_t t : r->tstream)
         if (t) cudaStreamDestroy(t);
     for (cudaEvent_t ev : {r->ev_start, r->ev_traced[0], r->ev_traced[1], r->ev_free[0], r->ev_free[1]})
