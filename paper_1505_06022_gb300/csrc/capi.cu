@@ -181,6 +181,7 @@ k_trace_wide(DevScene S, const float4* __restrict__ rays, int64_t n, const uint3
              int32_t* __restrict__ tri, float* __restrict__ tout, float2* __restrict__ uv,
              unsigned long long* __restrict__ ctr, int2* __restrict__ rlist, float refine_factor, int32_t out_slot,
              int32_t chunk) {
+    wait_previous();
     if (d_n) n = min(n, (int64_t)*d_n);
     const int lane = threadIdx.x & 31;
     const uint32_t lt = lanemask_lt();
@@ -258,6 +259,7 @@ k_trace_wide(DevScene S, const float4* __restrict__ rays, int64_t n, const uint3
 }
 
 __global__ void k_zero_u64x2(unsigned long long* p) {
+    gspd::release_next();
     p[0] = 0ull;
     p[1] = 0ull;
 }
@@ -312,8 +314,8 @@ static void run_trace(const gspd::DevScene& S, int device, const float4* rays, i
     if (e0) cudaEventRecord(e0, st);
     if (S.wide) {
         auto* const kernel = list ? gspd::k_trace_wide<true> : gspd::k_trace_wide<false>;
-        kernel<<<(unsigned)wide_grid, kTraceThreads, 0, st>>>(S, rays, n, d_n, tri, t, uv, ctr, rlist, refine_factor,
-                                                              out_slot, chunk);
+        gsp_launch_after(kernel, wide_grid, kTraceThreads, st, S, rays, n, d_n, tri, t, uv, ctr, rlist, refine_factor,
+                         out_slot, chunk);
     } else
         gspd::k_trace<<<links_grid, kTraceThreads, 0, st>>>(S, rays, n, d_n, tri, t, uv, ctr, rlist, refine_factor,
                                                             out_slot);

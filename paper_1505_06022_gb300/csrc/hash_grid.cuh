@@ -124,6 +124,8 @@ __global__ void __launch_bounds__(kGridThreads) k_grid_tiles(GridIn in, GridPlan
     __shared__ uint32_t s_count[kGridMaxParts];
     __shared__ uint32_t s_list[kGridList];
     __shared__ uint32_t s_warp[kGridWarps];
+    release_next();
+    wait_previous();
     const int64_t first = (int64_t)blockIdx.x * plan.per_tile, end = min(first + plan.per_tile, in.items);
     uint32_t* vals = buf.vals0 + first * in.per;
     uint32_t* keys = buf.keys0 + first * in.per;
@@ -181,6 +183,8 @@ __global__ void __launch_bounds__(kScanThreads) k_grid_scan(GridPlan plan, GridB
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, d = blockIdx.x * 32 + lane;
     const bool live = d < plan.parts;
     uint32_t c[kRun], sum = 0;
+    release_next();
+    wait_previous();
 #pragma unroll
     for (int j = 0; j < kRun; ++j) {
         const int t = warp * kRun + j;
@@ -222,6 +226,8 @@ k_grid_split(GridIn in, GridPlan plan, GridBuf buf, uint32_t* __restrict__ clear
     const uint32_t lt = lanemask_lt();
     // where each part starts: an exclusive sum of the totals, then the tiles before this one
     const int run = (plan.parts + kGridThreads - 1) / kGridThreads;
+    release_next();
+    wait_previous();
     const int a = min((int)threadIdx.x * run, plan.parts), z = min(a + run, plan.parts);
     uint32_t mine = 0, n;
     for (int d = a; d < z; ++d) mine += buf.total()[d];
@@ -307,6 +313,8 @@ k_grid_parts(GridIn in, GridPlan plan, GridBuf buf, uint32_t* __restrict__ order
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t lt = lanemask_lt();
     const int nb = 1 << plan.low;
+    release_next();
+    wait_previous();
     const uint32_t start = buf.part_start()[blockIdx.x], stop = buf.part_start()[blockIdx.x + 1], m = stop - start;
     uint32_t* bs = bstart + (size_t)blockIdx.x * nb;
     if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) bstart[(size_t)gridDim.x * nb] = stop;

@@ -140,6 +140,7 @@ k_paths_pool(const __grid_constant__ PathJob one, const PathJob* __restrict__ jo
     PathPool& pl = pools[threadIdx.x >> 5];
     WarpQueue wq;
     MultiQueue mq;
+    wait_previous();
     const int32_t ne1 = !MULTI && one.ne_ptr ? (int32_t)*one.ne_ptr : 0;
     if (MULTI)
         mq.init(jobs, njobs, total_chunks);

@@ -501,10 +501,10 @@ static unsigned shade_blocks(int64_t n, int device) {
 // Exact gather with `lanes` lanes per hit point (1, 4, 8 or 16).
 static void launch_gather_exact(int lanes, const GatherDev& G, const PassDev& P, int64_t npix, cudaStream_t st) {
     switch (lanes) {
-        case 1: k_gather_exact<1><<<blocks(npix, 128), 128, 0, st>>>(G, P); break;
-        case 4: k_gather_exact<4><<<blocks(npix * 4, 128), 128, 0, st>>>(G, P); break;
-        case 16: k_gather_exact<16><<<blocks(npix * 16, 128), 128, 0, st>>>(G, P); break;
-        default: k_gather_exact<8><<<blocks(npix * 8, 128), 128, 0, st>>>(G, P); break;
+        case 1: gsp_launch_after(k_gather_exact<1>, blocks(npix, 128), 128, st, G, P); break;
+        case 4: gsp_launch_after(k_gather_exact<4>, blocks(npix * 4, 128), 128, st, G, P); break;
+        case 16: gsp_launch_after(k_gather_exact<16>, blocks(npix * 16, 128), 128, st, G, P); break;
+        default: gsp_launch_after(k_gather_exact<8>, blocks(npix * 8, 128), 128, st, G, P); break;
     }
 }
 
@@ -588,7 +588,7 @@ static gsp_status photon_front(gsp_sppm* r, const PassDev& P, const DepositDev& 
     }
     b = -1;
     if (r->P.photon_mode == GSP_FULL_PATH) {
-        k_photon_emit<<<blocks(r->np, 256), 256, 0, st>>>(E, P, r->q[0], r->pcount, qn, tctr, r->qctr + 12);
+        gsp_launch_after(k_photon_emit, blocks(r->np, 256), 256, st, E, P, r->q[0], r->pcount, qn, tctr, r->qctr + 12);
         for (b = 0; b < r->photon_steps && b < r->P.max_photon_depth; ++b) {
             const PathQ& cur = r->q[b & 1];
             GSP_CUDA_TRY(gsp_trace_queue(s, cur.ray, r->np, qn + b % 3, cur.tri, cur.t, rf, false, !list, tctr, r->rlist, st));
@@ -665,8 +665,8 @@ static gsp_status stage_paths(gsp_sppm* r, const PassDev& P, const EyeOut& O, co
         else if (walk == kWide)
         {
             const auto pooled = [&](auto kernel) {
-                kernel<<<grid, kTraceThreads, 0, st>>>(J, nullptr, 0, 0, r->qctr + 12, path_chunk(items, grid),
-                                                       pool_size(items, grid));
+                gsp_launch_after(kernel, grid, kTraceThreads, st, J, nullptr, 0, 0, r->qctr + 12, path_chunk(items, grid),
+                                 pool_size(items, grid));
             };
             if (J.nregen)
                 J.S.attr ? pooled(k_paths_pool<false, true, true>) : pooled(k_paths_pool<false, false, true>);
@@ -694,10 +694,10 @@ static cudaError_t grid_launch(const GridIn& in, int bits, uint32_t* keys, uint3
     const GridPlan plan = grid_plan(in.items, bits);
     const bool beside = (int64_t)plan.tiles * plan.parts <= kGspSortHistElems - kGridAux;
     const GridBuf buf{keys, vals, pairs, beside ? hist : bstart, hist + kGspSortHistElems - kGridAux};
-    if (plan.tiles) k_grid_tiles<<<plan.tiles, kGridThreads, 0, st>>>(in, plan, buf);
-    k_grid_scan<<<(plan.parts + 31) / 32, kScanThreads, 0, st>>>(plan, buf);
-    k_grid_split<<<std::max(1, plan.tiles), kGridThreads, 0, st>>>(in, plan, buf, clear);
-    k_grid_parts<<<plan.parts, kGridThreads, 0, st>>>(in, plan, buf, order, spos, spay, bstart);
+    if (plan.tiles) gsp_launch_after(k_grid_tiles, plan.tiles, kGridThreads, st, in, plan, buf);
+    gsp_launch_after(k_grid_scan, (plan.parts + 31) / 32, kScanThreads, st, plan, buf);
+    gsp_launch_after(k_grid_split, std::max(1, plan.tiles), kGridThreads, st, in, plan, buf, clear);
+    gsp_launch_after(k_grid_parts, plan.parts, kGridThreads, st, in, plan, buf, order, spos, spay, bstart);
     return cudaGetLastError();
 }
 
@@ -773,7 +773,7 @@ static gsp_status gather_half(gsp_sppm* r, const PassDev& P, cudaStream_t st, bo
             G.nheavy = r->nheavy;  // cleared by the deposit
         }
         launch_gather_exact(r->gather_lanes, G, P, r->npix, st);
-        if (r->heavy) k_gather_heavy<<<2 * sm_count(r->scene->ctx->device), kHeavyThreads, 0, st>>>(G, P);
+        if (r->heavy) gsp_launch_after(k_gather_heavy, 2 * sm_count(r->scene->ctx->device), kHeavyThreads, st, G, P);
     }
     if (P.work) k_work_add<<<1, 1, 0, st>>>(P.work + kWorkDeposits, r->counters);
     GSP_CUDA_TRY(cudaGetLastError());
@@ -995,14 +995,13 @@ gsp_status gsp_render_grad(gsp_sppm* r, const float* d_dloss_dimg, float* d_grad
         A.work = r->count_work ? r->work : nullptr;
         A.hp_rec = r->hp_rec;
         if (A.work) k_work_sum<<<1, 256, 0, st>>>(A.work + kWorkDeposits, A.tile_count, list.tiles);
-        k_adj_hp_records<<<blocks(r->npix, 256), 256, 0, st>>>(A, r->npix, r->hp_rec);
-        k_adj_photons<GSP_ADJ_LANES><<<dim3(list.tiles, GSP_ADJ_COLUMNS), 128, 0, st>>>(A);
-        k_adj_pixels<<<grid, 256, 0, st>>>(r->hx, r->hw, A.rhist, r->shist + (size_t)i * r->npix, d_dloss_dimg,
+        gsp_launch_after(k_adj_hp_records, blocks(r->npix, 256), 256, st, A, r->npix, r->hp_rec);
+        gsp_launch_after(k_adj_photons<GSP_ADJ_LANES>, dim3(list.tiles, GSP_ADJ_COLUMNS), 128, st, A);
+        gsp_launch_after(k_adj_pixels, grid, 256, st, r->hx, r->hw, A.rhist, r->shist + (size_t)i * r->npix, d_dloss_dimg,
                                            r->npix, r->gacc, nmat);
         // a path per thread hides its loads best; past 16 blocks per SM their sums in global memory cost more
         // (262,144 paths: 4 blocks per SM 28 us, 8 25, 16 24)
-        k_adj_paths<<<(unsigned)std::min<int64_t>(blocks(r->np, 128), 4 * grid), 128, 0, st>>>(
-            r->slots, r->pcount, r->smat, r->badj, r->scene->d_mats, r->np, r->gacc, nmat);
+        gsp_launch_after(k_adj_paths, std::min<int64_t>(blocks(r->np, 128), 4 * grid), 128, st, r->slots, r->pcount, r->smat, r->badj, r->scene->d_mats, r->np, r->gacc, nmat);
         GSP_CUDA_TRY(cudaEventRecord(r->ev_free[j], st));
     }
     const double ne = (double)r->passes * (double)r->np;

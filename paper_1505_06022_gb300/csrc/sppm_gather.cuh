@@ -288,6 +288,8 @@ constexpr int64_t kGatherWideBelow = 256 * 256;
 template <int L>
 __global__ void __launch_bounds__(128) k_gather_exact(GatherDev G, PassDev P) {
     static_assert(L >= 1 && L <= 32 && (L & (L - 1)) == 0, "group size");
+    release_next();
+    wait_previous();
     const int gl = threadIdx.x & (L - 1);
     const int64_t p = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / L;
     if (G.total && blockIdx.x == 0 && threadIdx.x == 0) *G.total = G.bstart[(size_t)P.tmask + 1];
@@ -337,6 +339,8 @@ __global__ void __launch_bounds__(128) k_gather_exact(GatherDev G, PassDev P) {
 constexpr int kHeavyThreads = 256;
 
 __global__ void __launch_bounds__(kHeavyThreads) k_gather_heavy(GatherDev G, PassDev P) {
+    release_next();
+    wait_previous();
     __shared__ float s_sum[kHeavyThreads / 32][4];
     __shared__ uint32_t s_scan[kHeavyThreads / 32];
     const uint32_t count = *G.nheavy;
@@ -415,6 +419,8 @@ struct AdjDev {
 // instead of through the order array, with the loss term already formed (the same operations as
 // forming it per photon).
 __global__ void __launch_bounds__(256) k_adj_hp_records(AdjDev A, int64_t npix, float4* __restrict__ rec) {
+    release_next();
+    wait_previous();
     const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= npix || j >= A.hp_bstart[(size_t)A.hp_mask + 1]) return;  // pixels without a hit point are in no bucket
     const uint32_t p = A.hp_order[j];
@@ -435,6 +441,8 @@ __global__ void __launch_bounds__(256) k_adj_hp_records(AdjDev A, int64_t npix, 
 // blockIdx.x is the tile of paths whose deposits the block serves, with the blocks of its column.
 template <int L>
 __global__ void __launch_bounds__(128) k_adj_photons(AdjDev A) {
+    release_next();
+    wait_previous();
     const int nd = (int)A.tile_count[blockIdx.x];
     const uint32_t* list = A.list + blockIdx.x * A.tile_stride;
     const int gl = threadIdx.x & (L - 1);
@@ -508,6 +516,8 @@ __global__ void __launch_bounds__(256)
 k_adj_pixels(const float4* __restrict__ hx, const float4* __restrict__ hw, const float* __restrict__ rhist,
              const float4* __restrict__ shist, const float* __restrict__ g, int64_t npix, double* __restrict__ acc,
              int32_t nmat) {
+    release_next();
+    wait_previous();
     __shared__ float s_acc[kMaxGradMats * 3];
     for (int i = threadIdx.x; i < nmat * 3; i += blockDim.x) s_acc[i] = 0.0f;
     __syncthreads();
@@ -536,6 +546,8 @@ __global__ void __launch_bounds__(128)
 k_adj_paths(const float4* __restrict__ slots, const uint32_t* __restrict__ pcount, const int32_t* __restrict__ smat,
             const float4* __restrict__ badj, const float4* __restrict__ mats, int64_t np, double* __restrict__ acc,
             int32_t nmat) {
+    release_next();
+    wait_previous();
     __shared__ float s_acc[kMaxGradMats * 3];
     for (int i = threadIdx.x; i < nmat * 3; i += blockDim.x) s_acc[i] = 0.0f;
     __syncthreads();

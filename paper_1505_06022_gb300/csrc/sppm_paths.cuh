@@ -469,6 +469,7 @@ __device__ __forceinline__ bool path_interact(const DevScene& S, const PassDev& 
 __global__ void __launch_bounds__(256)
 k_eye_emit(CamDev C, PassDev P, PathQ Q, EyeOut O, uint32_t* __restrict__ qn, unsigned long long* __restrict__ trace_ctr,
            uint32_t* __restrict__ tail_ctr) {
+    release_next();
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t npix = (int64_t)C.w * C.h;
     if (p == 0) {
@@ -584,6 +585,7 @@ __device__ __forceinline__ void emit_photon(const EmitDev& E, Rng& rng, float3& 
 __global__ void __launch_bounds__(256)
 k_photon_emit(EmitDev E, PassDev P, PathQ Q, uint32_t* __restrict__ pcount, uint32_t* __restrict__ qn,
               unsigned long long* __restrict__ trace_ctr, uint32_t* __restrict__ tail_ctr) {
+    release_next();
     const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (k == 0) {
         trace_ctr[0] = 0ull;
@@ -602,6 +604,7 @@ k_photon_emit(EmitDev E, PassDev P, PathQ Q, uint32_t* __restrict__ pcount, uint
     Q.rng[k] = make_int4(rng.s[0], rng.s[1], rng.s[2], rng.s[3]);
     Q.meta[k] = 0;
     pcount[k] = 0;
+    wait_previous();  // nothing above needs it, but this grid must not end before k_eye_emit's
 }
 
 // Wavefront step b of the photon pass: shade the traced queue qn[b % 3] (deposit, Russian
