@@ -280,58 +280,12 @@ std::string bvh_build_host(const float* verts, int64_t nv, const int32_t* tris, 
             dst[2 * q + 1] = float4{nd.hi[0], nd.hi[1], nd.hi[2], as_float(word)};
         }
     };
-    // ---- the same tree four-wide: internal nodes of even depth, numbered in preorder ----
-    auto wide_tree = [&]() {
-        std::vector<int32_t> wid(nn, -1), order;
-        std::vector<int8_t> odd(nn, 0);
-        for (int64_t n = 0; n < nn; ++n)  // parents come before their children
-            if (nodes[n].left >= 0) odd[nodes[n].left] = odd[nodes[n].right] = !odd[n];
-        std::vector<int32_t> st{0};
-        while (!st.empty()) {
-            const int32_t n = st.back();
-            st.pop_back();
-            if (nodes[n].left < 0) continue;
-            if (!odd[n]) {
-                wid[n] = (int32_t)order.size();
-                order.push_back(n);
-            }
-            st.push_back(nodes[n].right);
-            st.push_back(nodes[n].left);
-        }
-        out.wide.resize(order.size() * 8);
-        for (size_t i = 0; i < order.size(); ++i) {
-            int32_t ch[4], m = 0;
-            for (int32_t c : {nodes[order[i]].left, nodes[order[i]].right}) {
-                if (nodes[c].left < 0) {
-                    ch[m++] = c;
-                } else {
-                    ch[m++] = nodes[c].left;
-                    ch[m++] = nodes[c].right;
-                }
-            }
-            float q[32];
-            for (int k = 0; k < 4; ++k) {
-                for (int a = 0; a < 3; ++a)
-                    if (k < m)
-                        gsp_wide_box(nodes[ch[k]].lo[a], nodes[ch[k]].hi[a], q[8 * a + k], q[8 * a + 4 + k]);
-                    else
-                        q[8 * a + k] = 0.0f, q[8 * a + 4 + k] = -FLT_MAX;  // near beyond far on every ray
-                int32_t ref = INT32_MIN;  // no child
-                if (k < m) ref = nodes[ch[k]].left >= 0 ? wid[ch[k]] : ~((nodes[ch[k]].first << 3) | nodes[ch[k]].count);
-                q[24 + k] = as_float(ref);
-                q[28 + k] = 0.0f;
-            }
-            std::memcpy(&out.wide[8 * i], q, sizeof q);
-        }
-    };
     {
         std::vector<std::thread> th;
         for (int c = 1; c < sets; ++c) {
             if (nthreads > 1) th.emplace_back(thread_set, c);
             else thread_set(c);
         }
-        if (nthreads > 1) th.emplace_back(wide_tree);  // beside the link sets
-        else wide_tree();
         thread_set(0);
         for (auto& x : th) x.join();
     }
@@ -340,9 +294,10 @@ std::string bvh_build_host(const float* verts, int64_t nv, const int32_t* tris, 
     // ---- the same tree as child pairs (stack-based traversal), internal nodes in preorder ----
     {
         std::vector<int32_t> ref(nn, 0), st;
+        std::vector<int8_t> odd(nn, 0);
         int32_t ni = 0;
         st.push_back(0);
-        while (!st.empty()) {  // preorder numbering of the internal nodes
+        while (!st.empty()) {  // preorder numbering of the internal nodes, and of those of even depth
             int32_t n = st.back();
             st.pop_back();
             if (nodes[n].left < 0) {
@@ -350,6 +305,8 @@ std::string bvh_build_host(const float* verts, int64_t nv, const int32_t* tris, 
                 continue;
             }
             ref[n] = ni++;
+            out.wide_of.push_back(odd[n] ? -1 : (int32_t)out.nwide++);
+            odd[nodes[n].left] = odd[nodes[n].right] = !odd[n];
             st.push_back(nodes[n].right);
             st.push_back(nodes[n].left);
         }

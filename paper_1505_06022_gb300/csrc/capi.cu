@@ -732,10 +732,17 @@ gsp_status gsp_build_bvh(gsp_scene* s, const gsp_bvh_params* params, gsp_bvh_sta
         GSP_CUDA_TRY(cudaMalloc(&s->d_bin, bb));
         if (!bvh.bin.empty())
             GSP_CUDA_TRY(cudaMemcpy(s->d_bin, bvh.bin.data(), bvh.bin.size() * sizeof(float4), cudaMemcpyHostToDevice));
-        if (!bvh.wide.empty()) {
-            GSP_CUDA_TRY(cudaMalloc(&s->d_wide, bvh.wide.size() * sizeof(float4)));
-            GSP_CUDA_TRY(cudaMemcpy(s->d_wide, bvh.wide.data(), bvh.wide.size() * sizeof(float4), cudaMemcpyHostToDevice));
-            std::vector<float4>().swap(bvh.wide);  // only the device walks it
+        if (bvh.nwide) {
+            uint32_t* of = nullptr;
+            const size_t ob = bvh.wide_of.size() * sizeof(int32_t);
+            GSP_CUDA_TRY(cudaMalloc(&s->d_wide, (size_t)bvh.nwide * 8 * sizeof(float4)));
+            GSP_CUDA_TRY(cudaMalloc(&of, ob));
+            cudaError_t e = cudaMemcpy(of, bvh.wide_of.data(), ob, cudaMemcpyHostToDevice);
+            if (e == cudaSuccess) e = gsp_wide_build(s->d_bin, (int64_t)bvh.wide_of.size(), nullptr, of, s->d_wide);
+            if (e == cudaSuccess) e = cudaDeviceSynchronize();
+            cudaFree(of);
+            GSP_CUDA_TRY(e);
+            std::vector<int32_t>().swap(bvh.wide_of);
         }
     }
     s->bvh = std::move(bvh);

@@ -4,6 +4,7 @@
 #include <nvtx3/nvToolsExt.h>
 #include <cuda_runtime.h>
 
+#include <cfloat>
 #include <cstdint>
 #include <string>
 #include <vector>
@@ -26,10 +27,10 @@ struct HostBVH {
     // >= 0 is an internal node, < 0 is ~(leaf word). bin_root: ref of the root.
     std::vector<float4> bin;
     int32_t bin_root = 0;
-    // The same tree four-wide (wide.cuh): an entry of eight float4 per internal node of even depth,
-    // whose children are that node's grandchildren (or the child itself where it is a leaf).
-    // Empty for a tree that is a single leaf. The device build keeps none here.
-    std::vector<float4> wide;
+    // The same tree four-wide (wide.cuh): the entry of each of bin's nodes, -1 for a node of odd depth
+    // (gsp_wide_entry makes them). Empty for a tree that is a single leaf. The device build keeps none here.
+    std::vector<int32_t> wide_of;
+    int64_t nwide = 0;
     double build_ms = 0, thread_ms = 0;
 };
 
@@ -43,6 +44,44 @@ inline void gsp_wide_box(float lo, float hi, float& c, float& h) {
     const float a = hi - c, b = c - lo;  // each within one rounding (2^-24) of the exact value
     h = (a > b ? a : b) * (1.0f + 0x1p-19f + 0x1p-22f);
 }
+
+// The entry of the four-wide tree (layout in wide.cuh) of node i of the child pairs: the boxes of its
+// grandchildren, or a child's own where that is a leaf. of(j) is the entry of node j.
+template <class Of>
+#ifdef __CUDACC__
+__host__ __device__
+#endif
+inline void gsp_wide_entry(const float4* bin, int64_t i, Of of, float4* entry) {
+    float* q = (float*)entry;
+    int32_t* ref = (int32_t*)entry + 24;
+    int m = 0;
+    const auto add = [&](const float4& lo, const float4& hi, int32_t r) {
+        const float l[3] = {lo.x, lo.y, lo.z}, h[3] = {hi.x, hi.y, hi.z};
+        for (int a = 0; a < 3; ++a) gsp_wide_box(l[a], h[a], q[8 * a + m], q[8 * a + 4 + m]);
+        ref[m++] = r < 0 ? r : of(r);
+    };
+    const auto word = [](const float& f) { return *(const int32_t*)&f; };
+    for (int c = 0; c < 2; ++c) {
+        const float4* b = bin + 4 * i;
+        const int32_t r = word(c ? b[1].w : b[0].w);
+        if (r < 0) {
+            add(b[2 * c], b[2 * c + 1], r);
+            continue;
+        }
+        b = bin + 4 * (int64_t)r;
+        add(b[0], b[1], word(b[0].w));
+        add(b[2], b[3], word(b[1].w));
+    }
+    for (; m < 4; ++m) {
+        for (int a = 0; a < 3; ++a) q[8 * a + m] = 0.0f, q[8 * a + 4 + m] = -FLT_MAX;  // near beyond far on every ray
+        ref[m] = INT32_MIN;  // no child
+    }
+    for (int k = 28; k < 32; ++k) q[k] = 0.0f;
+}
+
+// The entries of all of them on the device: node i has entry index[i], if head is given only where
+// head[i] is set, else where it is not -1.
+cudaError_t gsp_wide_build(const float4* bin, int64_t n, const uint32_t* head, const uint32_t* index, float4* wide);
 
 // Builds the binned-SAH tree and writes its hit/miss links (one set per ray direction
 // class when link_sets == 6). Returns an empty string on success, else an error message.

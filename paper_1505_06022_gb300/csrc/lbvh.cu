@@ -256,46 +256,19 @@ __global__ void k_wide_heads(int n, const int32_t* __restrict__ parent, const in
     head[i] = even ? 1u : 0u;
 }
 
-// The entries of the four-wide tree (layout in wide.cuh), numbered by a scan of the heads: a head's
-// grandchildren, or a child itself where it is a leaf.
-__global__ void k_wide_nodes(int n, const int32_t* __restrict__ left, const int32_t* __restrict__ right,
-                             const int32_t* __restrict__ first, const int32_t* __restrict__ last, int max_leaf,
-                             const Box* __restrict__ box, const uint32_t* __restrict__ head,
-                             const uint32_t* __restrict__ index, float4* __restrict__ wide) {
-    const int i = (int)((int64_t)blockIdx.x * blockDim.x + threadIdx.x);
-    if (i >= n - 1 || !head[i]) return;
-    int ch[4], m = 0;
-    for (int c : {left[i], right[i]}) {
-        if (final_leaf(c, n, first, last, max_leaf)) {
-            ch[m++] = c;
-        } else {
-            ch[m++] = left[c];
-            ch[m++] = right[c];
-        }
-    }
-    float* q = (float*)(wide + 8 * (size_t)index[i]);
-    for (int k = 0; k < 4; ++k) {
-        int32_t ref = INT32_MIN;  // no child
-        if (k < m) {
-            const int c = ch[k];
-            if (c >= n - 1)
-                ref = ~(((c - (n - 1)) << 3) | 1);
-            else if (final_leaf(c, n, first, last, max_leaf))
-                ref = ~((first[c] << 3) | (last[c] - first[c] + 1));
-            else
-                ref = (int32_t)index[c];
-        }
-        for (int a = 0; a < 3; ++a)
-            if (k < m)
-                gsp_wide_box(box[ch[k]].lo[a], box[ch[k]].hi[a], q[8 * a + k], q[8 * a + 4 + k]);
-            else
-                q[8 * a + k] = 0.0f, q[8 * a + 4 + k] = -FLT_MAX;  // near beyond far on every ray
-        q[24 + k] = __int_as_float(ref);
-        q[28 + k] = 0.0f;
-    }
+__global__ void k_wide_entries(const float4* __restrict__ bin, int64_t n, const uint32_t* __restrict__ head,
+                               const uint32_t* __restrict__ index, float4* __restrict__ wide) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n || (head ? !head[i] : index[i] == 0xffffffffu)) return;
+    gsp_wide_entry(bin, i, [&](int32_t j) { return (int32_t)index[j]; }, wide + 8 * (size_t)index[i]);
 }
 
 }  // namespace
+
+cudaError_t gsp_wide_build(const float4* bin, int64_t n, const uint32_t* head, const uint32_t* index, float4* wide) {
+    k_wide_entries<<<nblocks(n), kThreads>>>(bin, n, head, index, wide);
+    return cudaGetLastError();
+}
 
 extern "C" gsp_status gsp_build_bvh_device(gsp_scene* s, int32_t link_sets, int32_t max_leaf, gsp_bvh_stats* stats) {
     if (!s || !s->ctx || (link_sets != 1 && link_sets != 6) || max_leaf < 1 || max_leaf > 7)
@@ -418,7 +391,7 @@ extern "C" gsp_status gsp_build_bvh_device(gsp_scene* s, int32_t link_sets, int3
     k_padding<<<1, 32>>>(link_sets, nfinal, stride, d_nodes);
     k_leaf_tris<<<nblocks(nt), kThreads>>>(d_verts, d_tris, ids, nt, d_tri4);
     k_child_pairs<<<nblocks(n), kThreads>>>(n, left, right, parent, first, last, max_leaf, box, d_bin);
-    if (nwide) k_wide_nodes<<<nblocks(n - 1), kThreads>>>(n, left, right, first, last, max_leaf, box, head, windex, d_wide);
+    if (nwide) gsp_wide_build(d_bin, n - 1, head, windex, d_wide);
     cudaEventRecord(ev[2]);
     e = cudaEventSynchronize(ev[2]);
     if (e == cudaSuccess) e = cudaGetLastError();

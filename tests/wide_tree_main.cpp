@@ -28,12 +28,15 @@ static int check(const std::vector<float>& v, const std::vector<int32_t>& t, int
     const int nt = (int)t.size() / 3;
     HostBVH b;
     CHECK(bvh_build_host(v.data(), (int64_t)v.size() / 3, t.data(), nt, gsp_bvh_params{16, 4, 7, 6}, b).empty());
-    const int64_t nw = (int64_t)b.wide.size() / 8;
+    const int64_t nw = b.nwide;
+    std::vector<float4> wide((size_t)nw * 8);
+    for (int64_t i = 0; i < (int64_t)b.wide_of.size(); ++i)
+        if (b.wide_of[i] >= 0) gsp_wide_entry(b.bin.data(), i, [&](int32_t j) { return b.wide_of[j]; }, &wide[8 * b.wide_of[i]]);
     if (b.nnodes == 1) {
         CHECK(nw == 0);
         return 0;
     }
-    const float* W = (const float*)b.wide.data();
+    const float* W = (const float*)wide.data();
     std::vector<int> tri_seen(nt, 0), node_seen(nw, 0);
     node_seen[0] = 1;
     for (int64_t i = 0; i < nw; ++i)
