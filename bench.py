@@ -8,7 +8,8 @@ Default workload (one line of JSON on rank 0):
   * "e2e": the same rays through gsp_trace_closest_hit_host from pinned host memory (the
     host->device transfer of the rays and the device->host copy of the hits inside the timed
     region).
-  * "traversal_fig4": MTBVH vs TBVH vs stack traversal (Fig. 4) and the device BVH build.
+  * "traversal_fig4": MTBVH vs TBVH vs stack traversal (Fig. 4), the four-wide form of the tree that
+    closest-hit calls walk by default, and the device BVH build.
   * "sppm_512": SPPM passes/s at 512x512 on a 247,234-triangle scene with 1M photon paths/pass
     (a 64-pass render; default and autotuned settings).
   * "sppm_512_shaded": the 512x512 render with per-vertex normals, texture coordinates and albedo
@@ -224,7 +225,7 @@ def run_ours(args, world, rank, local):
         step()
     torch.cuda.synchronize()
     ctx.sync()
-    # the library brackets each timed step's k_trace launch with a pair of events made here
+    # the library brackets each timed step's traversal launch with a pair of events made here
     gsp.gsp_trace_time_launches(scene.h, args.steps)
     clocks = ClockSampler(local)
     if pg:
@@ -358,7 +359,8 @@ def fp32_peak_tflops(sm_count, peaks):
 
 def traversal_roofline(v_node, v_tri, n, ms, call_ms, sm_count, peaks, tiers):
     """The bench line's roofline block for closest hit: algorithmic bytes and flops of n rays with
-    v_node node visits and v_tri triangle tests per ray, against the traversal kernel's mean launch
+    v_node node visits and v_tri triangle tests per ray (of the hit/miss links' walk, whichever form of
+    the tree the kernel walks), against the traversal kernel's mean launch
     time `ms` (call_ms: the whole call, with the counter reset and the refinement of flagged hits)."""
     bytes_ray = BYTES_PER_NODE * v_node + BYTES_PER_TRI * v_tri + BYTES_PER_RAY_IO
     flops_ray = FLOPS_PER_NODE * v_node + FLOPS_PER_TRI * v_tri
@@ -376,7 +378,7 @@ def traversal_roofline(v_node, v_tri, n, ms, call_ms, sm_count, peaks, tiers):
             "unit": "GB/s", "frac": round(achieved / hbm, 4), "traffic": None, "peak_source": hbm_src,
             "roofline_ms": round(1000 * max(t_hbm, t_flop), 4), "kernel_ms": round(ms, 4),
             "call_ms": round(call_ms, 4),
-            "kernel_timing": "mean over the timed steps of k_trace's own launch: CUDA events that the library "
+            "kernel_timing": "mean over the timed steps of the traversal kernel's own launch: CUDA events that the library "
                              "records on the call's stream right before and after it (gsp_trace_time_launches)",
             "l2": {"peak": l2, "frac": round(achieved / l2, 4), "unit": "GB/s",
                    "source": "gsp_measure_read_bandwidth, buffers of 32 and 48 MB resident in L2"},
@@ -661,7 +663,8 @@ def bench_grad(args, ctx, dev, stream, rl):
 def bench_traversals(args, ctx, dev, stream, sc, scene, rays):
     """Fig. 4's comparison on the closest-hit workload: the multiple-threaded BVH (6 link sets),
     the original threaded BVH (1 link set, one fixed order) and a stack-based near-first
-    traversal of the same SAH tree, each on all rays and on the coherent and random halves."""
+    traversal of the same SAH tree, and the tree's four-wide form, each on all rays and on the
+    coherent and random halves. A step limit that no ray reaches has a scene walk its links."""
     import torch
     from paper_1505_06022_gb300 import gsp
     n = rays.shape[0]
@@ -673,13 +676,17 @@ def bench_traversals(args, ctx, dev, stream, sc, scene, rays):
     tt = torch.empty(n, dtype=torch.float32, device=dev)
     parts = {"all": (0, n), "coherent": (0, n // 2), "random": (n // 2, n)}
     kinds = {"mtbvh": (scene, gsp.gsp_trace_closest_hit), "tbvh": (tbvh, gsp.gsp_trace_closest_hit),
-             "stack": (scene, gsp.gsp_trace_closest_hit_stack),
+             "stack": (scene, gsp.gsp_trace_closest_hit_stack), "four_wide": (scene, gsp.gsp_trace_closest_hit),
              "mtbvh_on_device_lbvh": (lbvh, gsp.gsp_trace_closest_hit),
-             "stack_on_device_lbvh": (lbvh, gsp.gsp_trace_closest_hit_stack)}
+             "stack_on_device_lbvh": (lbvh, gsp.gsp_trace_closest_hit_stack),
+             "four_wide_on_device_lbvh": (lbvh, gsp.gsp_trace_closest_hit)}
     reps = max(3, min(args.steps, 30))
     out = {}
     for kind, (scn, fn) in kinds.items():
         out[kind] = {}
+        links = "mtbvh" in kind or kind == "tbvh"
+        if links:
+            gsp.gsp_scene_set_step_limit(scn.h, 2**31 - 1)
         for part, (a, b) in parts.items():
             r, o1, o2 = rays[a:b], tri[a:b], tt[a:b]
             for _ in range(2):
@@ -692,6 +699,8 @@ def bench_traversals(args, ctx, dev, stream, sc, scene, rays):
             torch.cuda.synchronize()
             ms = e0.elapsed_time(e1) / reps
             out[kind][part] = round((b - a) / (ms / 1000.0) / 1e6, 1)
+        if links:
+            gsp.gsp_scene_set_step_limit(scn.h, 0)
     ctx.sync()
     tbvh.close()
     out["mtbvh_over_tbvh"] = {p: round(out["mtbvh"][p] / out["tbvh"][p], 3) for p in parts}

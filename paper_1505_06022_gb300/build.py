@@ -47,9 +47,9 @@ def _digest() -> str:
     return h.hexdigest()
 
 
-# Everything the closest-hit kernel (k_trace, k_refine) is compiled from: a change elsewhere in the
+# Everything the closest-hit kernel (k_trace_wide, k_refine) is compiled from: a change elsewhere in the
 # library leaves its profile counters valid.
-TRACE_SOURCES = ["capi.cu", "devcommon.cuh", "launch.h", "persist.cuh", "gsp_internal.h"]
+TRACE_SOURCES = ["capi.cu", "devcommon.cuh", "launch.h", "persist.cuh", "wide.cuh", "gsp_internal.h"]
 
 
 def trace_digest() -> str:
