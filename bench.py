@@ -385,6 +385,7 @@ def traversal_roofline(v_node, v_tri, n, ms, call_ms, sm_count, peaks, tiers):
             "fp32": {"achieved": round(flops_ray * n / s / 1e12, 3), "peak": round(fp32, 2), "unit": "TFLOP/s",
                      "frac": round(flops_ray * n / s / 1e12 / fp32, 4),
                      "source": f"{sm_count} SMs x 128 FP32 lanes x 2 (FMA) x {sm_max:.0f} MHz"},
+            "model": "bytes and operations of the hit/miss links' walk",
             "node_visits_per_ray": round(v_node, 3), "tri_tests_per_ray": round(v_tri, 3),
             "algorithmic_bytes_per_ray": round(bytes_ray, 1), "flops_per_ray": round(flops_ray, 1),
             "algorithmic_bytes_per_launch": int(round(bytes_ray * n)), "tiers": tiers}

@@ -264,8 +264,6 @@ __global__ void k_zero_u64x2(unsigned long long* p) {
     p[1] = 0ull;
 }
 
-__global__ void k_zero_u64(unsigned long long* p) { *p = 0ull; }
-
 // out[k * ndraw + j] = draw j of stream (seed, scene, domain, pass, ids[k])
 __global__ void k_rng_fill(uint64_t seed, uint32_t scene, uint32_t domain, uint32_t pass,
                            const uint64_t* __restrict__ ids, int64_t n, int32_t ndraw, float* __restrict__ out) {

@@ -35,7 +35,7 @@ struct HostBVH {
 };
 
 // Centre and half extent of an interval of the four-wide tree's boxes: c - h <= lo and hi <= c + h
-// with h widened by kWideGrow (1 + 2^-19; wide.cuh says what that covers). lo <= hi.
+// with h widened by the factor 1 + 2^-19 (wide.cuh says what that covers). lo <= hi.
 #ifdef __CUDACC__
 __host__ __device__
 #endif

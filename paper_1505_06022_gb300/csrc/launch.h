@@ -31,7 +31,6 @@ constexpr int kTraceInner = GSP_TRACE_INNER;           // traversal steps betwee
 constexpr int kTraceLeafBatch = GSP_TRACE_LEAF_BATCH;  // pending leaves that trigger a warp-wide leaf test
 constexpr int kWideStack = 64;     // children a walk of the four-wide tree may keep (at most three per wide level)
 constexpr int kWideMaxDepth = 38;  // depth of the binary tree up to which that is enough
-constexpr float kWideGrow = 1.0f + 0x1p-19f;  // half extents of its boxes are widened by this factor (wide.cuh)
 constexpr float kWideMaxExtent = 1e8f;  // larger scenes: (c - o) / d could overflow for a tiny d inside a box
 constexpr int kPathChunk = GSP_PATH_CHUNK;  // paths a warp of the path kernels takes at once (a block's
                                             // grid share is 128 paths: every warp of a short launch gets some)

@@ -14,9 +14,11 @@
 // copies of the nodes; the wide form makes 13 node fetches for the same ray from one copy (20 MB
 // instead of 123 MB for a million triangles, so that it stays in L2). Four children rather than
 // eight: eight would make 9 fetches but test 72 boxes for 52, and the trees fill 3.1 of 4 slots but
-// 3.4 of 8. Measured against the links: 4,194,304 rays over 1,003,520 triangles 815 -> 596 us,
-// 262,147 rays over 247,234 triangles 138 -> 86 us, 1,021 rays 64 -> 24 us (with the last ray of a
-// warp walked by all lanes, below), a 512x512 pass 1.30 -> 1.00 ms, a 131x97 one 752 -> 430 us.
+// 3.4 of 8. Measured against the links when it came: 4,194,304 rays over 1,003,520 triangles 815 -> 596 us,
+// 262,147 rays over 247,234 triangles 138 -> 86 us, 1,021 rays 64 -> 24 us (with the last ray of a warp
+// walked by all lanes, below), a 512x512 pass 1.30 -> 1.00 ms, a 131x97 one 752 -> 430 us. With what
+// followed (four lanes to a ray at the end, the stack's upper entries in shared memory, fewer launches,
+// path pools): 570, 67 and 18 us, 0.82 ms and 252 us.
 #pragma once
 
 #include "launch.h"
@@ -41,7 +43,7 @@ constexpr int kWideLeafBatch = GSP_WIDE_LEAF_BATCH;  // lanes at a leaf that tri
 
 // Slab interval of the box c +- h along one axis: tc = (c - o) inv, tc -+ h |inv|. With unit
 // roundoff u and an inverse good to 2u, either end is off by at most 5u |tc| + 3u h |inv|. Where
-// |tc| <= 2 h |inv| that is below the 32u h |inv| by which the builders widen h (kWideGrow); else
+// |tc| <= 2 h |inv| that is below the 32u h |inv| by which gsp_wide_box widens h; else
 // both ends have the sign of tc and a relative error of at most 13u, which the far end's factor
 // kWideFar = 1 + 32u covers. The test is conservative then, for t >= 0; for a negative tmin the
 // pad adds 64u |tmin|, more than the factor takes off a negative far end. Two operations of the
