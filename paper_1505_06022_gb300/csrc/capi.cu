@@ -173,8 +173,11 @@ k_refine(DevScene S, const float4* __restrict__ rays, const int2* __restrict__ r
 }
 
 // Closest hit through the four-wide form of the tree (wide.cuh): the kernel of scenes that have
-// one, with k_trace's work distribution and outputs. LIST: hits for FP64 re-evaluation go to k_trace's
-// list; otherwise a warp collects its own and re-evaluates them 32 at a time.
+// one, with k_trace's work distribution and outputs. A warp takes chunks of 32 rays, half of k_trace's:
+// with four box tests a fetch a ray is over sooner, and shorter chunks keep the warps of an SM in one
+// part of the tree (4,194,304 rays 622 -> 572 us, 1,024,000 over a triangle soup 319 -> 290, 4,194,304 over
+// 247,234 triangles 310 -> 304; 24 rays 575 and 322, 16 rays 584 and 342). LIST: hits for FP64
+// re-evaluation go to k_trace's list; otherwise a warp collects its own and re-evaluates them 32 at a time.
 template <bool LIST>
 __global__ void __launch_bounds__(kTraceThreads, GSP_WIDE_MIN_BLOCKS)
 k_trace_wide(DevScene S, const float4* __restrict__ rays, int64_t n, const uint32_t* __restrict__ d_n,
@@ -223,7 +226,7 @@ k_trace_wide(DevScene S, const float4* __restrict__ rays, int64_t n, const uint3
         } else if (quad)
             quad_steps<GSP_WIDE_KEEP_TRACE>(S.wide, S.tris, st, w, stk, ray >= 0);
         else
-            wide_steps(S.wide, S.tris, st, w, stk, ray >= 0, GSP_WIDE_KEEP_TRACE);
+            wide_steps(S.wide, S.tris, st, w, stk, ray >= 0, LIST ? GSP_WIDE_KEEP_LONG : GSP_WIDE_KEEP_TRACE);
         const bool fin = ray >= 0 && w.cur == kWalkDone;
         bool flag = false;
         if (fin && (!quad || (lane & 3) == 0)) {
@@ -306,7 +309,7 @@ static void run_trace(const gspd::DevScene& S, int device, const float4* rays, i
     const int links_grid = gsp_trace_grid(device);
     constexpr int kWarps = kTraceThreads / 32;
     const int64_t wide_grid = std::min<int64_t>(trace_wide_grid(device), (n + kWarps - 1) / kWarps);
-    const int chunk = gsp_chunk(n, wide_grid * kWarps, kTraceChunk);
+    const int chunk = gsp_chunk(n, wide_grid * kWarps, GSP_WIDE_CHUNK);
     const bool list = refine_factor < INFINITY && !(S.wide && n <= GSP_REFINE_INLINE * wide_grid * kWarps);
     if (zero && (list || !S.wide || chunk * wide_grid * kWarps < n)) gspd::k_zero_u64x2<<<1, 1, 0, st>>>(ctr);
     if (e0) cudaEventRecord(e0, st);

@@ -33,6 +33,12 @@
 #ifndef GSP_WIDE_TOP_TRACE
 #define GSP_WIDE_TOP_TRACE 12
 #endif
+#ifndef GSP_WIDE_KEEP_LONG
+#define GSP_WIDE_KEEP_LONG 3
+#endif
+#ifndef GSP_WIDE_CHUNK
+#define GSP_WIDE_CHUNK 32
+#endif
 #ifndef GSP_WIDE_LEAF_BATCH
 #define GSP_WIDE_LEAF_BATCH 12
 #endif
@@ -180,8 +186,10 @@ __device__ __forceinline__ void wide_node(const float4* __restrict__ nodes, cons
 
 // Walks the warp's active lanes until no more than `keep` quarters of them still walk: what follows a
 // walk then runs for many lanes at once. A path kernel's shading is long (1 of 4; 8.0 ms per eight
-// 512x512 passes, against 8.07 with 2 and 8.33 with 3), a ray's end in the closest-hit kernel short
-// (2; 3 costs 1 %, 1 costs 8 %). Lanes at a leaf wait until kWideLeafBatch of them are, or no lane
+// 512x512 passes, against 8.07 with 2 and 8.33 with 3), a ray's end in the closest-hit kernel short:
+// 3 in calls that list hits for refinement (4,194,304 rays 574 us, 572 with 3; random ones alone 474 and
+// 463), 2 in shorter ones, which end sooner (262,147 rays 67.4 us, 68.1 with 3).
+// Lanes at a leaf wait until kWideLeafBatch of them are, or no lane
 // has a node left to test, and test their leaves together (12; 8 costs 1-2 %, 4 costs 5 %).
 template <class Stack>
 __device__ __forceinline__ void wide_steps(const float4* __restrict__ wide, const float4* __restrict__ tris, WideRay& st,
