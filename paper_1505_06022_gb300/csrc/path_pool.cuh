@@ -19,8 +19,10 @@
 
 #include "sppm_paths.cuh"
 
-#ifndef GSP_POOL  // paths a warp keeps (64: the same but for 5.39 against 5.26 ms in the batch; 96 slower)
-#define GSP_POOL 48
+// Paths a warp keeps. More leave the L1 cache less: 48 against 44: a 131x97 pass 251.5 against 248.0 us, the
+// batch 5.18 against 5.13 ms, one bounce per pass 1.186 against 1.172 ms; 36: batch 5.20; 64: 5.39 (of 5.26 then).
+#ifndef GSP_POOL
+#define GSP_POOL 44
 #endif
 // Resident blocks per SM: 72 registers without spills (8: 1 % slower, 6: 1 % faster in the batch, 1 %
 // slower at 512x512); with shading data 96 (6 spill: 1.50 against 1.41 ms).
