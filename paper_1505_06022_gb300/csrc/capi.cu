@@ -183,7 +183,7 @@ __global__ void __launch_bounds__(kTraceThreads, GSP_WIDE_MIN_BLOCKS)
 k_trace_wide(DevScene S, const float4* __restrict__ rays, int64_t n, const uint32_t* __restrict__ d_n,
              int32_t* __restrict__ tri, float* __restrict__ tout, float2* __restrict__ uv,
              unsigned long long* __restrict__ ctr, int2* __restrict__ rlist, float refine_factor, int32_t out_slot,
-             int32_t chunk) {
+             int32_t chunk, int32_t keep) {
     wait_previous();
     if (d_n) n = min(n, (int64_t)*d_n);
     const int lane = threadIdx.x & 31;
@@ -226,7 +226,7 @@ k_trace_wide(DevScene S, const float4* __restrict__ rays, int64_t n, const uint3
         } else if (quad)
             quad_steps<GSP_WIDE_KEEP_TRACE>(S.wide, S.tris, st, w, stk, ray >= 0);
         else
-            wide_steps(S.wide, S.tris, st, w, stk, ray >= 0, LIST ? GSP_WIDE_KEEP_LONG : GSP_WIDE_KEEP_TRACE);
+            wide_steps(S.wide, S.tris, st, w, stk, ray >= 0, keep);
         const bool fin = ray >= 0 && w.cur == kWalkDone;
         bool flag = false;
         if (fin && (!quad || (lane & 3) == 0)) {
@@ -305,7 +305,8 @@ static int trace_wide_grid(int device) {
 // a kernel uses them; the wide kernel without a list uses none when each warp's first chunk covers n.
 static void run_trace(const gspd::DevScene& S, int device, const float4* rays, int64_t n, const uint32_t* d_n,
                       int32_t* tri, float* t, float2* uv, unsigned long long* ctr, int2* rlist, float refine_factor,
-                      int32_t out_slot, bool zero, cudaStream_t st, cudaEvent_t e0 = nullptr, cudaEvent_t e1 = nullptr) {
+                      int32_t out_slot, bool zero, cudaStream_t st, cudaEvent_t e0 = nullptr, cudaEvent_t e1 = nullptr,
+                      bool host = false) {
     const int links_grid = gsp_trace_grid(device);
     constexpr int kWarps = kTraceThreads / 32;
     const int64_t wide_grid = std::min<int64_t>(trace_wide_grid(device), (n + kWarps - 1) / kWarps);
@@ -316,7 +317,7 @@ static void run_trace(const gspd::DevScene& S, int device, const float4* rays, i
     if (S.wide) {
         auto* const kernel = list ? gspd::k_trace_wide<true> : gspd::k_trace_wide<false>;
         gsp_launch_after(kernel, wide_grid, kTraceThreads, st, S, rays, n, d_n, tri, t, uv, ctr, rlist, refine_factor,
-                         out_slot, chunk);
+                         out_slot, chunk, list && !host ? GSP_WIDE_KEEP_LONG : GSP_WIDE_KEEP_TRACE);
     } else
         gspd::k_trace<<<links_grid, kTraceThreads, 0, st>>>(S, rays, n, d_n, tri, t, uv, ctr, rlist, refine_factor,
                                                             out_slot);
@@ -328,13 +329,14 @@ static void run_trace(const gspd::DevScene& S, int device, const float4* rays, i
 
 // One closest-hit call on device buffers: the traversal and the FP64 refinement of the flagged hits.
 // ctr (2 u64) and rlist (n entries) belong to this call's stream.
-// With e0 and e1 (gsp_trace_time_launches), the two events bracket the traversal launch alone.
+// With e0 and e1 (gsp_trace_time_launches), the two events bracket the traversal launch alone. host: the
+// rays are read over the link.
 static void launch_trace(const gsp_scene* s, const float4* rays, int64_t n, int32_t* tri, float* t, float2* uv,
                          unsigned long long* ctr, int2* rlist, cudaStream_t st, cudaEvent_t e0 = nullptr,
-                         cudaEvent_t e1 = nullptr) {
+                         cudaEvent_t e1 = nullptr, bool host = false) {
     NvtxRange nvtx("gsp: closest hit");
     run_trace(gsp_dev_scene(s), s->ctx->device, rays, n, nullptr, tri, t, uv, ctr, rlist, GSP_REFINE_FACTOR, 0, true, st,
-              e0, e1);
+              e0, e1, host);
 }
 
 cudaError_t gsp_trace_queue(const gsp_scene* s, const float4* rays, int64_t max_n, const uint32_t* d_n, int32_t* tri,
@@ -911,7 +913,8 @@ gsp_status gsp_trace_closest_hit_host(gsp_scene* s, const float* h_rays, int64_t
             const int64_t off = k * per, m = std::min(per, n - off);
             if (m <= 0) break;
             auto& L = s->lanes[k];
-            launch_trace(s, m_rays + 2 * off, m, L.d_tri, L.d_t, h_uv ? L.d_uv : nullptr, L.d_ctr, L.d_rlist, L.st);
+            launch_trace(s, m_rays + 2 * off, m, L.d_tri, L.d_t, h_uv ? L.d_uv : nullptr, L.d_ctr, L.d_rlist, L.st,
+                         nullptr, nullptr, true);
             GSP_CUDA_TRY(cudaMemcpyAsync(h_tri + off, L.d_tri, (size_t)m * 4, cudaMemcpyDeviceToHost, L.st));
             GSP_CUDA_TRY(cudaMemcpyAsync(h_t + off, L.d_t, (size_t)m * 4, cudaMemcpyDeviceToHost, L.st));
             if (h_uv)
