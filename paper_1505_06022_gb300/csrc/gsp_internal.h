@@ -5,7 +5,9 @@
 #include <cuda_runtime.h>
 
 #include <cfloat>
+#include <cmath>
 #include <cstdint>
+#include <cstring>
 #include <string>
 #include <vector>
 
@@ -34,12 +36,31 @@ struct HostBVH {
     double build_ms = 0, thread_ms = 0;
 };
 
+#ifdef __CUDACC__
+#define GSP_HOST_DEVICE __host__ __device__
+#else
+#define GSP_HOST_DEVICE
+#endif
+
+// The far end x of an interval of box distances, moved out by 2^-19 of its size: what the rounding of a
+// box test is covered by (wide.cuh). The slack follows the sign of x, which a factor would not, and is
+// relative, so that it is as good behind the origin (a negative tmin) as in front of it; +inf stays, and
+// -inf gives a NaN, which no entry distance is at or below.
+GSP_HOST_DEVICE inline float gsp_reach(float x) { return x + fabsf(x) * 0x1p-19f; }
+
+// Whether a child of the four-wide tree put by with this key (its entry distance, the two low bits
+// replaced; wide.cuh) may still hold a closer hit. Dropping the low bits rounds a distance down unless it
+// is negative (negative tmin, origin inside the box): never culled then.
+GSP_HOST_DEVICE inline bool gsp_wide_keep(int32_t key, float tbest) {
+    const int32_t bits = key & ~3;
+    float t;
+    memcpy(&t, &bits, sizeof t);
+    return key < 0 || t <= tbest;
+}
+
 // Centre and half extent of an interval of the four-wide tree's boxes: c - h <= lo and hi <= c + h
 // with h widened by the factor 1 + 2^-19 (wide.cuh says what that covers). lo <= hi.
-#ifdef __CUDACC__
-__host__ __device__
-#endif
-inline void gsp_wide_box(float lo, float hi, float& c, float& h) {
+GSP_HOST_DEVICE inline void gsp_wide_box(float lo, float hi, float& c, float& h) {
     c = 0.5f * lo + 0.5f * hi;
     const float a = hi - c, b = c - lo;  // each within one rounding (2^-24) of the exact value
     h = (a > b ? a : b) * (1.0f + 0x1p-19f + 0x1p-22f);
@@ -48,10 +69,7 @@ inline void gsp_wide_box(float lo, float hi, float& c, float& h) {
 // The entry of the four-wide tree (layout in wide.cuh) of node i of the child pairs: the boxes of its
 // grandchildren, or a child's own where that is a leaf. of(j) is the entry of node j.
 template <class Of>
-#ifdef __CUDACC__
-__host__ __device__
-#endif
-inline void gsp_wide_entry(const float4* bin, int64_t i, Of of, float4* entry) {
+GSP_HOST_DEVICE inline void gsp_wide_entry(const float4* bin, int64_t i, Of of, float4* entry) {
     float* q = (float*)entry;
     int32_t* ref = (int32_t*)entry + 24;
     int m = 0;
@@ -74,7 +92,7 @@ inline void gsp_wide_entry(const float4* bin, int64_t i, Of of, float4* entry) {
     }
     for (; m < 4; ++m) {
         for (int a = 0; a < 3; ++a) q[8 * a + m] = 0.0f, q[8 * a + 4 + m] = -FLT_MAX;  // near beyond far on every ray
-        ref[m] = INT32_MIN;  // no child
+        ref[m] = ~0;  // a leaf of no triangles
     }
     for (int k = 28; k < 32; ++k) q[k] = 0.0f;
 }

@@ -154,7 +154,7 @@ k_paths_pool(const __grid_constant__ PathJob one, const PathJob* __restrict__ jo
     }
     __syncwarp();
     int nready = 0, ndone = pool;
-    WideRay st;
+    PathRay st;
     WideWalk w;
     int2 deep[kWideStack];
     const WideStack<0> stk{deep, nullptr};
@@ -178,7 +178,6 @@ k_paths_pool(const __grid_constant__ PathJob one, const PathJob* __restrict__ jo
                     tris = J.S.tris;
                 }
                 wide_ray(o, d, path_tmin(pl.meta[at], J.P.eps), __int_as_float(0x7f800000), st);
-                st.pad = 0.0f;  // tmin >= 0
                 wide_init(w);
             }
             nready = max(nready - __popc(idle), 0);
@@ -299,7 +298,6 @@ k_paths_pool(const __grid_constant__ PathJob one, const PathJob* __restrict__ jo
             if (pool_shade<SHADE, REGEN>(J, id, st.slot, st.tbest, o, d, v, rng, meta, lead)) {
                 if (lead) pl.put_state(at, v, rng, meta);
                 wide_ray(o, d, J.P.eps, __int_as_float(0x7f800000), st);
-                st.pad = 0.0f;
                 wide_init(w);
             } else {
                 at = -1;

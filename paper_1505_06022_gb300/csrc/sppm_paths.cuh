@@ -308,7 +308,7 @@ struct PathWalk<kStack> {
 
 template <>
 struct PathWalk<kWide> {
-    WideRay st;
+    PathRay st;
     WideWalk w;
     int2 stk[kWideStack];
     __device__ __forceinline__ PathWalk() {
@@ -318,7 +318,6 @@ struct PathWalk<kWide> {
     }
     __device__ __forceinline__ void start(const DevScene&, float3 o, float3 d, float tmin) {
         wide_ray(o, d, tmin, __int_as_float(0x7f800000), st);
-        st.pad = 0.0f;  // tmin >= 0
         wide_init(w);
     }
     __device__ __forceinline__ void steps(const DevScene& S, bool active, int32_t, uint32_t&) {

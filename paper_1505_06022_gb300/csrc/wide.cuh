@@ -5,9 +5,11 @@
 // child that is a leaf stands for itself): their boxes as centres and half extents, plane by
 // plane, and a reference per child -- eight float4, 128 bytes, one cache line:
 //   {c.x}x4 {h.x}x4 | {c.y}x4 {h.y}x4 | {c.z}x4 {h.z}x4 | {ref}x4, unused
-// ref >= 0 is a wide node, < 0 is ~(leaf word), kWalkDone no child. Leaves are the binary tree's,
-// and the hit is the lexicographic (t, index) minimum of the same triangle tests, so the result
-// does not depend on the form walked.
+// ref >= 0 is a wide node, < 0 is ~(leaf word); an absent child is a leaf of no triangles behind a box
+// that no ray meets unless its distances overflow on every axis (an origin at 1e10 with a direction of
+// length 1e-29, an infinite direction), so that a walk which goes there goes on after it. Leaves are the
+// binary tree's, and the hit is the lexicographic (t, index) minimum of the same triangle tests, so the
+// result does not depend on the form walked.
 //
 // What bounds a walk is the chain of dependent node fetches and the instructions per box. The links
 // visit 53 boxes for a bounce ray of the 247,234-triangle scene (two per fetch at best) and need six
@@ -50,16 +52,18 @@ constexpr int kWideLeafBatch = GSP_WIDE_LEAF_BATCH;  // lanes at a leaf that tri
 // Slab interval of the box c +- h along one axis: tc = (c - o) inv, tc -+ h |inv|. With unit
 // roundoff u and an inverse good to 2u, either end is off by at most 5u |tc| + 3u h |inv|. Where
 // |tc| <= 2 h |inv| that is below the 32u h |inv| by which gsp_wide_box widens h; else
-// both ends have the sign of tc and a relative error of at most 13u, which the far end's factor
-// kWideFar = 1 + 32u covers. The test is conservative then, for t >= 0; for a negative tmin the
-// pad adds 64u |tmin|, more than the factor takes off a negative far end. Two operations of the
-// half-rate min/max pipe fewer per axis and box than min and max over the two planes: that pipe
-// was the busiest at 57-61 % of its cycles.
-constexpr float kWideFar = 1.0f + 0x1p-19f;
+// both ends have the sign of tc and a relative error of at most 13u, which gsp_reach's 32u cover: the
+// test is conservative on both sides of the origin. (A pad of 64u |tmin| for negative tmin, which this
+// once had, lets every box through when |tmin| is large against the scene: 683 instead of 14 nodes per
+// line through 2,000 triangles at tmin = -FLT_MAX.) Two operations of the half-rate min/max pipe fewer
+// per axis and box than min and max over the two planes: that pipe was the busiest at 57-61 % of its cycles.
+struct WideRay : RayHit {};
+// A path's ray, whose tmin is not negative: one product does (an FMA has no absolute value of its own; two
+// operations per box instead of one: 4,194,304 rays 575 -> 581 us, the batch of 16 scenes 5.11 -> 5.14 ms).
+struct PathRay : RayHit {};
 
-struct WideRay : RayHit {
-    float pad;
-};
+__device__ __forceinline__ float wide_far(const WideRay&, float x) { return gsp_reach(x); }
+__device__ __forceinline__ float wide_far(const PathRay&, float x) { return __fmul_rn(x, 1.0f + 0x1p-19f); }
 
 // 1 / d to 1 ulp (2u): all that the slab test needs.
 __device__ __forceinline__ float wide_inv(float d) {
@@ -68,7 +72,7 @@ __device__ __forceinline__ float wide_inv(float d) {
     return r;
 }
 
-__device__ __forceinline__ void wide_ray(float3 o, float3 d, float tmin, float tmax, WideRay& st) {
+__device__ __forceinline__ void wide_ray(float3 o, float3 d, float tmin, float tmax, RayHit& st) {
     st.o = o;
     st.d = d;
     st.inv = make_float3(wide_inv(d.x), wide_inv(d.y), wide_inv(d.z));
@@ -76,7 +80,6 @@ __device__ __forceinline__ void wide_ray(float3 o, float3 d, float tmin, float t
     st.tbest = tmax;
     st.best = -1;
     st.slot = -1;
-    st.pad = fmaxf(-tmin, 0.0f) * 0x1p-18f;
 }
 
 // One ray's walk: the node or leaf it is at (kWalkDone: the walk is over) and the children still
@@ -117,31 +120,26 @@ __device__ __forceinline__ void wide_init(WideWalk& w) {
 
 constexpr int32_t kWideMiss = 0x7fffffff;  // sorts behind every key
 
-// Whether a child with this key may still hold a closer hit. Dropping the low bits rounds a
-// distance down unless it is negative (negative tmin, origin inside the box): never culled then.
-__device__ __forceinline__ bool wide_keep(int32_t key, float tbest) {
-    return key < 0 || __int_as_float(key & ~3) <= tbest;
-}
-
 template <class Stack>
 __device__ __forceinline__ int32_t wide_pop(const RayHit& st, WideWalk& w, const Stack& stk) {
     while (w.sp > 0) {
         const int2 e = stk.get(--w.sp);
-        if (wide_keep(e.x, st.tbest)) return e.y;
+        if (gsp_wide_keep(e.x, st.tbest)) return e.y;
     }
     return kWalkDone;
 }
 
 // Key of child i: the bits of its entry distance with the child number in the two low bits, or
 // kWideMiss. Signed order is the order of the distances where they are not negative.
-__device__ __forceinline__ int32_t wide_key(const WideRay& st, float cx, float hx, float cy, float hy, float cz,
+template <class Ray>
+__device__ __forceinline__ int32_t wide_key(const Ray& st, float cx, float hx, float cy, float hy, float cz,
                                             float hz, int i) {
     const float tx = __fmul_rn(cx - st.o.x, st.inv.x), ty = __fmul_rn(cy - st.o.y, st.inv.y),
                 tz = __fmul_rn(cz - st.o.z, st.inv.z);
     const float ax = fabsf(st.inv.x), ay = fabsf(st.inv.y), az = fabsf(st.inv.z);
     const float tn = max3f(__fmaf_rn(-hx, ax, tx), __fmaf_rn(-hy, ay, ty), fmaxf(__fmaf_rn(-hz, az, tz), st.tmin));
     const float tf = min3f(__fmaf_rn(hx, ax, tx), __fmaf_rn(hy, ay, ty), __fmaf_rn(hz, az, tz));
-    return tn <= __fmaf_rn(fminf(st.tbest, tf), kWideFar, st.pad) ? ((__float_as_int(tn) & ~3) | i) : kWideMiss;
+    return tn <= wide_far(st, fminf(st.tbest, tf)) ? ((__float_as_int(tn) & ~3) | i) : kWideMiss;
 }
 
 template <class Stack>
@@ -168,8 +166,8 @@ __device__ __forceinline__ void wide_next(int32_t k0, int32_t k1, int32_t k2, in
 }
 
 // Tests the four children of node w.cur and moves on.
-template <class Stack>
-__device__ __forceinline__ void wide_node(const float4* __restrict__ nodes, const WideRay& st, WideWalk& w,
+template <class Ray, class Stack>
+__device__ __forceinline__ void wide_node(const float4* __restrict__ nodes, const Ray& st, WideWalk& w,
                                           const Stack& stk) {
     const float4* p = nodes + 8 * (int64_t)w.cur;
     float4 cx, hx, cy, hy, cz, hz;
@@ -192,8 +190,8 @@ __device__ __forceinline__ void wide_node(const float4* __restrict__ nodes, cons
 // the link (4,194,304 of them 4,607 Mrays/s, 4,514 with 3).
 // Lanes at a leaf wait until kWideLeafBatch of them are, or no lane
 // has a node left to test, and test their leaves together (12; 8 costs 1-2 %, 4 costs 5 %).
-template <class Stack>
-__device__ __forceinline__ void wide_steps(const float4* __restrict__ wide, const float4* __restrict__ tris, WideRay& st,
+template <class Ray, class Stack>
+__device__ __forceinline__ void wide_steps(const float4* __restrict__ wide, const float4* __restrict__ tris, Ray& st,
                                            WideWalk& w, const Stack& stk, bool active, int keep) {
     const int stop = (__popc(__ballot_sync(0xffffffffu, active)) * keep) >> 2;
     uint32_t nm, lm;
@@ -235,7 +233,7 @@ __device__ __forceinline__ float3 shfl3(float3 v, int src) {
 
 // Copies lane src's walk to this lane (every lane calls it; src: a lane, its own if it has no use).
 template <class Stack>
-__device__ __forceinline__ void quad_take(WideRay& st, WideWalk& w, const Stack& stk, int src) {
+__device__ __forceinline__ void quad_take(RayHit& st, WideWalk& w, const Stack& stk, int src) {
     const uint32_t F = 0xffffffffu;
     st.o = shfl3(st.o, src);
     st.d = shfl3(st.d, src);
@@ -244,7 +242,6 @@ __device__ __forceinline__ void quad_take(WideRay& st, WideWalk& w, const Stack&
     st.tbest = __shfl_sync(F, st.tbest, src);
     st.best = __shfl_sync(F, st.best, src);
     st.slot = __shfl_sync(F, st.slot, src);
-    st.pad = __shfl_sync(F, st.pad, src);
     w.cur = __shfl_sync(F, w.cur, src);
     const int old = w.sp;
     w.sp = __shfl_sync(F, old, src);
@@ -257,8 +254,8 @@ __device__ __forceinline__ void quad_take(WideRay& st, WideWalk& w, const Stack&
 }
 
 // As wide_steps, for groups of four lanes; `active` is the same in the lanes of a group.
-template <int KEEP, class Stack>
-__device__ __forceinline__ void quad_steps(const float4* __restrict__ wide, const float4* __restrict__ tris, WideRay& st,
+template <int KEEP, class Ray, class Stack>
+__device__ __forceinline__ void quad_steps(const float4* __restrict__ wide, const float4* __restrict__ tris, Ray& st,
                                            WideWalk& w, const Stack& stk, bool active) {
     const uint32_t F = 0xffffffffu;
     const int c = threadIdx.x & 3;
@@ -334,9 +331,9 @@ static_assert(kCoopNarrow + 24 + 3 * (kWideMaxDepth / 2 + 1) < kCoopStack && kWi
 
 // Walks lane owner's ray (st, w and stk are that lane's) to its end; every lane calls it and
 // receives the ray with its final best hit. Not inlined: the callers' loops keep their registers.
-template <class Stack>
-__device__ __noinline__ WideRay coop_wide(const float4* __restrict__ wide, const float4* __restrict__ tris,
-                                          WideRay st, WideWalk w, Stack stk, int owner, CoopScratch* sc) {
+template <class Ray, class Stack>
+__device__ __noinline__ Ray coop_wide(const float4* __restrict__ wide, const float4* __restrict__ tris, Ray st,
+                                      WideWalk w, Stack stk, int owner, CoopScratch* sc) {
     const uint32_t F = 0xffffffffu;
     const int lane = threadIdx.x & 31, slot = lane >> 2, c = lane & 3;
     const uint32_t lt = lanemask_lt();
@@ -347,7 +344,6 @@ __device__ __noinline__ WideRay coop_wide(const float4* __restrict__ wide, const
     st.tbest = __shfl_sync(F, st.tbest, owner);
     st.best = __shfl_sync(F, st.best, owner);
     st.slot = __shfl_sync(F, st.slot, owner);
-    st.pad = __shfl_sync(F, st.pad, owner);
     int n = __shfl_sync(F, w.sp, owner) + 1;
     if (lane == owner) {
         for (int i = 0; i < n - 1; ++i) sc->stk[i] = stk.get(i);
@@ -360,7 +356,7 @@ __device__ __noinline__ WideRay coop_wide(const float4* __restrict__ wide, const
         if (slot < take) e = sc->stk[n - 1 - slot];
         n -= take;
         int32_t key = kWideMiss, ref = kWalkDone;
-        if (e.y != kWalkDone && wide_keep(e.x, st.tbest)) {
+        if (e.y != kWalkDone && gsp_wide_keep(e.x, st.tbest)) {
             if (e.y >= 0) {
                 const float* q = (const float*)(wide + 8 * (int64_t)e.y) + c;
                 key = wide_key(st, __ldg(q), __ldg(q + 4), __ldg(q + 8), __ldg(q + 12), __ldg(q + 16), __ldg(q + 20), c);
