@@ -48,14 +48,19 @@ struct HostBVH {
 // -inf gives a NaN, which no entry distance is at or below.
 GSP_HOST_DEVICE inline float gsp_reach(float x) { return x + fabsf(x) * 0x1p-19f; }
 
+// The same where only an x that is not negative counts (what is compared with it is not): one product.
+GSP_HOST_DEVICE inline float gsp_reach_ahead(float x) { return x * (1.0f + 0x1p-19f); }
+
 // Whether a child of the four-wide tree put by with this key (its entry distance, the two low bits
-// replaced; wide.cuh) may still hold a closer hit. Dropping the low bits rounds a distance down unless it
-// is negative (negative tmin, origin inside the box): never culled then.
+// replaced; wide.cuh) may still hold a closer hit, by the rule it was put by with: where surfaces coincide,
+// a triangle's t can be below its box's entry distance by the rounding of either, and without the slack the
+// winner of a tie would depend on the order of the walk. Dropping the low bits rounds a distance down unless
+// it is negative (negative tmin, origin inside the box): never culled then.
 GSP_HOST_DEVICE inline bool gsp_wide_keep(int32_t key, float tbest) {
     const int32_t bits = key & ~3;
     float t;
     memcpy(&t, &bits, sizeof t);
-    return key < 0 || t <= tbest;
+    return key < 0 || t <= gsp_reach_ahead(tbest);
 }
 
 // Centre and half extent of an interval of the four-wide tree's boxes: c - h <= lo and hi <= c + h

@@ -8,8 +8,10 @@
 // ref >= 0 is a wide node, < 0 is ~(leaf word); an absent child is a leaf of no triangles behind a box
 // that no ray meets unless its distances overflow on every axis (an origin at 1e10 with a direction of
 // length 1e-29, an infinite direction), so that a walk which goes there goes on after it. Leaves are the
-// binary tree's, and the hit is the lexicographic (t, index) minimum of the same triangle tests, so the
-// result does not depend on the form walked.
+// binary tree's, and the hit is the lexicographic (t, index) minimum of the same triangle tests. A box is
+// passed over only when it begins more than 2^-19 of the best t behind it (gsp_reach, gsp_wide_keep), which
+// covers the rounding of a triangle's t where that is well conditioned: the hit does not depend on the order
+// of the walk then, coincident surfaces included.
 //
 // What bounds a walk is the chain of dependent node fetches and the instructions per box. The links
 // visit 53 boxes for a bounce ray of the 247,234-triangle scene (two per fetch at best) and need six
@@ -63,7 +65,7 @@ struct WideRay : RayHit {};
 struct PathRay : RayHit {};
 
 __device__ __forceinline__ float wide_far(const WideRay&, float x) { return gsp_reach(x); }
-__device__ __forceinline__ float wide_far(const PathRay&, float x) { return __fmul_rn(x, 1.0f + 0x1p-19f); }
+__device__ __forceinline__ float wide_far(const PathRay&, float x) { return gsp_reach_ahead(x); }
 
 // 1 / d to 1 ulp (2u): all that the slab test needs.
 __device__ __forceinline__ float wide_inv(float d) {

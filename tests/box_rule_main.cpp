@@ -29,7 +29,7 @@ struct Best {
     int32_t id;
 };
 
-// Moller-Trumbore on one triangle {v0, id}, {v1, .}, {v2, .}, as the library's
+// Moller-Trumbore on one triangle {v0, id}, {v1, .}, {v2, .}
 static void test_tri(const float4* tri, const float* r, Best& b) {
     const float *P = (const float*)tri, *d = r + 4;
     float e1[3], e2[3], s[3];
@@ -182,6 +182,19 @@ int main(int argc, char** argv) {
         }
         // distances that overflow for the box of an absent child, at the origin, but not for the scene's
         bad += check("far away, short directions", soup(300, -1e10f, 1e7f), 1500, -1e10f, 1e7f, 1e-29f);
+    }
+    if (group == "ties") {
+        for (float len : {1.0f, 20.0f, 0.05f}) {
+            Mesh floors;  // two floors at one height, differently divided
+            add_floor(floors, 30, 0.3f, 0.0f);
+            add_floor(floors, 23, 0.3f, 0.013f);
+            bad += check("two floors", floors, 1500, 0.0f, 1.0f, len);
+            for (float slope : {0.0f, 0.5f}) {  // triangles over one another in one plane
+                Mesh m = soup(2000, 0.0f, 1.0f);
+                for (size_t i = 0; i < m.v.size(); i += 3) m.v[i + 1] = 0.37f + slope * m.v[i] - 0.5f * slope * m.v[i + 2];
+                bad += check("one plane", m, 1500, 0.0f, 1.0f, len);
+            }
+        }
     }
     if (!bad) std::puts("ok");
     return bad != 0;

@@ -30,3 +30,8 @@ def run(exe, group):
 def test_negative_tmin(exe):
     """tmin behind the origin, down to -inf, with unit, long and short directions."""
     run(exe, "tmin")
+
+
+def test_coincident_surfaces(exe):
+    """Ties in t between triangles of different leaves: the smallest index wins in any order of the walk."""
+    run(exe, "ties")

@@ -22,20 +22,25 @@ def floor(g):
                    tri_mat=np.zeros(len(tris), np.int32), mats=sc.mats, camera=sc.camera)
 
 
+def fma(a, b, c):
+    """FP32 a b + c rounded once (but for the rounding of the sum to FP64 before that)."""
+    return (a.double() * b.double() + c.double()).float()
+
+
 def every_triangle(sc, rays):
-    """Index of the closest triangle of each ray, -1 for none (ties: the smallest index)."""
+    """Index of the closest triangle of each ray, -1 for none (ties: the smallest index). The products and
+    fused sums of the library's device code, in its order."""
     v = torch.from_numpy(sc.verts).cuda()[torch.from_numpy(sc.tris).cuda().long()]
     v0, e1, e2 = v[:, 0], v[:, 1] - v[:, 0], v[:, 2] - v[:, 0]
     out = []
-    for r in rays.split(512):
+    for r in rays.split(256):
         o, d = r[:, None, 0:3], r[:, None, 4:7]
 
         def cross(a, b):
-            return (a[..., 1] * b[..., 2] - a[..., 2] * b[..., 1], a[..., 2] * b[..., 0] - a[..., 0] * b[..., 2],
-                    a[..., 0] * b[..., 1] - a[..., 1] * b[..., 0])
+            return tuple(fma(a[..., i], b[..., j], -(a[..., j] * b[..., i])) for i, j in ((1, 2), (2, 0), (0, 1)))
 
         def dot(a, b):
-            return a[..., 0] * b[0] + a[..., 1] * b[1] + a[..., 2] * b[2]
+            return fma(a[..., 2], b[2], fma(a[..., 1], b[1], a[..., 0] * b[0]))
 
         p = cross(d, e2)
         det = dot(e1, p)
