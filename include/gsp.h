@@ -245,6 +245,10 @@ gsp_status gsp_build_bvh_device(gsp_scene* scene, int32_t link_sets, int32_t max
  * diagonal of at most 1e8 is walked in the tree's four-wide form: each node holds the boxes of a
  * binary node's grandchildren, the nearest one hit is visited next and the others wait on a stack
  * (about a quarter of the fetches that depend on one another). Other scenes follow the hit/miss links.
+ * Either walk passes over a box that begins more than 2^-19 of the best t behind it. That covers the
+ * rounding of the box test and of a well-conditioned t, so that coincident surfaces give the smallest
+ * index; where Moller-Trumbore rounds by more (slivers, rays along a surface), triangles whose t differ by
+ * that rounding may give another of them in another walk. tmin may be negative, down to -inf.
  *  d_rays [n][8] float: ox, oy, oz, tmin, dx, dy, dz, tmax (d need not be unit length)
  *  d_tri  [n] int32 out: triangle index in the uploaded order, -1 on a miss
  *  d_t    [n] float out: hit distance (in units of |d|), +inf on a miss

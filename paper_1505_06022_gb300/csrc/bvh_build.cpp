@@ -361,7 +361,6 @@ inline int ray_class(float dx, float dy, float dz) {
 
 void bvh_host_walk(const HostBVH& bvh, const float* rays, int64_t n, int32_t* out_tri, float* out_t,
                    int32_t* visits, int32_t* tests) {
-    const float kRobust = 1.0f + 2.0f * (3.0f * 5.9604645e-8f) / (1.0f - 3.0f * 5.9604645e-8f);
     for (int64_t i = 0; i < n; ++i) {
         const float* r = rays + 8 * i;
         float o[3] = {r[0], r[1], r[2]}, d[3] = {r[4], r[5], r[6]};
@@ -387,9 +386,8 @@ void bvh_host_walk(const HostBVH& bvh, const float* rays, int64_t n, int32_t* ou
                 tn = std::max(tn, std::min(t0, t1));
                 tf = std::min(tf, std::max(t0, t1));
             }
-            tf = std::min(tbest, tf * kRobust);
             int32_t miss = as_int(A.w), word = as_int(B.w);
-            if (tn <= tf) {
+            if (tn <= gsp_reach(std::min(tbest, tf))) {
                 if (word >= 0) {
                     int32_t first = word >> 3, cnt = word & 7;
                     for (int32_t k = 0; k < cnt; ++k) {

@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "gsp_internal.h"
+
 namespace gspd {
 
 // ----------------------------------------------------------------------------------------------
@@ -147,10 +149,6 @@ __device__ __forceinline__ int ray_class(float3 d) {
 __device__ __forceinline__ float safe_inv(float d) {
     return __frcp_rn(fabsf(d) < 1e-30f ? copysignf(1e-30f, d) : d);
 }
-
-// 1 + 2 gamma_3 with gamma_n = n u / (1 - n u), u = 2^-24: the far-plane scale that makes the
-// FP32 slab test conservative against relative rounding errors (Ize 2013).
-#define GSP_ROBUST_FAR 1.0000003576278687f
 
 // Three-input minimum and maximum (one instruction each on sm_100 and later).
 __device__ __forceinline__ float max3f(float a, float b, float c) {
@@ -445,8 +443,11 @@ __device__ __forceinline__ void ldg64(const float4* p, float4& A, float4& B, flo
 }
 
 // Slab test of the box [lo, hi] against [tmin, best t] (Fig. 3's intersect(node.aabb, ray)):
-// t = (b - o) inv per plane, three-input min and max for the interval, the far end scaled by
-// GSP_ROBUST_FAR; conservative. On a hit tn is the entry distance. (The fused form
+// t = (b - o) inv per plane, three-input min and max for the interval. A plane's t errs by 3u at most
+// (u = 2^-24; Ize 2013), either end of the interval by as much, and gsp_reach's 32u cover both on either
+// side of the origin; they also cover the rounding of the best t on coincident surfaces (gsp_wide_keep
+// says why that matters). A factor on the far end, as this once had, moves a negative one the wrong way:
+// every hit behind the origin on a flat box was missed. On a hit tn is the entry distance. (The fused form
 // t = b inv + (-o inv) saves six instructions per box but errs in absolute terms by about
 // u |o inv|, which needs a per-plane pad held in six more registers per ray; on GB300 the spills
 // and lost residency that cost made the traversal slower: 5,132 against 5,217 Mrays/s.)
@@ -457,7 +458,7 @@ __device__ __forceinline__ bool slab(const RayHit& st, float3 lo, float3 hi, flo
     const float t0z = __fmul_rn(lo.z - o.z, inv.z), t1z = __fmul_rn(hi.z - o.z, inv.z);
     tn = max3f(fminf(t0x, t1x), fminf(t0y, t1y), fmaxf(fminf(t0z, t1z), st.tmin));
     const float tf = min3f(fmaxf(t0x, t1x), fmaxf(t0y, t1y), fmaxf(t0z, t1z));
-    return tn <= fminf(st.tbest, __fmul_rn(tf, GSP_ROBUST_FAR));
+    return tn <= gsp_reach(fminf(st.tbest, tf));
 }
 
 // Box test of a node {A, B} = {min.xyz, miss | max.xyz, leaf word} against [tmin, best t].

@@ -2,7 +2,7 @@
 // gsp_wide_entry), a lane's steps as csrc/wide.cuh makes them, against every triangle in turn: the same
 // triangle and t, whatever tmin, the length of the direction, and the last bit of the reciprocals (which
 // the device takes from an approximation). Lines (tmin far behind the origin) cost what long rays cost.
-// Argument: the group of cases (tests/test_box_rule.py).
+// Arguments: the group of cases (tests/test_box_rule.py); "links" for the library's walk of the hit/miss links.
 #include <algorithm>
 #include <cfloat>
 #include <cmath>
@@ -97,6 +97,8 @@ static Best walk(const HostBVH& b, const std::vector<float4>& wide, const float*
     return best;
 }
 
+static bool links;  // the library's host walk of the hit/miss links instead
+
 // nr rays from the box around `at` with half extent 2 `size`, directions of length about `len`. Returns
 // the number of rays whose walk differs from the triangles in turn.
 static int check(const char* name, const Mesh& m, int nr, float at, float size, float len) {
@@ -129,12 +131,19 @@ static int check(const char* name, const Mesh& m, int nr, float at, float size, 
             Best want{r[7], -1};
             for (int k = 0; k < nt; ++k) test_tri(&b.tris[3 * k], r, want);
             hits += want.id >= 0;
-            for (int ulp = -1; ulp <= 1; ++ulp) {
+            if (links) {
+                Best got;
+                int32_t visits;
+                bvh_host_walk(b, r, 1, &got.id, &got.t, &visits, nullptr);
+                cost[j] += visits;
+                wrong += got.id != want.id || (want.id >= 0 && got.t != want.t);
+            }
+            for (int ulp = -1; ulp <= 1 && !links; ++ulp) {
                 const Best got = walk(b, wide, r, ulp, cost[j]);
                 wrong += got.id != want.id || (want.id >= 0 && got.t != want.t);
             }
         }
-        if (wrong || !hits) std::printf("%s, direction %g, tmin %g: %d of %d walks wrong, %d hits\n", name, len, tmins[j], wrong, 3 * nr, hits);
+        if (wrong || !hits) std::printf("%s, direction %g, tmin %g: %d of %d walks wrong, %d hits\n", name, len, tmins[j], wrong, links ? nr : 3 * nr, hits);
         bad += wrong + !hits;
     }
     for (int j = 3; j < 6; ++j)  // the boxes a line meets do not depend on where far behind it starts
@@ -172,6 +181,7 @@ static void add_floor(Mesh& m, int G, float y, float shift) {
 
 int main(int argc, char** argv) {
     const std::string group = argc > 1 ? argv[1] : "";
+    links = argc > 2 && std::string(argv[2]) == "links";
     int bad = 0;
     if (group == "tmin") {
         for (float len : {1.0f, 20.0f, 0.05f}) {

@@ -1,5 +1,5 @@
-"""The four-wide walk's box and stack rules on the CPU against every triangle in turn
-(tests/box_rule_main.cpp)."""
+"""The box and stack rules of the four-wide walk and of the walk of the hit/miss links on the CPU against
+every triangle in turn (tests/box_rule_main.cpp)."""
 import os
 import shutil
 import subprocess
@@ -22,8 +22,8 @@ def exe(tmp_path_factory):
     return path
 
 
-def run(exe, group):
-    r = subprocess.run([exe, group], capture_output=True, text=True, timeout=600)
+def run(exe, *group):
+    r = subprocess.run([exe, *group], capture_output=True, text=True, timeout=600)
     assert r.returncode == 0 and "ok" in r.stdout, (r.stdout + r.stderr)[-3000:]
 
 
@@ -35,3 +35,9 @@ def test_negative_tmin(exe):
 def test_coincident_surfaces(exe):
     """Ties in t between triangles of different leaves: the smallest index wins in any order of the walk."""
     run(exe, "ties")
+
+
+@pytest.mark.parametrize("group", ["tmin", "ties"])
+def test_links(exe, group):
+    """The same of the walk of the hit/miss links: boxes without extent behind the origin among them."""
+    run(exe, group, "links")
