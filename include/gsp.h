@@ -105,8 +105,8 @@ typedef struct {
     int32_t depth;
     int32_t link_sets;
     double build_ms;      /* SAH build on the host */
-    double thread_ms;     /* writing the hit/miss links of every link set on the host */
-    int64_t device_bytes; /* node + triangle + shading bytes resident on the device */
+    double thread_ms;     /* writing the hit/miss links of every link set on the host, and the four-wide form */
+    int64_t device_bytes; /* node (in every form), triangle and shading bytes resident on the device */
 } gsp_bvh_stats;
 
 /* SPPM parameters.

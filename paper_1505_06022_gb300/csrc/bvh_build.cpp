@@ -280,35 +280,25 @@ std::string bvh_build_host(const float* verts, int64_t nv, const int32_t* tris, 
             dst[2 * q + 1] = float4{nd.hi[0], nd.hi[1], nd.hi[2], as_float(word)};
         }
     };
-    {
-        std::vector<std::thread> th;
-        for (int c = 1; c < sets; ++c) {
-            if (nthreads > 1) th.emplace_back(thread_set, c);
-            else thread_set(c);
-        }
-        thread_set(0);
-        for (auto& x : th) x.join();
-    }
-    auto t2 = clk::now();
-
-    // ---- the same tree as child pairs (stack-based traversal), internal nodes in preorder ----
-    {
+    // ---- the same tree as child pairs (stack-based traversal), internal nodes in preorder, beside the links:
+    // numbering them and the four-wide entries would add to the build's time (1 % of it) ----
+    const auto pairs = [&] {
         std::vector<int32_t> ref(nn, 0), st;
-        std::vector<int8_t> odd(nn, 0);
         int32_t ni = 0;
+        if (sets == 6) out.wide_of.resize((size_t)(nn - 1) / 2);  // a binary tree's internal nodes
+        int32_t* const wide = out.wide_of.data();
         st.push_back(0);
         while (!st.empty()) {  // preorder numbering of the internal nodes, and of those of even depth
-            int32_t n = st.back();
+            const int32_t n = st.back() & 0x7fffffff, odd = st.back() & INT32_MIN;
             st.pop_back();
             if (nodes[n].left < 0) {
                 ref[n] = ~((nodes[n].first << 3) | nodes[n].count);
                 continue;
             }
+            if (sets == 6) wide[ni] = odd ? -1 : (int32_t)out.nwide++;
             ref[n] = ni++;
-            out.wide_of.push_back(odd[n] ? -1 : (int32_t)out.nwide++);
-            odd[nodes[n].left] = odd[nodes[n].right] = !odd[n];
-            st.push_back(nodes[n].right);
-            st.push_back(nodes[n].left);
+            st.push_back(nodes[n].right | (odd ^ INT32_MIN));
+            st.push_back(nodes[n].left | (odd ^ INT32_MIN));
         }
         out.bin.assign((size_t)ni * 4, float4{0, 0, 0, 0});
         for (int64_t n = 0; n < nn; ++n) {
@@ -322,7 +312,19 @@ std::string bvh_build_host(const float* verts, int64_t nv, const int32_t* tris, 
             q[3] = float4{R.hi[0], R.hi[1], R.hi[2], 0.0f};
         }
         out.bin_root = ref[0];
+    };
+    {
+        std::vector<std::thread> th;
+        if (nthreads > 1) th.emplace_back(pairs);
+        else pairs();
+        for (int c = 1; c < sets; ++c) {
+            if (nthreads > 1) th.emplace_back(thread_set, c);
+            else thread_set(c);
+        }
+        thread_set(0);
+        for (auto& x : th) x.join();
     }
+    auto t2 = clk::now();
 
     // ---- triangles in leaf order: exact vertices v0, v1, v2 (edges are formed in the kernel) ----
     out.tris.resize((size_t)nt * 3);

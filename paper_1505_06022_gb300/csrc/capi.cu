@@ -1,4 +1,5 @@
 // capi.cu -- context, scene, BVH and closest-hit entry points of the C ABI (include/gsp.h).
+#include <chrono>
 #include <cmath>
 #include <cstring>
 #include <mutex>
@@ -353,12 +354,7 @@ gspd::DevScene gsp_dev_scene(const gsp_scene* s) {
     d.tris = s->d_tris;
     d.bin = s->d_bin;
     d.bin_root = s->bvh.bin_root;
-    // a step limit counts the box tests of the links' walk; a single link set is there to be walked
-    // in its one order (Fig. 4); and a deeper tree could need more than the wide walk's stack
-    d.wide = s->step_limit == 0 && s->bvh.link_sets == 6 && s->bvh.depth <= kWideMaxDepth &&
-                     s->extent <= kWideMaxExtent
-                 ? s->d_wide
-                 : nullptr;
+    d.wide = s->step_limit == 0 ? s->d_wide : nullptr;  // a step limit counts the box tests of the links' walk
     d.step_limit = s->step_limit;
     d.shade = s->d_shade;
     d.nlo = s->d_nlo;
@@ -454,6 +450,11 @@ static void host_lanes_free(gsp_scene* s) {
         L = gsp_scene::HostLane{};
     }
     s->lane_cap = 0;
+}
+
+// What a tree takes on the device (links, child pairs, four-wide form, triangles), with the shading records.
+static int64_t bvh_device_bytes(const HostBVH& b, int64_t nt) {
+    return (int64_t)sizeof(float4) * ((int64_t)(b.nodes.size() + b.tris.size() + b.bin.size()) + 8 * b.nwide + 2 * nt);
 }
 
 static void scene_free_bvh(gsp_scene* s) {
@@ -723,6 +724,7 @@ gsp_status gsp_build_bvh(gsp_scene* s, const gsp_bvh_params* params, gsp_bvh_sta
         gsp_set_last_error(err);
         return GSP_ERR_INVALID_ARG;
     }
+    if (!gsp_wide_usable(bvh.link_sets, bvh.depth, s->extent)) bvh.nwide = 0;
     size_t nb = bvh.nodes.size() * sizeof(float4), tb = bvh.tris.size() * sizeof(float4);
     const size_t bb = std::max<size_t>(1, bvh.bin.size()) * sizeof(float4);
     if (s->ctx) {
@@ -736,6 +738,7 @@ gsp_status gsp_build_bvh(gsp_scene* s, const gsp_bvh_params* params, gsp_bvh_sta
         if (!bvh.bin.empty())
             GSP_CUDA_TRY(cudaMemcpy(s->d_bin, bvh.bin.data(), bvh.bin.size() * sizeof(float4), cudaMemcpyHostToDevice));
         if (bvh.nwide) {
+            const auto t0 = std::chrono::steady_clock::now();
             uint32_t* of = nullptr;
             const size_t ob = bvh.wide_of.size() * sizeof(int32_t);
             GSP_CUDA_TRY(cudaMalloc(&s->d_wide, (size_t)bvh.nwide * 8 * sizeof(float4)));
@@ -745,12 +748,13 @@ gsp_status gsp_build_bvh(gsp_scene* s, const gsp_bvh_params* params, gsp_bvh_sta
             if (e == cudaSuccess) e = cudaDeviceSynchronize();
             cudaFree(of);
             GSP_CUDA_TRY(e);
-            std::vector<int32_t>().swap(bvh.wide_of);
+            bvh.thread_ms += std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
         }
+        std::vector<int32_t>().swap(bvh.wide_of);
     }
+    s->device_bytes = bvh_device_bytes(bvh, s->nt);
     s->bvh = std::move(bvh);
     s->built = true;
-    s->device_bytes = (int64_t)(nb + tb) + s->nt * (int64_t)sizeof(float4);  // MTBVH + triangles + shading
     if (stats) {
         stats->nodes = s->bvh.nnodes;
         stats->leaves = s->bvh.nleaves;
@@ -1040,7 +1044,7 @@ void gsp_scene_adopt_bvh(gsp_scene* s, HostBVH&& bvh, float4* d_nodes, float4* d
     s->d_tris = d_tris;
     s->d_bin = d_bin;
     s->d_wide = d_wide;
-    s->device_bytes = (int64_t)((bvh.nodes.size() + bvh.tris.size()) * sizeof(float4)) + s->nt * (int64_t)sizeof(float4);
+    s->device_bytes = bvh_device_bytes(bvh, s->nt);
     s->bvh = std::move(bvh);
     s->built = true;
 }

@@ -30,9 +30,10 @@ struct HostBVH {
     std::vector<float4> bin;
     int32_t bin_root = 0;
     // The same tree four-wide (wide.cuh): the entry of each of bin's nodes, -1 for a node of odd depth
-    // (gsp_wide_entry makes them). Empty for a tree that is a single leaf. The device build keeps none here.
+    // (gsp_wide_entry makes them). Empty for a tree that is a single leaf or has one link set. The device
+    // build keeps none here.
     std::vector<int32_t> wide_of;
-    int64_t nwide = 0;
+    int64_t nwide = 0;  // entries
     double build_ms = 0, thread_ms = 0;
 };
 
@@ -102,6 +103,15 @@ GSP_HOST_DEVICE inline void gsp_wide_entry(const float4* bin, int64_t i, Of of, 
     for (int k = 28; k < 32; ++k) q[k] = 0.0f;
 }
 
+// Which scenes have a four-wide tree: a single link set is there to be walked in its one order (Fig. 4), a
+// deeper tree could need more than the walk's stack holds, and in a larger scene (c - o) / d could overflow
+// for a tiny d inside a box. Others follow the links, and the tree is not made for them.
+constexpr int kWideMaxDepth = 38;
+constexpr double kWideMaxExtent = 1e8;
+inline bool gsp_wide_usable(int32_t link_sets, int32_t depth, double extent) {
+    return link_sets == 6 && depth <= kWideMaxDepth && extent <= kWideMaxExtent;
+}
+
 // The entries of all of them on the device: node i has entry index[i], if head is given only where
 // head[i] is set, else where it is not -1.
 cudaError_t gsp_wide_build(const float4* bin, int64_t n, const uint32_t* head, const uint32_t* index, float4* wide);
@@ -140,7 +150,7 @@ struct gsp_scene {
     float4* d_nodes = nullptr;
     float4* d_tris = nullptr;
     float4* d_bin = nullptr;  // child-pair layout (HostBVH::bin)
-    float4* d_wide = nullptr;  // four-wide layout (HostBVH::wide); null if the tree is one leaf
+    float4* d_wide = nullptr;  // four-wide layout; null if the tree is one leaf or not gsp_wide_usable
     unsigned long long* d_counter = nullptr;  // trace kernel: next ray, refine-list length
     int2* d_rlist = nullptr;                  // trace kernel: hits re-evaluated in FP64
     int64_t rlist_cap = 0;

@@ -30,8 +30,6 @@ constexpr int kTraceChunk = GSP_TRACE_CHUNK;           // rays a warp takes from
 constexpr int kTraceInner = GSP_TRACE_INNER;           // traversal steps between refills
 constexpr int kTraceLeafBatch = GSP_TRACE_LEAF_BATCH;  // pending leaves that trigger a warp-wide leaf test
 constexpr int kWideStack = 64;     // children a walk of the four-wide tree may keep (at most three per wide level)
-constexpr int kWideMaxDepth = 38;  // depth of the binary tree up to which that is enough
-constexpr float kWideMaxExtent = 1e8f;  // larger scenes: (c - o) / d could overflow for a tiny d inside a box
 constexpr int kPathChunk = GSP_PATH_CHUNK;  // paths a warp of the path kernels takes at once (a block's
                                             // grid share is 128 paths: every warp of a short launch gets some)
 

@@ -358,14 +358,15 @@ extern "C" gsp_status gsp_build_bvh_device(gsp_scene* s, int32_t link_sets, int3
     if (n > 1) k_internal<<<nblocks(n - 1), kThreads>>>(keys, n, left, right, parent, first, last);
     k_bottom_up<<<nblocks(n), kThreads>>>(d_verts, d_tris, ids, n, left, right, parent, first, last, max_leaf, box,
                                           size, arrived);
-    if (n > 1) {
+    const bool wide = n > 1 && gsp_wide_usable(link_sets, 0, s->extent);  // the depth is not known yet
+    if (wide) {
         k_wide_heads<<<nblocks(n - 1), kThreads>>>(n, parent, first, last, max_leaf, head);
         e = gsp_scan_u32(head, windex, n - 1, windex + (n - 1), stemp, nullptr);
     }
     int32_t nfinal = 0;
     uint32_t nwide = 0;
     if (e == cudaSuccess) e = cudaGetLastError();
-    if (e == cudaSuccess && n > 1)
+    if (e == cudaSuccess && wide)
         e = cudaMemcpy(&nwide, windex + (n - 1), sizeof nwide, cudaMemcpyDeviceToHost);
     if (e == cudaSuccess) e = cudaMemcpy(&nfinal, size, sizeof nfinal, cudaMemcpyDeviceToHost);  // root: node 0
     if (e != cudaSuccess) return fail(e);
@@ -421,6 +422,11 @@ extern "C" gsp_status gsp_build_bvh_device(gsp_scene* s, int32_t link_sets, int3
         return fail(e);
     }
     for (void* p : tmp) cudaFree(p);
+    if (!gsp_wide_usable(link_sets, depth, s->extent)) {
+        cudaFree(d_wide);
+        d_wide = nullptr;
+        nwide = 0;
+    }
     int64_t leaves = 0;
     for (int64_t q = 0; q < nfinal; ++q) {
         int32_t w;
@@ -437,6 +443,7 @@ extern "C" gsp_status gsp_build_bvh_device(gsp_scene* s, int32_t link_sets, int3
     bvh.stride = stride;
     bvh.nleaves = leaves;
     bvh.depth = depth;
+    bvh.nwide = nwide;
     bvh.link_sets = link_sets;
     bvh.build_ms = build_ms;
     bvh.thread_ms = thread_ms;
