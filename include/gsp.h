@@ -272,7 +272,7 @@ gsp_status gsp_trace_time_launches(gsp_scene* scene, int64_t n);
 gsp_status gsp_trace_launch_times(gsp_scene* scene, float* h_ms, int64_t capacity, int64_t* count);
 
 /* The same closest-hit query on HOST buffers (h_rays [n][8], h_tri [n], h_t [n], h_uv [n][2] or
- * NULL), synchronous. Page-locked buffers the device can address (cudaHostAlloc /
+ * NULL), synchronous. Buffers wholly in page-locked memory that the device can address (cudaHostAlloc /
  * cudaHostRegister, e.g. pinned torch tensors; h_rays 16-byte aligned): the traversal reads the
  * rays from host memory itself; up to 2^18 rays it also writes the results there (to buffers aligned
  * to their elements, uv to 8 bytes), more go in two halves on two streams, and each half's results are

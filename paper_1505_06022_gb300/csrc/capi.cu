@@ -1,4 +1,6 @@
 // capi.cu -- context, scene, BVH and closest-hit entry points of the C ABI (include/gsp.h).
+#include <cuda.h>  // driver types only: the call is reached through the runtime
+
 #include <chrono>
 #include <cmath>
 #include <cstring>
@@ -858,6 +860,35 @@ static gsp_status host_lanes_reserve(gsp_scene* s, int64_t cap, bool staged) {
 
 static constexpr int64_t kHostDirect = int64_t(1) << 18;
 
+// The device's address of the host buffer [p, p + bytes) if all of it is page-locked memory that the device
+// can address in one piece, else null. Its two ends are not enough: between two registrations there may be
+// memory of neither.
+static void* mapped(const void* p, size_t bytes) {
+    typedef CUresult (*Get)(void*, CUpointer_attribute, CUdeviceptr);
+    static const Get get = (Get)gsp_driver_fn("cuPointerGetAttribute");
+    if (!get) return nullptr;
+    char* dev = nullptr;
+    for (size_t at = 0; at < bytes;) {
+        const char* q = (const char*)p + at;
+        cudaPointerAttributes a{};
+        CUdeviceptr start = 0;
+        size_t size = 0;
+        if (cudaPointerGetAttributes(&a, q) != cudaSuccess) {
+            (void)cudaGetLastError();
+            return nullptr;
+        }
+        if (a.type != cudaMemoryTypeHost || !a.devicePointer || (at && a.devicePointer != dev + at) ||
+            get(&start, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, (CUdeviceptr)a.devicePointer) != CUDA_SUCCESS ||
+            get(&size, CU_POINTER_ATTRIBUTE_RANGE_SIZE, (CUdeviceptr)a.devicePointer) != CUDA_SUCCESS)
+            return nullptr;
+        if (!at) dev = (char*)a.devicePointer;
+        const CUdeviceptr end = start + size, here = (CUdeviceptr)a.devicePointer;
+        if (start > here || end <= here) return nullptr;
+        at += (size_t)(end - here);
+    }
+    return dev;
+}
+
 // Closest hits for host buffers. Page-locked buffers that the device can address, up to kHostDirect
 // rays: one launch reads the rays from host memory and writes the hits to it, which saves the copies
 // and the second launch (100 rays 35 -> 20 us, 10,000 with uv 58 -> 40, 30,000 69 -> 58, 100,000 95 -> 94,
@@ -880,27 +911,13 @@ gsp_status gsp_trace_closest_hit_host(gsp_scene* s, const float* h_rays, int64_t
     if (!h_rays || !h_tri || !h_t || n > INT32_MAX) return GSP_ERR_INVALID_ARG;
     GSP_CUDA_TRY(cudaSetDevice(s->ctx->device));
     GSP_NO_PENDING_ERROR("gsp_trace_closest_hit_host");
-    // page-locked host memory that the device can address directly (NULL if it cannot)
-    auto mapped = [](const void* p) -> const void* {
-        cudaPointerAttributes a{};
-        if (!p || cudaPointerGetAttributes(&a, p) != cudaSuccess) {
-            (void)cudaGetLastError();
-            return nullptr;
-        }
-        return a.type == cudaMemoryTypeHost ? a.devicePointer : nullptr;
-    };
-    const float4* m_rays = (const float4*)mapped(h_rays);
-    if (m_rays && !((uintptr_t)m_rays & 15) && mapped(h_tri) && mapped(h_t) && (!h_uv || mapped(h_uv))) {
-        // a result buffer that the device can write itself: all of it mapped, and aligned to its stores
-        auto writable = [&](void* p, size_t bytes, size_t align) -> void* {
-            char* d = (char*)mapped(p);
-            return d && !((uintptr_t)d % align) && mapped((char*)p + bytes - 1) == d + bytes - 1 ? d : nullptr;
-        };
-        const bool small = n <= kHostDirect;
-        int32_t* m_tri = small ? (int32_t*)writable(h_tri, (size_t)n * 4, 4) : nullptr;
-        float* m_t = small ? (float*)writable(h_t, (size_t)n * 4, 4) : nullptr;
-        float2* m_uv = small && h_uv ? (float2*)writable(h_uv, (size_t)n * 8, 8) : nullptr;
-        if (m_tri && m_t && (!h_uv || m_uv)) {
+    const float4* m_rays = (const float4*)mapped(h_rays, (size_t)n * 32);
+    int32_t* m_tri = (int32_t*)mapped(h_tri, (size_t)n * 4);
+    float* m_t = (float*)mapped(h_t, (size_t)n * 4);
+    float2* m_uv = h_uv ? (float2*)mapped(h_uv, (size_t)n * 8) : nullptr;
+    if (m_rays && !((uintptr_t)m_rays & 15) && m_tri && m_t && (!h_uv || m_uv)) {
+        // results that the device writes itself are aligned to its stores
+        if (n <= kHostDirect && !((uintptr_t)m_tri & 3) && !((uintptr_t)m_t & 3) && !((uintptr_t)m_uv & 7)) {
             gsp_status e = host_lanes_reserve(s, n, false);
             if (e != GSP_OK) return e;
             auto& L = s->lanes[0];

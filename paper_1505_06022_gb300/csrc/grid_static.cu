@@ -20,6 +20,19 @@ int64_t gsp_grid_scratch_words(int64_t n, int64_t T);
 gsp_status gsp_grid_build_with(const float4* pos, int64_t n, float cell_h, int64_t T, uint32_t* order,
                                uint32_t* bstart, uint32_t* scratch, cudaStream_t st, bool skip_invalid);
 
+// A driver entry point through the runtime's query (no link against libcuda); null if the
+// driver does not offer it.
+void* gsp_driver_fn(const char* name) {
+    void* p = nullptr;
+    cudaDriverEntryPointQueryResult q = cudaDriverEntryPointSymbolNotFound;
+    if (cudaGetDriverEntryPointByVersion(name, &p, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+        q != cudaDriverEntryPointSuccess) {
+        (void)cudaGetLastError();  // the query's own failure: not left for the next call to report
+        return nullptr;
+    }
+    return p;
+}
+
 namespace {
 
 constexpr int64_t kMaxPoints = GSP_GRID_STATIC_MAX_POINTS;
@@ -48,23 +61,10 @@ Slot g_slot[kMaxDevices];
 using CtxGetCurrent = CUresult (*)(CUcontext*);
 using CtxGetId = CUresult (*)(CUcontext, unsigned long long*);
 
-// A driver entry point through the runtime's query (no link against libcuda); null if the
-// driver does not offer it.
-void* driver_fn(const char* name) {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q = cudaDriverEntryPointSymbolNotFound;
-    if (cudaGetDriverEntryPointByVersion(name, &p, 12000, cudaEnableDefault, &q) != cudaSuccess ||
-        q != cudaDriverEntryPointSuccess) {
-        (void)cudaGetLastError();  // the query's own failure: not left for the next call to report
-        return nullptr;
-    }
-    return p;
-}
-
 // ID of the calling thread's current context; 0 when there is none or the driver cannot say.
 unsigned long long current_context_id() {
-    static const CtxGetCurrent get = (CtxGetCurrent)driver_fn("cuCtxGetCurrent");
-    static const CtxGetId get_id = (CtxGetId)driver_fn("cuCtxGetId");
+    static const CtxGetCurrent get = (CtxGetCurrent)gsp_driver_fn("cuCtxGetCurrent");
+    static const CtxGetId get_id = (CtxGetId)gsp_driver_fn("cuCtxGetId");
     CUcontext c = nullptr;
     unsigned long long id = 0;
     if (!get || !get_id || get(&c) != CUDA_SUCCESS || !c || get_id(c, &id) != CUDA_SUCCESS) return 0;

@@ -191,6 +191,10 @@ struct gsp_scene {
 // replacing the scene's current one.
 void gsp_scene_adopt_bvh(gsp_scene* s, HostBVH&& bvh, float4* d_nodes, float4* d_tris, float4* d_bin, float4* d_wide);
 
+// A driver entry point through the runtime's query (no link against libcuda); null if the driver does not
+// offer it (grid_static.cu).
+void* gsp_driver_fn(const char* name);
+
 // NVTX range around a host-side stage (header-only NVTX3: a no-op unless a profiler attaches).
 struct NvtxRange {
     explicit NvtxRange(const char* name) { nvtxRangePushA(name); }
