@@ -289,7 +289,11 @@ def run_ours(args, world, rank, local):
         try:
             tf = json.load(open(traffic_file))
             if tf.get("kernel_digest") == gsp_kernel_digest():
-                roofline["traffic"] = tf.get("dram_bytes_per_launch")
+                roofline["traffic"] = tf["dram_bytes_per_launch"]
+                gbs = roofline["traffic"] / (ms_kernel * 1e-3) / 1e9
+                roofline["dram"] = {"achieved": round(gbs, 1), "peak": roofline["peak"], "unit": "GB/s",
+                                    "frac": round(gbs / roofline["peak"], 4),
+                                    "source": "the launch's DRAM bytes as profiled (trace_traffic.json) over its time here"}
         except Exception:
             pass
 
@@ -360,7 +364,7 @@ def fp32_peak_tflops(sm_count, peaks):
 def traversal_roofline(v_node, v_tri, n, ms, call_ms, sm_count, peaks, tiers):
     """The bench line's roofline block for closest hit: algorithmic bytes and flops of n rays with
     v_node node visits and v_tri triangle tests per ray (of the hit/miss links' walk, whichever form of
-    the tree the kernel walks), against the traversal kernel's mean launch
+    the tree the kernel walks: WORK_MODEL), against the traversal kernel's mean launch
     time `ms` (call_ms: the whole call, with the counter reset and the refinement of flagged hits)."""
     bytes_ray = BYTES_PER_NODE * v_node + BYTES_PER_TRI * v_tri + BYTES_PER_RAY_IO
     flops_ray = FLOPS_PER_NODE * v_node + FLOPS_PER_TRI * v_tri
@@ -385,10 +389,16 @@ def traversal_roofline(v_node, v_tri, n, ms, call_ms, sm_count, peaks, tiers):
             "fp32": {"achieved": round(flops_ray * n / s / 1e12, 3), "peak": round(fp32, 2), "unit": "TFLOP/s",
                      "frac": round(flops_ray * n / s / 1e12 / fp32, 4),
                      "source": f"{sm_count} SMs x 128 FP32 lanes x 2 (FMA) x {sm_max:.0f} MHz"},
-            "model": "bytes and operations of the hit/miss links' walk",
+            "model": WORK_MODEL,
             "node_visits_per_ray": round(v_node, 3), "tri_tests_per_ray": round(v_tri, 3),
             "algorithmic_bytes_per_ray": round(bytes_ray, 1), "flops_per_ray": round(flops_ray, 1),
             "algorithmic_bytes_per_launch": int(round(bytes_ray * n)), "tiers": tiers}
+
+
+# What `achieved`, `frac` and `bound` of a roofline block are taken from.
+WORK_MODEL = ("bytes and operations of the hit/miss links' walk (32 bytes per box test) over the time of the walk that ran: a "
+              "rate of work held against HBM's rate, which may pass 1, not the memory traffic; the four-wide walk is bound by "
+              "instructions")
 
 
 # Work model of an SPPM pass (the measurement plan's per-pass figures): every traced ray as a
@@ -409,7 +419,7 @@ def sppm_work(c, npix, passes, adjoint=False):
 
 
 def work_roofline(nbytes, flops, seconds, rl, counts=None, parts=None, per=None):
-    """Roofline block of a whole workload: algorithmic bytes and flops over its measured time."""
+    """Roofline block of a whole workload: algorithmic bytes and flops (WORK_MODEL) over its measured time."""
     peaks, tiers, sm_count = rl["peaks"], rl["tiers"], rl["sm_count"]
     hbm = (peaks or {}).get("hbm_gbs") or FALLBACK_HBM_GBS
     fp32, _ = fp32_peak_tflops(sm_count, peaks)
@@ -420,7 +430,7 @@ def work_roofline(nbytes, flops, seconds, rl, counts=None, parts=None, per=None)
            "l2": {"peak": tiers["l2_peak_gbs"], "frac": round(achieved / tiers["l2_peak_gbs"], 4)},
            "fp32": {"achieved": round(flops / seconds / 1e12, 3), "peak": round(fp32, 2), "unit": "TFLOP/s",
                     "frac": round(flops / seconds / 1e12 / fp32, 4)},
-           "algorithmic_bytes": int(nbytes), "flops": int(flops)}
+           "algorithmic_bytes": int(nbytes), "flops": int(flops), "model": WORK_MODEL}
     if per:
         out["per"] = per
     if parts:

@@ -30,8 +30,9 @@ constexpr int kTraceChunk = GSP_TRACE_CHUNK;           // rays a warp takes from
 constexpr int kTraceInner = GSP_TRACE_INNER;           // traversal steps between refills
 constexpr int kTraceLeafBatch = GSP_TRACE_LEAF_BATCH;  // pending leaves that trigger a warp-wide leaf test
 constexpr int kWideStack = 64;     // children a walk of the four-wide tree may keep (at most three per wide level)
-constexpr int kPathChunk = GSP_PATH_CHUNK;  // paths a warp of the path kernels takes at once (a block's
-                                            // grid share is 128 paths: every warp of a short launch gets some)
+// most paths a warp of the path kernels takes at once (gsp_chunk); a launch has a block for every four paths (for
+// every 128 in a batch) up to what is resident, so that every warp of a short one gets some
+constexpr int kPathChunk = GSP_PATH_CHUNK;
 
 // Persistent grid size of the closest-hit kernel: SMs x resident blocks per SM.
 int gsp_trace_grid(int device);

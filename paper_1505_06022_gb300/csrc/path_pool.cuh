@@ -24,8 +24,9 @@
 #ifndef GSP_POOL
 #define GSP_POOL 44
 #endif
-// Resident blocks per SM: 72 registers without spills (8: 1 % slower, 6: 1 % faster in the batch, 1 %
-// slower at 512x512); with shading data 96 (6 spill: 1.50 against 1.41 ms).
+// Resident blocks per SM: 72 registers, without spills for one scene, 16 bytes for many (8: 1 % slower, 6: 1 %
+// faster in the batch, 1 % slower at 512x512); with shading data 96, none for one scene, 36 bytes for many (6 spill
+// for one: 1.50 against 1.41 ms).
 #ifndef GSP_POOL_MIN_BLOCKS
 #define GSP_POOL_MIN_BLOCKS 7
 #endif

@@ -78,8 +78,10 @@ struct gsp_sppm {
     // tracing stream, in arrays of the set's own: a small pass's gather is short, and four grid
     // launches before each one were a third of the chain that its passes wait for (four passes of
     // 64x64 pixels and 16,384 photons 436 -> 399 us). The arrays take 48 bytes per slot; for larger renderers
-    // that costs more (a gradient step that makes a renderer of 8.4 million slots: 5.65 -> 5.90 ms,
-    // 400 MB more to map) than it gives (512x512 passes of 2^20 photons 1.4 %).
+    // mapping them costs a renderer that is made for a few passes more (a gradient step that makes one of 8.4
+    // million slots: 5.65 -> 5.90 ms, 400 MB more) than they give. One that is made once and run long goes
+    // without the gain there: 1.42 -> 1.34 ms for four 333x217 passes of 262,144 photons with shading data (8.4
+    // million slots), 1.4 % at 512x512 with 2^20 (34 million).
     struct TraceBuf {
         float4 *hx = nullptr, *hn = nullptr, *hf = nullptr, *hd = nullptr, *slots = nullptr;
         uint32_t* pcount = nullptr;
@@ -817,8 +819,7 @@ static gsp_status sppm_one_pass(gsp_sppm* r, cudaStream_t st, bool graph = false
 // when only the longest paths are still going, and beside pass i's sort and gather (the sort goes to
 // the tracing stream where the set has a grid of its own). Events order
 // each set's reuse (and, with paths carried from pass to pass, the tracing itself); results are
-// those of one pass after the other. Exact hashing only (stochastic hashing shares its table
-// between the two halves).
+// those of one pass after the other. Stochastic passes overlap in the same way: each set has a table.
 static gsp_status passes_overlapped(gsp_sppm* r, int32_t npasses, cudaStream_t st) {
     // the tracing streams start after everything the caller queued before
     GSP_CUDA_TRY(cudaEventRecord(r->ev_start, st));

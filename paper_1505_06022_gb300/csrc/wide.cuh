@@ -95,7 +95,7 @@ struct WideWalk {
 // points to the lane's first), the others in the lane's local memory. The closest-hit kernel pops 1.5
 // times per node it tests, for four lanes of a warp at once; lanes at different depths make a local access
 // two L1 wavefronts a lane, beside the nodes' in a pipe that is busy 65 % of the time, but meet no bank
-// conflict in shared memory. K = 12 (the kernel's 60 KB of stacks per SM come out of the L1 cache):
+// conflict in shared memory. K = 12 (the 96 KB of an SM's 32 warps come out of the L1 cache):
 // 4,194,304 rays 643 -> 625 us, the random half alone 496 -> 474 us, 1,048,576 rays in host memory
 // 288 -> 279 us; 4 entries give 650 us, 8 628, 16 628, 20 633. The path kernels, whose path pools have
 // taken that shared memory, keep K = 0: with 4 or 8 a 512x512 pass is level and a 131x97 one 6 % slower.
