@@ -389,7 +389,7 @@ void bvh_host_walk(const HostBVH& bvh, const float* rays, int64_t n, int32_t* ou
                 tf = std::min(tf, std::max(t0, t1));
             }
             int32_t miss = as_int(A.w), word = as_int(B.w);
-            if (tn <= gsp_reach(std::min(tbest, tf))) {
+            if (tn <= gsp_reach<true>(std::min(tbest, tf))) {
                 if (word >= 0) {
                     int32_t first = word >> 3, cnt = word & 7;
                     for (int32_t k = 0; k < cnt; ++k) {

@@ -7,6 +7,7 @@
 #include <mutex>
 #include <new>
 #include <string>
+#include <type_traits>
 
 #include "devcommon.cuh"
 #include "gsp_internal.h"
@@ -197,7 +198,7 @@ k_trace_wide(DevScene S, const float4* __restrict__ rays, int64_t n, const uint3
     int32_t nlist = 0;  // warp-uniform, below 32 at the loop's head
     WarpQueue wq;
     wq.init((int32_t)n, chunk);
-    WideRay st;
+    RayHit st;
     st.slot = -1;
     WideWalk w;
     __shared__ int2 tops[kTraceThreads / 32][GSP_WIDE_TOP_TRACE * 32];
@@ -207,60 +208,67 @@ k_trace_wide(DevScene S, const float4* __restrict__ rays, int64_t n, const uint3
     w.sp = 0;
     int32_t ray = -1;
     bool quad = false;  // the last rays, four lanes to a ray
-    while (true) {
-        const int32_t got = quad ? -1 : wq.take(ray < 0, ctr);
-        if (got >= 0) {
-            ray = got;
-            const float4 a = __ldcs(rays + 2 * (int64_t)ray), b = __ldcs(rays + 2 * (int64_t)ray + 1);
-            wide_ray(f3(a), f3(b), a.w, b.w, st);
-            wide_init(w);
-        }
-        const uint32_t act = __ballot_sync(0xffffffffu, ray >= 0);
-        if (act == 0) break;
-        if (wq.done && __popc(act) == (quad ? 4 : 1)) {
-            st = coop_wide(S.wide, S.tris, st, w, stk, __ffs(act) - 1, &scratch[threadIdx.x >> 5]);
-            w.cur = kWalkDone;
-        } else if (!quad && wq.done && __popc(act) <= kQuadRays) {
-            quad = true;
-            const int src = quad_source(act);
-            quad_take(st, w, stk, src < 0 ? lane : src);
-            ray = __shfl_sync(0xffffffffu, ray, src < 0 ? lane : src);
-            if (src < 0) ray = -1;
-        } else if (quad)
-            quad_steps<GSP_WIDE_KEEP_TRACE>(S.wide, S.tris, st, w, stk, ray >= 0);
-        else
-            wide_steps(S.wide, S.tris, st, w, stk, ray >= 0, keep);
-        const bool fin = ray >= 0 && w.cur == kWalkDone;
-        bool flag = false;
-        if (fin && (!quad || (lane & 3) == 0)) {
-            float u = 0.0f, v = 0.0f;
-            if (st.slot >= 0)
-                flag = hit_needs_refine(S.tris + 3 * st.slot, st.o, st.d, st.tbest, refine_factor, uv != nullptr, u, v);
-            __stcs(tri + ray, out_slot ? st.slot : st.best);
-            __stcs(tout + ray, st.best >= 0 ? st.tbest : __int_as_float(0x7f800000));
-            if (uv) __stcs(uv + ray, make_float2(u, v));
-        }
-        const uint32_t fm = __ballot_sync(0xffffffffu, flag);
-        if (fm) {
-            if (LIST) {
-                const int leader = __ffs(fm) - 1;
-                unsigned long long b = 0;
-                if (lane == leader) b = atomicAdd(ctr + 1, (unsigned long long)__popc(fm));
-                b = __shfl_sync(0xffffffffu, b, leader);
-                if (flag) rlist[b + __popc(fm & lt)] = make_int2(ray, st.slot);
-            } else {
-                if (flag) list[nlist + __popc(fm & lt)] = make_int2(ray, st.slot);
-                nlist += __popc(fm);
-                __syncwarp();
-                if (nlist >= 32) {
-                    nlist -= 32;
-                    refine_listed(S, rays, list[nlist + lane], tout, uv);
+    // Takes and walks rays until none is left, or until one with a negative tmin is there.
+    const auto walk = [&](auto form) {
+        constexpr bool BEHIND = decltype(form)::value;
+        while (true) {
+            const int32_t got = quad ? -1 : wq.take(ray < 0, ctr);
+            if (got >= 0) {
+                ray = got;
+                const float4 a = __ldcs(rays + 2 * (int64_t)ray), b = __ldcs(rays + 2 * (int64_t)ray + 1);
+                wide_ray(f3(a), f3(b), a.w, b.w, st);
+                wide_init(w);
+            }
+            const uint32_t act = __ballot_sync(0xffffffffu, ray >= 0);
+            if (act == 0) return;
+            if (!BEHIND && __any_sync(0xffffffffu, got >= 0 && st.tmin < 0.0f)) return;
+            if (wq.done && __popc(act) == (quad ? 4 : 1)) {
+                st = coop_wide<BEHIND>(S.wide, S.tris, st, w, stk, __ffs(act) - 1, &scratch[threadIdx.x >> 5]);
+                w.cur = kWalkDone;
+            } else if (!quad && wq.done && __popc(act) <= kQuadRays) {
+                quad = true;
+                const int src = quad_source(act);
+                quad_take(st, w, stk, src < 0 ? lane : src);
+                ray = __shfl_sync(0xffffffffu, ray, src < 0 ? lane : src);
+                if (src < 0) ray = -1;
+            } else if (quad)
+                quad_steps<GSP_WIDE_KEEP_TRACE, BEHIND>(S.wide, S.tris, st, w, stk, ray >= 0);
+            else
+                wide_steps<BEHIND>(S.wide, S.tris, st, w, stk, ray >= 0, keep);
+            const bool fin = ray >= 0 && w.cur == kWalkDone;
+            bool flag = false;
+            if (fin && (!quad || (lane & 3) == 0)) {
+                float u = 0.0f, v = 0.0f;
+                if (st.slot >= 0)
+                    flag = hit_needs_refine(S.tris + 3 * st.slot, st.o, st.d, st.tbest, refine_factor, uv != nullptr, u, v);
+                __stcs(tri + ray, out_slot ? st.slot : st.best);
+                __stcs(tout + ray, st.best >= 0 ? st.tbest : __int_as_float(0x7f800000));
+                if (uv) __stcs(uv + ray, make_float2(u, v));
+            }
+            const uint32_t fm = __ballot_sync(0xffffffffu, flag);
+            if (fm) {
+                if (LIST) {
+                    const int leader = __ffs(fm) - 1;
+                    unsigned long long b = 0;
+                    if (lane == leader) b = atomicAdd(ctr + 1, (unsigned long long)__popc(fm));
+                    b = __shfl_sync(0xffffffffu, b, leader);
+                    if (flag) rlist[b + __popc(fm & lt)] = make_int2(ray, st.slot);
+                } else {
+                    if (flag) list[nlist + __popc(fm & lt)] = make_int2(ray, st.slot);
+                    nlist += __popc(fm);
                     __syncwarp();
+                    if (nlist >= 32) {
+                        nlist -= 32;
+                        refine_listed(S, rays, list[nlist + lane], tout, uv);
+                        __syncwarp();
+                    }
                 }
             }
+            if (fin) ray = -1;
         }
-        if (fin) ray = -1;
-    }
+    };
+    walk(std::false_type{});
+    walk(std::true_type{});  // what is left then, in the form that such rays ask for (wide.cuh)
     if (!LIST && lane < nlist) refine_listed(S, rays, list[lane], tout, uv);
 }
 

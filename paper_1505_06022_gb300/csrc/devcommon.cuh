@@ -458,7 +458,7 @@ __device__ __forceinline__ bool slab(const RayHit& st, float3 lo, float3 hi, flo
     const float t0z = __fmul_rn(lo.z - o.z, inv.z), t1z = __fmul_rn(hi.z - o.z, inv.z);
     tn = max3f(fminf(t0x, t1x), fminf(t0y, t1y), fmaxf(fminf(t0z, t1z), st.tmin));
     const float tf = min3f(fmaxf(t0x, t1x), fmaxf(t0y, t1y), fmaxf(t0z, t1z));
-    return tn <= gsp_reach(fminf(st.tbest, tf));
+    return tn <= gsp_reach<true>(fminf(st.tbest, tf));
 }
 
 // Box test of a node {A, B} = {min.xyz, miss | max.xyz, leaf word} against [tmin, best t].

@@ -44,24 +44,31 @@ struct HostBVH {
 #endif
 
 // The far end x of an interval of box distances, moved out by 2^-19 of its size: what the rounding of a
-// box test is covered by (wide.cuh). The slack follows the sign of x, which a factor would not, and is
+// box test is covered by (wide.cuh). BEHIND: the slack follows the sign of x, which a factor would not, and is
 // relative, so that it is as good behind the origin (a negative tmin) as in front of it; +inf stays, and
-// -inf gives a NaN, which no entry distance is at or below.
-GSP_HOST_DEVICE inline float gsp_reach(float x) { return x + fabsf(x) * 0x1p-19f; }
+// -inf gives a NaN, which no entry distance is at or below. Otherwise only an x that is not negative counts
+// (the entry distances compared with it are not), and one product does.
+template <bool BEHIND>
+GSP_HOST_DEVICE inline float gsp_reach(float x) {
+    return BEHIND ? x + fabsf(x) * 0x1p-19f : x * (1.0f + 0x1p-19f);
+}
 
-// The same where only an x that is not negative counts (what is compared with it is not): one product.
-GSP_HOST_DEVICE inline float gsp_reach_ahead(float x) { return x * (1.0f + 0x1p-19f); }
+// The bits of an entry distance as an integer in the order of the distances (-0 below +0): as they are, or
+// where there can be negative ones (BEHIND) with the order of those turned round.
+template <bool BEHIND>
+GSP_HOST_DEVICE inline int32_t gsp_wide_order(float t) {
+    int32_t i;
+    memcpy(&i, &t, sizeof i);
+    return BEHIND ? i ^ ((i >> 31) & 0x7fffffff) : i;
+}
 
-// Whether a child of the four-wide tree put by with this key (its entry distance, the two low bits
-// replaced; wide.cuh) may still hold a closer hit, by the rule it was put by with: where surfaces coincide,
-// a triangle's t can be below its box's entry distance by the rounding of either, and without the slack the
-// winner of a tie would depend on the order of the walk. Dropping the low bits rounds a distance down unless
-// it is negative (negative tmin, origin inside the box): never culled then.
+// Whether a child of the four-wide tree put by with this key (its entry distance in gsp_wide_order, the two
+// low bits replaced, which rounds it down) may still hold a closer hit, by the rule it was put by with: where
+// surfaces coincide, a triangle's t can be below its box's entry distance by the rounding of either, and
+// without the slack the winner of a tie would depend on the order of the walk.
+template <bool BEHIND>
 GSP_HOST_DEVICE inline bool gsp_wide_keep(int32_t key, float tbest) {
-    const int32_t bits = key & ~3;
-    float t;
-    memcpy(&t, &bits, sizeof t);
-    return key < 0 || t <= gsp_reach_ahead(tbest);
+    return (key & ~3) <= gsp_wide_order<BEHIND>(gsp_reach<BEHIND>(tbest) + 0.0f);  // -0 counts as +0
 }
 
 // Centre and half extent of an interval of the four-wide tree's boxes: c - h <= lo and hi <= c + h

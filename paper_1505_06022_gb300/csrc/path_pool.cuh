@@ -155,7 +155,7 @@ k_paths_pool(const __grid_constant__ PathJob one, const PathJob* __restrict__ jo
     }
     __syncwarp();
     int nready = 0, ndone = pool;
-    PathRay st;
+    RayHit st;
     WideWalk w;
     int2 deep[kWideStack];
     const WideStack<0> stk{deep, nullptr};
@@ -242,7 +242,7 @@ k_paths_pool(const __grid_constant__ PathJob one, const PathJob* __restrict__ jo
         }
         if (busy == 0) break;
         if ((MULTI ? mq.done : wq.done) && nready == 0 && ndone == 0 && busy <= kQuadRays) break;
-        wide_steps(wide, tris, st, w, stk, at >= 0, nready ? GSP_POOL_KEEP_READY : GSP_POOL_KEEP_DRY);
+        wide_steps<false>(wide, tris, st, w, stk, at >= 0, nready ? GSP_POOL_KEEP_READY : GSP_POOL_KEEP_DRY);
         const bool fin = at >= 0 && w.cur == kWalkDone;
         const uint32_t fm = __ballot_sync(F, fin);
         if (fin) {
@@ -279,10 +279,10 @@ k_paths_pool(const __grid_constant__ PathJob one, const PathJob* __restrict__ jo
                 wide = (const float4*)__shfl_sync(F, (unsigned long long)wide, owner);
                 tris = (const float4*)__shfl_sync(F, (unsigned long long)tris, owner);
             }
-            st = coop_wide(wide, tris, st, w, stk, owner, &scratch[threadIdx.x >> 5]);
+            st = coop_wide<false>(wide, tris, st, w, stk, owner, &scratch[threadIdx.x >> 5]);
             w.cur = kWalkDone;
         } else {
-            quad_steps<GSP_WIDE_KEEP>(wide, tris, st, w, stk, at >= 0);
+            quad_steps<GSP_WIDE_KEEP, false>(wide, tris, st, w, stk, at >= 0);
         }
         const bool fin = at >= 0 && w.cur == kWalkDone;
         float3 o = st.o, d = st.d, v = make_float3(0.0f, 0.0f, 0.0f);

@@ -224,7 +224,7 @@ static __device__ __noinline__ CoopWalk coop_walk(const float4* __restrict__ tri
             if (++st.steps > cap) {
                 if (lane == owner) report(status, -4);
                 cur = -1;
-            } else if (((hm >> k) & 1u) && tk <= gsp_reach(st.tbest)) {
+            } else if (((hm >> k) & 1u) && tk <= gsp_reach<true>(st.tbest)) {
                 if (wk >= 0) {
                     coop_leaf(tris, st, wk >> 3, wk & 7);
                     ntri += (uint32_t)(wk & 7);
@@ -262,7 +262,7 @@ __device__ __forceinline__ void stack_init(const DevScene& S, StackWalk& w) {
 __device__ __forceinline__ int32_t stack_pop(const Trav& st, StackWalk& w) {
     while (w.sp > 0) {
         --w.sp;
-        if (w.stk_t[w.sp] <= gsp_reach(st.tbest)) return w.stk_node[w.sp];  // ties may still hold a smaller index
+        if (w.stk_t[w.sp] <= gsp_reach<true>(st.tbest)) return w.stk_node[w.sp];  // ties may still hold a smaller index
     }
     return kWalkDone;
 }

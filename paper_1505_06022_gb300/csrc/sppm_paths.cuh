@@ -308,7 +308,7 @@ struct PathWalk<kStack> {
 
 template <>
 struct PathWalk<kWide> {
-    PathRay st;
+    RayHit st;
     WideWalk w;
     int2 stk[kWideStack];
     __device__ __forceinline__ PathWalk() {
@@ -321,10 +321,10 @@ struct PathWalk<kWide> {
         wide_init(w);
     }
     __device__ __forceinline__ void steps(const DevScene& S, bool active, int32_t, uint32_t&) {
-        wide_steps(S.wide, S.tris, st, w, WideStack<0>{stk, nullptr}, active, GSP_WIDE_KEEP);
+        wide_steps<false>(S.wide, S.tris, st, w, WideStack<0>{stk, nullptr}, active, GSP_WIDE_KEEP);
     }
     __device__ __forceinline__ void quad_steps(const DevScene& S, bool active) {
-        gspd::quad_steps<GSP_WIDE_KEEP>(S.wide, S.tris, st, w, WideStack<0>{stk, nullptr}, active);
+        gspd::quad_steps<GSP_WIDE_KEEP, false>(S.wide, S.tris, st, w, WideStack<0>{stk, nullptr}, active);
     }
     __device__ __forceinline__ bool done() const { return w.cur == kWalkDone; }
 };

@@ -59,13 +59,14 @@ constexpr int kWideLeafBatch = GSP_WIDE_LEAF_BATCH;  // lanes at a leaf that tri
 // once had, lets every box through when |tmin| is large against the scene: 683 instead of 14 nodes per
 // line through 2,000 triangles at tmin = -FLT_MAX.) Two operations of the half-rate min/max pipe fewer
 // per axis and box than min and max over the two planes: that pipe was the busiest at 57-61 % of its cycles.
-struct WideRay : RayHit {};
-// A path's ray, whose tmin is not negative: one product does (an FMA has no absolute value of its own; two
-// operations per box instead of one: 4,194,304 rays 575 -> 581 us, the batch of 16 scenes 5.11 -> 5.14 ms).
-struct PathRay : RayHit {};
 
-__device__ __forceinline__ float wide_far(const WideRay&, float x) { return gsp_reach(x); }
-__device__ __forceinline__ float wide_far(const PathRay&, float x) { return gsp_reach_ahead(x); }
+// BEHIND: the form of the rules for rays with a negative tmin (gsp_reach, gsp_wide_order, gsp_wide_keep). A warp of the
+// closest-hit kernel changes to it with its first such ray; the rays beside and after that one may be of either
+// kind. In one form for all, the far end would cost every ray an operation per box (an FMA has no absolute value
+// of its own; 4,194,304 rays 575 -> 581 us) and the order of negative distances two; the two forms chosen anew
+// in every round of the loop cost 2 % (577 -> 590). Without that order, rays behind their origin visited their
+// boxes farthest first and dropped none from the stack: 1,048,576 lines through 20,000 triangles 1,338 us, with
+// it 684 (917 along the links), through 1,003,520 triangles 608 and 450 (722).
 
 // 1 / d to 1 ulp (2u): all that the slab test needs.
 __device__ __forceinline__ float wide_inv(float d) {
@@ -122,26 +123,26 @@ __device__ __forceinline__ void wide_init(WideWalk& w) {
 
 constexpr int32_t kWideMiss = 0x7fffffff;  // sorts behind every key
 
-template <class Stack>
+template <bool BEHIND, class Stack>
 __device__ __forceinline__ int32_t wide_pop(const RayHit& st, WideWalk& w, const Stack& stk) {
     while (w.sp > 0) {
         const int2 e = stk.get(--w.sp);
-        if (gsp_wide_keep(e.x, st.tbest)) return e.y;
+        if (gsp_wide_keep<BEHIND>(e.x, st.tbest)) return e.y;
     }
     return kWalkDone;
 }
 
-// Key of child i: the bits of its entry distance with the child number in the two low bits, or
-// kWideMiss. Signed order is the order of the distances where they are not negative.
-template <class Ray>
-__device__ __forceinline__ int32_t wide_key(const Ray& st, float cx, float hx, float cy, float hy, float cz,
+// Key of child i: its entry distance as an integer in the same order, with the child number in the two low
+// bits, or kWideMiss.
+template <bool BEHIND>
+__device__ __forceinline__ int32_t wide_key(const RayHit& st, float cx, float hx, float cy, float hy, float cz,
                                             float hz, int i) {
     const float tx = __fmul_rn(cx - st.o.x, st.inv.x), ty = __fmul_rn(cy - st.o.y, st.inv.y),
                 tz = __fmul_rn(cz - st.o.z, st.inv.z);
     const float ax = fabsf(st.inv.x), ay = fabsf(st.inv.y), az = fabsf(st.inv.z);
     const float tn = max3f(__fmaf_rn(-hx, ax, tx), __fmaf_rn(-hy, ay, ty), fmaxf(__fmaf_rn(-hz, az, tz), st.tmin));
     const float tf = min3f(__fmaf_rn(hx, ax, tx), __fmaf_rn(hy, ay, ty), __fmaf_rn(hz, az, tz));
-    return tn <= wide_far(st, fminf(st.tbest, tf)) ? ((__float_as_int(tn) & ~3) | i) : kWideMiss;
+    return tn <= gsp_reach<BEHIND>(fminf(st.tbest, tf)) ? ((gsp_wide_order<BEHIND>(tn) & ~3) | i) : kWideMiss;
 }
 
 template <class Stack>
@@ -151,12 +152,12 @@ __device__ __forceinline__ void wide_push(WideWalk& w, const Stack& stk, int32_t
 
 // Moves to the nearest of the children hit; the others go on the stack as they come (sorting them
 // too saves under 1 % of the visits and costs more).
-template <class Stack>
+template <bool BEHIND, class Stack>
 __device__ __forceinline__ void wide_next(int32_t k0, int32_t k1, int32_t k2, int32_t k3, int4 ref, const RayHit& st,
                                           WideWalk& w, const Stack& stk) {
     const int32_t k = min(min(k0, k1), min(k2, k3));
     if (k == kWideMiss) {
-        w.cur = wide_pop(st, w, stk);
+        w.cur = wide_pop<BEHIND>(st, w, stk);
         return;
     }
     wide_push(w, stk, k0, k, ref.x);
@@ -168,8 +169,8 @@ __device__ __forceinline__ void wide_next(int32_t k0, int32_t k1, int32_t k2, in
 }
 
 // Tests the four children of node w.cur and moves on.
-template <class Ray, class Stack>
-__device__ __forceinline__ void wide_node(const float4* __restrict__ nodes, const Ray& st, WideWalk& w,
+template <bool BEHIND, class Stack>
+__device__ __forceinline__ void wide_node(const float4* __restrict__ nodes, const RayHit& st, WideWalk& w,
                                           const Stack& stk) {
     const float4* p = nodes + 8 * (int64_t)w.cur;
     float4 cx, hx, cy, hy, cz, hz;
@@ -177,11 +178,11 @@ __device__ __forceinline__ void wide_node(const float4* __restrict__ nodes, cons
     ldg32(p + 2, cy, hy);
     ldg32(p + 4, cz, hz);
     const int4 ref = __ldg((const int4*)(p + 6));
-    const int32_t k0 = wide_key(st, cx.x, hx.x, cy.x, hy.x, cz.x, hz.x, 0);
-    const int32_t k1 = wide_key(st, cx.y, hx.y, cy.y, hy.y, cz.y, hz.y, 1);
-    const int32_t k2 = wide_key(st, cx.z, hx.z, cy.z, hy.z, cz.z, hz.z, 2);
-    const int32_t k3 = wide_key(st, cx.w, hx.w, cy.w, hy.w, cz.w, hz.w, 3);
-    wide_next(k0, k1, k2, k3, ref, st, w, stk);
+    const int32_t k0 = wide_key<BEHIND>(st, cx.x, hx.x, cy.x, hy.x, cz.x, hz.x, 0);
+    const int32_t k1 = wide_key<BEHIND>(st, cx.y, hx.y, cy.y, hy.y, cz.y, hz.y, 1);
+    const int32_t k2 = wide_key<BEHIND>(st, cx.z, hx.z, cy.z, hy.z, cz.z, hz.z, 2);
+    const int32_t k3 = wide_key<BEHIND>(st, cx.w, hx.w, cy.w, hy.w, cz.w, hz.w, 3);
+    wide_next<BEHIND>(k0, k1, k2, k3, ref, st, w, stk);
 }
 
 // Walks the warp's active lanes until no more than `keep` quarters of them still walk: what follows a
@@ -192,20 +193,20 @@ __device__ __forceinline__ void wide_node(const float4* __restrict__ nodes, cons
 // the link (4,194,304 of them 4,607 Mrays/s, 4,514 with 3).
 // Lanes at a leaf wait until kWideLeafBatch of them are, or no lane
 // has a node left to test, and test their leaves together (12; 8 costs 1-2 %, 4 costs 5 %).
-template <class Ray, class Stack>
-__device__ __forceinline__ void wide_steps(const float4* __restrict__ wide, const float4* __restrict__ tris, Ray& st,
+template <bool BEHIND, class Stack>
+__device__ __forceinline__ void wide_steps(const float4* __restrict__ wide, const float4* __restrict__ tris, RayHit& st,
                                            WideWalk& w, const Stack& stk, bool active, int keep) {
     const int stop = (__popc(__ballot_sync(0xffffffffu, active)) * keep) >> 2;
     uint32_t nm, lm;
     do {
-        if (active && w.cur >= 0) wide_node(wide, st, w, stk);
+        if (active && w.cur >= 0) wide_node<BEHIND>(wide, st, w, stk);
         const bool leaf = active && w.cur < 0 && w.cur != kWalkDone;
         lm = __ballot_sync(0xffffffffu, leaf);
         nm = __ballot_sync(0xffffffffu, active && w.cur >= 0);
         if (lm && (!nm || __popc(lm) >= kWideLeafBatch)) {
             if (leaf) {
                 trav_leaf(tris, st, (~w.cur) >> 3, (~w.cur) & 7);
-                w.cur = wide_pop(st, w, stk);
+                w.cur = wide_pop<BEHIND>(st, w, stk);
             }
             lm = __ballot_sync(0xffffffffu, active && w.cur != kWalkDone);
         }
@@ -256,8 +257,8 @@ __device__ __forceinline__ void quad_take(RayHit& st, WideWalk& w, const Stack& 
 }
 
 // As wide_steps, for groups of four lanes; `active` is the same in the lanes of a group.
-template <int KEEP, class Ray, class Stack>
-__device__ __forceinline__ void quad_steps(const float4* __restrict__ wide, const float4* __restrict__ tris, Ray& st,
+template <int KEEP, bool BEHIND, class Stack>
+__device__ __forceinline__ void quad_steps(const float4* __restrict__ wide, const float4* __restrict__ tris, RayHit& st,
                                            WideWalk& w, const Stack& stk, bool active) {
     const uint32_t F = 0xffffffffu;
     const int c = threadIdx.x & 3;
@@ -268,14 +269,14 @@ __device__ __forceinline__ void quad_steps(const float4* __restrict__ wide, cons
         int32_t key = kWideMiss, ref = kWalkDone;
         if (node) {
             const float* q = (const float*)(wide + 8 * (int64_t)w.cur) + c;
-            key = wide_key(st, __ldg(q), __ldg(q + 4), __ldg(q + 8), __ldg(q + 12), __ldg(q + 16), __ldg(q + 20), c);
+            key = wide_key<BEHIND>(st, __ldg(q), __ldg(q + 4), __ldg(q + 8), __ldg(q + 12), __ldg(q + 16), __ldg(q + 20), c);
             ref = __ldg((const int32_t*)q + 24);
         }
         const int32_t k0 = __shfl_sync(F, key, 0, 4), k1 = __shfl_sync(F, key, 1, 4), k2 = __shfl_sync(F, key, 2, 4),
                       k3 = __shfl_sync(F, key, 3, 4);
         const int4 r = make_int4(__shfl_sync(F, ref, 0, 4), __shfl_sync(F, ref, 1, 4), __shfl_sync(F, ref, 2, 4),
                                  __shfl_sync(F, ref, 3, 4));
-        if (node) wide_next(k0, k1, k2, k3, r, st, w, stk);
+        if (node) wide_next<BEHIND>(k0, k1, k2, k3, r, st, w, stk);
         const bool leaf = active && w.cur < 0 && w.cur != kWalkDone;
         if (__ballot_sync(F, leaf)) {
             const int32_t word = leaf ? ~w.cur : 0;  // 0: no triangles
@@ -310,7 +311,7 @@ __device__ __forceinline__ void quad_steps(const float4* __restrict__ wide, cons
                     st.best = id;
                     st.slot = slot;
                 }
-                w.cur = wide_pop(st, w, stk);
+                w.cur = wide_pop<BEHIND>(st, w, stk);
             }
         }
         walking = __ballot_sync(F, active && w.cur != kWalkDone);
@@ -333,9 +334,9 @@ static_assert(kCoopNarrow + 24 + 3 * (kWideMaxDepth / 2 + 1) < kCoopStack && kWi
 
 // Walks lane owner's ray (st, w and stk are that lane's) to its end; every lane calls it and
 // receives the ray with its final best hit. Not inlined: the callers' loops keep their registers.
-template <class Ray, class Stack>
-__device__ __noinline__ Ray coop_wide(const float4* __restrict__ wide, const float4* __restrict__ tris, Ray st,
-                                      WideWalk w, Stack stk, int owner, CoopScratch* sc) {
+template <bool BEHIND, class Stack>
+__device__ __noinline__ RayHit coop_wide(const float4* __restrict__ wide, const float4* __restrict__ tris, RayHit st,
+                                         WideWalk w, Stack stk, int owner, CoopScratch* sc) {
     const uint32_t F = 0xffffffffu;
     const int lane = threadIdx.x & 31, slot = lane >> 2, c = lane & 3;
     const uint32_t lt = lanemask_lt();
@@ -349,7 +350,7 @@ __device__ __noinline__ Ray coop_wide(const float4* __restrict__ wide, const flo
     int n = __shfl_sync(F, w.sp, owner) + 1;
     if (lane == owner) {
         for (int i = 0; i < n - 1; ++i) sc->stk[i] = stk.get(i);
-        sc->stk[n - 1] = make_int2(-1, w.cur);  // a negative key: not culled
+        sc->stk[n - 1] = make_int2(INT32_MIN, w.cur);  // the least key: kept
     }
     __syncwarp();
     while (n > 0) {
@@ -358,10 +359,10 @@ __device__ __noinline__ Ray coop_wide(const float4* __restrict__ wide, const flo
         if (slot < take) e = sc->stk[n - 1 - slot];
         n -= take;
         int32_t key = kWideMiss, ref = kWalkDone;
-        if (e.y != kWalkDone && gsp_wide_keep(e.x, st.tbest)) {
+        if (e.y != kWalkDone && gsp_wide_keep<BEHIND>(e.x, st.tbest)) {
             if (e.y >= 0) {
                 const float* q = (const float*)(wide + 8 * (int64_t)e.y) + c;
-                key = wide_key(st, __ldg(q), __ldg(q + 4), __ldg(q + 8), __ldg(q + 12), __ldg(q + 16), __ldg(q + 20), c);
+                key = wide_key<BEHIND>(st, __ldg(q), __ldg(q + 4), __ldg(q + 8), __ldg(q + 12), __ldg(q + 16), __ldg(q + 20), c);
                 ref = __ldg((const int32_t*)q + 24);
             } else if (c == 0) {
                 key = e.x & ~3;

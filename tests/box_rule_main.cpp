@@ -48,6 +48,7 @@ static void test_tri(const float4* tri, const float* r, Best& b) {
     if (u >= 0 && v >= 0 && u + v <= 1 && t > r[3] && (t < b.t || (t == b.t && b.id >= 0 && id < b.id))) b = {t, id};
 }
 
+template <bool BEHIND>
 static Best walk(const HostBVH& b, const std::vector<float4>& wide, const float* r, int ulp, int64_t& nodes) {
     const float *W = (const float*)wide.data(), *d = r + 4;
     float inv[3];
@@ -59,7 +60,7 @@ static Best walk(const HostBVH& b, const std::vector<float4>& wide, const float*
     const auto pop = [&] {
         while (sp > 0) {
             --sp;
-            if (gsp_wide_keep(stk[sp].key, best.t)) return stk[sp].ref;
+            if (gsp_wide_keep<BEHIND>(stk[sp].key, best.t)) return stk[sp].ref;
         }
         return kNone;
     };
@@ -79,7 +80,7 @@ static Best walk(const HostBVH& b, const std::vector<float4>& wide, const float*
                 tn = std::fmax(tn, std::fmaf(-h, a, tc));
                 tf = std::fmin(tf, std::fmaf(h, a, tc));
             }
-            key[c] = tn <= gsp_reach(std::fmin(best.t, tf)) ? ((as_int(tn) & ~3) | c) : kMiss;
+            key[c] = tn <= gsp_reach<BEHIND>(std::fmin(best.t, tf)) ? ((gsp_wide_order<BEHIND>(tn) & ~3) | c) : kMiss;
             nearest = std::min(nearest, key[c]);
         }
         if (nearest == kMiss) {
@@ -111,7 +112,7 @@ static int check(const char* name, const Mesh& m, int nr, float at, float size, 
     int bad = 0;
     // -16 size / len: behind everything that a ray's line meets
     const float behind = -16.0f * size / len;
-    int64_t cost[6] = {};
+    int64_t cost[6] = {}, line = 0, moved = 0;
     const float tmins[6] = {0.0f, behind / 16, behind, 1e6f * behind, -FLT_MAX, -INFINITY};
     for (int j = 0; j < 6; ++j) {
         std::mt19937 g(nt);
@@ -139,12 +140,27 @@ static int check(const char* name, const Mesh& m, int nr, float at, float size, 
                 wrong += got.id != want.id || (want.id >= 0 && got.t != want.t);
             }
             for (int ulp = -1; ulp <= 1 && !links; ++ulp) {
-                const Best got = walk(b, wide, r, ulp, cost[j]);
+                const Best got = walk<true>(b, wide, r, ulp, cost[j]);
                 wrong += got.id != want.id || (want.id >= 0 && got.t != want.t);
+                if (tmins[j] < 0) continue;
+                int64_t nodes = 0;  // the rays in front of the origin have a form of the rules of their own
+                const Best ahead = walk<false>(b, wide, r, ulp, nodes);
+                wrong += ahead.id != got.id || (got.id >= 0 && ahead.t != got.t);
+            }
+            if (j == 2 && !links) {  // the same line from where it starts
+                walk<true>(b, wide, r, 0, line);
+                for (int k = 0; k < 3; ++k) r[k] += behind * r[4 + k];
+                r[3] = 0.0f;
+                r[7] -= behind;
+                walk<false>(b, wide, r, 0, moved);
             }
         }
         if (wrong || !hits) std::printf("%s, direction %g, tmin %g: %d of %d walks wrong, %d hits\n", name, len, tmins[j], wrong, links ? nr : 3 * nr, hits);
         bad += wrong + !hits;
+    }
+    if (line > 1.05 * moved) {  // the nearest box first and the far ones dropped, behind the origin too
+        std::printf("%s, direction %g: %lld nodes from behind, %lld from a start there\n", name, len, (long long)line, (long long)moved);
+        ++bad;
     }
     for (int j = 3; j < 6; ++j)  // the boxes a line meets do not depend on where far behind it starts
         if (cost[j] > 1.05 * cost[2]) {

@@ -75,3 +75,24 @@ def test_closest_hits(make, builder, length):
             assert torch.equal(s.trace(rays[:n])[0], want[:n]), (tmin, n)
     ctx.sync()
     ctx.close()
+
+
+@pytest.mark.parametrize("every", [2, 7, 400])
+@pytest.mark.parametrize("n", [33, 9001, 700_000])
+def test_among_other_rays(every, n):
+    """Every second, seventh or 400th ray starts behind its origin: warps that change to the form of the walk for
+    such rays, at their first rays and in between, give every ray the hit it has alone."""
+    ctx = gsp.Context(0)
+    s = gsp.Scene(ctx, I.random_soup(3000, seed=2, size=0.1))
+    rays = torch.from_numpy(I.random_rays(n, seed=9)).cuda()
+    ahead = s.trace(rays)
+    rays[:, 3] = -2.0
+    behind = s.trace(rays)
+    some = torch.zeros(n, dtype=torch.bool, device="cuda")
+    some[every - 1::every] = True
+    rays[:, 3] = torch.where(some, -2.0, 0.0)
+    mixed = s.trace(rays)
+    for a, b, m in zip(ahead, behind, mixed):
+        assert torch.equal(torch.where(some, b, a), m)
+    ctx.sync()
+    ctx.close()
