@@ -288,8 +288,7 @@ constexpr int64_t kGatherWideBelow = 256 * 256;
 template <int L>
 __global__ void __launch_bounds__(128) k_gather_exact(GatherDev G, PassDev P) {
     static_assert(L >= 1 && L <= 32 && (L & (L - 1)) == 0, "group size");
-    release_next();
-    wait_previous();
+    wait_previous();  // and no release_next(): k_gather_heavy says why
     const int gl = threadIdx.x & (L - 1);
     const int64_t p = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / L;
     if (G.total && blockIdx.x == 0 && threadIdx.x == 0) *G.total = G.bstart[(size_t)P.tmask + 1];
@@ -335,7 +334,9 @@ __global__ void __launch_bounds__(128) k_gather_exact(GatherDev G, PassDev P) {
 // The listed heavy queries, a block of kHeavyThreads per hit point (persistent over the list):
 // the same lane split as k_gather_exact with kHeavyThreads lanes, lane sums combined by a fixed
 // butterfly in each warp and then warp by warp in order, so the result does not depend on
-// scheduling either.
+// scheduling either. Two blocks per SM, which hold if they are placed on an empty chip: started while the last
+// blocks of k_gather_exact run, they crowd onto the SMs that fall free first and stay there (512x512 renders that
+// spend most of a pass here: 13.9 -> 12.6 ms and 8.4 -> 7.6 ms a pass without that start; others level).
 constexpr int kHeavyThreads = 256;
 
 __global__ void __launch_bounds__(kHeavyThreads) k_gather_heavy(GatherDev G, PassDev P) {
