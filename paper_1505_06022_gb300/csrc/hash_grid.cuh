@@ -11,7 +11,7 @@
 // A least-significant-digit radix sort (scan_sort.cu) takes five launches per eight bits, a scan for
 // the compaction, one for the bucket starts, and an atomic per point for their counts: 17 to 25
 // launches of a few microseconds each, on the critical path of a small pass. Here the starts fall out
-// of the last step. Measured: 1,000,003 points in 2^21 buckets 152 -> 59.5 us; a 131x97 pass of 65,536
+// of the last step. Measured: 1,000,003 points in 2^21 buckets 152 -> 56 us; a 131x97 pass of 65,536
 // photons 387 -> 303 us, four passes of the 64x64 Cornell box 625 -> 470 us, in each the launches saved
 // times the few microseconds of a dependent one.
 // Every step is ordered by counts and scans alone, so the result does not depend on scheduling.
@@ -48,6 +48,7 @@ constexpr int kGridList = 4096;      // points of a tile whose list k_grid_tiles
 constexpr int kGridItems = 12;       // points per lane that k_grid_split holds in registers
 constexpr int kGridSegment = kGridWarps * 32 * kGridItems;  // and so ranks at once (16-bit counters)
 constexpr int kPartItems = 4;        // the same for k_grid_parts; larger parts are read again
+constexpr int kPartAhead = 8;        // points per lane of a larger part that are fetched at once
 constexpr int kScanThreads = 1024;   // of k_grid_scan
 
 // How a grid of `items` inputs and 2^bits buckets is split.
@@ -302,7 +303,10 @@ k_grid_split(GridIn in, GridPlan plan, GridBuf buf, uint32_t* __restrict__ clear
 }
 
 // One part: sorted by the low bits of the bucket number as k_grid_split sorts a tile, but with the
-// counts turned into bucket starts. Writes whichever of these is asked for: the order, the records in
+// counts turned into bucket starts. A part is one block's work however many points crowd into it, so a larger
+// one than the lanes hold is fetched kPartAhead points per lane at once, counted without ranking, and its points
+// are placed before any is moved: 1,000,003 points in one bucket 2,220 -> 758 us (745 with radix passes over
+// them), spread over some hundred 1,040 -> 362 (410), over 2^21 60.5 -> 56.1. Writes whichever of these is asked for: the order, the records in
 // that order (positions and payloads), and the bucket starts (the last part also the end).
 __global__ void __launch_bounds__(kGridThreads)
 k_grid_parts(GridIn in, GridPlan plan, GridBuf buf, uint32_t* __restrict__ order, float4* __restrict__ spos,
@@ -336,17 +340,20 @@ k_grid_parts(GridIn in, GridPlan plan, GridBuf buf, uint32_t* __restrict__ order
     }
     for (int b = lane; b < nb; b += 32) s_count[warp][b] = 0;
     __syncwarp();
-    const auto count = [&](uint32_t b) {
-        const uint32_t peers = __match_any_sync(0xffffffffu, b);
-        if (b != 0xffffffffu && (peers & lt) == 0) s_count[warp][b] += __popc(peers);
-        __syncwarp();
+    const auto count = [&](uint32_t b) {  // in any order; lanes that add to one counter are combined by the hardware
+        if (b != 0xffffffffu) atomicAdd(&s_count[warp][b], 1u);
     };
     if (held) {
 #pragma unroll
-        for (int j = 0; j < kPartItems; ++j)
-            if (e0 + 32 * j < e1) count(own[j].x);
+        for (int j = 0; j < kPartItems; ++j) count(own[j].x);
     } else {
-        for (uint32_t e = e0; e < e1; e += 32) count(point(e + lane).x);
+        for (uint32_t e = e0; e < e1; e += 32 * kPartAhead) {
+            uint32_t b[kPartAhead];
+#pragma unroll
+            for (int j = 0; j < kPartAhead; ++j) b[j] = point(e + 32 * j + lane).x;
+#pragma unroll
+            for (int j = 0; j < kPartAhead; ++j) count(b[j]);
+        }
     }
     __syncthreads();
     // bucket starts: sums over the warps, then over the buckets (four consecutive ones per thread)
@@ -385,31 +392,43 @@ k_grid_parts(GridIn in, GridPlan plan, GridBuf buf, uint32_t* __restrict__ order
         }
     }
     __syncthreads();
-    const auto place = [&](uint2 pt) {
-        const uint32_t b = pt.x, v = pt.y;
-        const uint32_t peers = __match_any_sync(0xffffffffu, b), rank = __popc(peers & lt);
+    // the place of each of 32 lanes' points, in order; then the records move there
+    const auto place = [&](const uint32_t b, const uint32_t peers) {
         const bool on = b != 0xffffffffu;
         const uint32_t off = on ? s_count[warp][b] : 0u;
         __syncwarp();
-        if (on) {
-            const uint32_t to = off + rank;
-            if (order) order[to] = v;
-            if (spos) {
-                const float4 x = __ldg(in.pos + 2 * (size_t)v), y = __ldg(in.pos + 2 * (size_t)v + 1);
-                spos[to] = x;
-                spay[to] = y;
-            }
-            if (rank == 0) s_count[warp][b] = off + __popc(peers);
-        }
+        if (on && (peers & lt) == 0) s_count[warp][b] = off + __popc(peers);
         __syncwarp();
+        return off + __popc(peers & lt);
+    };
+    const auto move = [&](uint2 pt, uint32_t to) {
+        if (pt.x == 0xffffffffu) return;
+        if (order) order[to] = pt.y;
+        if (spos) {
+            const float4 x = __ldg(in.pos + 2 * (size_t)pt.y), y = __ldg(in.pos + 2 * (size_t)pt.y + 1);
+            spos[to] = x;
+            spay[to] = y;
+        }
+    };
+    const auto place_all = [&](const auto& pt) {
+        constexpr int K = sizeof pt / sizeof pt[0];
+        uint32_t to[K];
+#pragma unroll
+        for (int j = 0; j < K; ++j) to[j] = __match_any_sync(0xffffffffu, pt[j].x);
+#pragma unroll
+        for (int j = 0; j < K; ++j) to[j] = place(pt[j].x, to[j]);
+#pragma unroll
+        for (int j = 0; j < K; ++j) move(pt[j], to[j]);
     };
     if (held) {
-#pragma unroll
-        for (int j = 0; j < kPartItems; ++j)
-            if (e0 + 32 * j < e1) place(own[j]);
+        place_all(own);
     } else {
-        for (uint32_t e = e0; e < e1; e += 32)
-            place(point(e + lane));
+        for (uint32_t e = e0; e < e1; e += 32 * kPartAhead) {
+            uint2 pt[kPartAhead];
+#pragma unroll
+            for (int j = 0; j < kPartAhead; ++j) pt[j] = point(e + 32 * j + lane);
+            place_all(pt);
+        }
     }
 }
 
