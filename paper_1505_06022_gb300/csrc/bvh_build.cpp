@@ -308,14 +308,14 @@ std::string bvh_build_host(const float* verts, int64_t nv, const int32_t* tris, 
             float4* q = out.bin.data() + (size_t)ref[n] * 4;
             q[0] = float4{L.lo[0], L.lo[1], L.lo[2], as_float(ref[nd.left])};
             q[1] = float4{L.hi[0], L.hi[1], L.hi[2], as_float(ref[nd.right])};
-            q[2] = float4{R.lo[0], R.lo[1], R.lo[2], 0.0f};
+            q[2] = float4{R.lo[0], R.lo[1], R.lo[2], as_float(sets == 6 ? wide[ref[n]] : -1)};
             q[3] = float4{R.hi[0], R.hi[1], R.hi[2], 0.0f};
         }
         out.bin_root = ref[0];
     };
     {
         std::vector<std::thread> th;
-        if (nthreads > 1) th.emplace_back(pairs);
+        if (nthreads > 1 && nn > 4096) th.emplace_back(pairs);  // (fewer take less than a thread)
         else pairs();
         for (int c = 1; c < sets; ++c) {
             if (nthreads > 1) th.emplace_back(thread_set, c);

@@ -471,7 +471,6 @@ static void scene_free_bvh(gsp_scene* s) {
     cudaFree(s->d_nodes);
     cudaFree(s->d_tris);
     cudaFree(s->d_bin);
-    cudaFree(s->d_wide);
     s->d_wide = nullptr;
     s->d_nodes = nullptr;
     s->d_tris = nullptr;
@@ -736,7 +735,8 @@ gsp_status gsp_build_bvh(gsp_scene* s, const gsp_bvh_params* params, gsp_bvh_sta
     }
     if (!gsp_wide_usable(bvh.link_sets, bvh.depth, s->extent)) bvh.nwide = 0;
     size_t nb = bvh.nodes.size() * sizeof(float4), tb = bvh.tris.size() * sizeof(float4);
-    const size_t bb = std::max<size_t>(1, bvh.bin.size()) * sizeof(float4);
+    const int64_t wide_at = gsp_wide_at(std::max<int64_t>(1, bvh.bin.size()));
+    const size_t bb = (size_t)(wide_at + 8 * bvh.nwide) * sizeof(float4);
     if (s->ctx) {
         GSP_CUDA_TRY(cudaSetDevice(s->ctx->device));
         scene_free_bvh(s);
@@ -749,15 +749,9 @@ gsp_status gsp_build_bvh(gsp_scene* s, const gsp_bvh_params* params, gsp_bvh_sta
             GSP_CUDA_TRY(cudaMemcpy(s->d_bin, bvh.bin.data(), bvh.bin.size() * sizeof(float4), cudaMemcpyHostToDevice));
         if (bvh.nwide) {
             const auto t0 = std::chrono::steady_clock::now();
-            uint32_t* of = nullptr;
-            const size_t ob = bvh.wide_of.size() * sizeof(int32_t);
-            GSP_CUDA_TRY(cudaMalloc(&s->d_wide, (size_t)bvh.nwide * 8 * sizeof(float4)));
-            GSP_CUDA_TRY(cudaMalloc(&of, ob));
-            cudaError_t e = cudaMemcpy(of, bvh.wide_of.data(), ob, cudaMemcpyHostToDevice);
-            if (e == cudaSuccess) e = gsp_wide_build(s->d_bin, (int64_t)bvh.wide_of.size(), nullptr, of, s->d_wide);
-            if (e == cudaSuccess) e = cudaDeviceSynchronize();
-            cudaFree(of);
-            GSP_CUDA_TRY(e);
+            s->d_wide = s->d_bin + wide_at;
+            GSP_CUDA_TRY(gsp_wide_build(s->d_bin, (int64_t)bvh.bin.size() / 4, nullptr, nullptr, s->d_wide));
+            GSP_CUDA_TRY(cudaDeviceSynchronize());
             bvh.thread_ms += std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
         }
         std::vector<int32_t>().swap(bvh.wide_of);

@@ -25,7 +25,7 @@ struct HostBVH {
     std::vector<float4> nodes;  // link_sets * stride * 2
     std::vector<float4> tris;   // nt * 3, leaf order
     // The same tree as child pairs, for stack-based traversal: per internal node (preorder) four
-    // float4 {left.min, left ref}, {left.max, right ref}, {right.min, 0}, {right.max, 0}; a ref
+    // float4 {left.min, left ref}, {left.max, right ref}, {right.min, wide_of}, {right.max, 0}; a ref
     // >= 0 is an internal node, < 0 is ~(leaf word). bin_root: ref of the root.
     std::vector<float4> bin;
     int32_t bin_root = 0;
@@ -119,8 +119,11 @@ inline bool gsp_wide_usable(int32_t link_sets, int32_t depth, double extent) {
     return link_sets == 6 && depth <= kWideMaxDepth && extent <= kWideMaxExtent;
 }
 
-// The entries of all of them on the device: node i has entry index[i], if head is given only where
-// head[i] is set, else where it is not -1.
+// The entries of all of them on the device: node i has entry index[i] where head[i] is set, or with null head and
+// index the one that bin holds (wide_of).
+// Where in an allocation of the child pairs the four-wide entries begin (in float4, a whole number of entries).
+inline int64_t gsp_wide_at(int64_t bin_size) { return (bin_size + 7) / 8 * 8; }
+
 cudaError_t gsp_wide_build(const float4* bin, int64_t n, const uint32_t* head, const uint32_t* index, float4* wide);
 
 // Builds the binned-SAH tree and writes its hit/miss links (one set per ray direction
@@ -157,7 +160,8 @@ struct gsp_scene {
     float4* d_nodes = nullptr;
     float4* d_tris = nullptr;
     float4* d_bin = nullptr;  // child-pair layout (HostBVH::bin)
-    float4* d_wide = nullptr;  // four-wide layout; null if the tree is one leaf or not gsp_wide_usable
+    float4* d_wide = nullptr;  // four-wide layout, behind d_bin in its allocation (gsp_wide_at); null if the tree is
+                               // one leaf or not gsp_wide_usable
     unsigned long long* d_counter = nullptr;  // trace kernel: next ray, refine-list length
     int2* d_rlist = nullptr;                  // trace kernel: hits re-evaluated in FP64
     int64_t rlist_cap = 0;

@@ -259,8 +259,9 @@ __global__ void k_wide_heads(int n, const int32_t* __restrict__ parent, const in
 __global__ void k_wide_entries(const float4* __restrict__ bin, int64_t n, const uint32_t* __restrict__ head,
                                const uint32_t* __restrict__ index, float4* __restrict__ wide) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n || (head ? !head[i] : index[i] == 0xffffffffu)) return;
-    gsp_wide_entry(bin, i, [&](int32_t j) { return (int32_t)index[j]; }, wide + 8 * (size_t)index[i]);
+    const auto of = [&](int64_t j) { return index ? (int32_t)index[j] : __float_as_int(bin[4 * j + 2].w); };
+    if (i >= n || (head ? !head[i] : of(i) < 0)) return;
+    gsp_wide_entry(bin, i, of, wide + 8 * (size_t)of(i));
 }
 
 }  // namespace
@@ -297,7 +298,7 @@ extern "C" gsp_status gsp_build_bvh_device(gsp_scene* s, int32_t link_sets, int3
         if (e == cudaSuccess && *p) tmp.push_back((void*)*p);
     };
     float* d_verts;
-    int32_t *d_tris, *left, *right, *parent, *first, *last, *size, *d_depth;
+    int32_t *d_tris, *left, *right, *parent, *first, *last, *size, *totals, *d_depth;
     uint32_t *ka, *va, *kb, *vb, *hist, *stemp, *d_n, *arrived, *head, *windex;
     Box* box;
     const int64_t nn = 2 * (int64_t)n - 1;
@@ -315,12 +316,13 @@ extern "C" gsp_status gsp_build_bvh_device(gsp_scene* s, int32_t link_sets, int3
     A(&first, std::max<int64_t>(1, n - 1));
     A(&last, std::max<int64_t>(1, n - 1));
     A(&parent, nn);
-    A(&size, nn);
+    A(&totals, nn + 1);  // the number of wide nodes, then the sizes (the root's first): read back together
+    size = totals ? totals + 1 : nullptr;
     A(&box, nn);
     A(&arrived, std::max<int64_t>(1, n - 1));
     A(&d_depth, 1);
-    A(&head, n);
-    A(&windex, n);  // [n - 1]: the number of wide nodes
+    A(&head, 2 * (int64_t)n);
+    windex = head ? head + n : nullptr;
     cudaEvent_t ev[3] = {nullptr, nullptr, nullptr};  // build and threading times
     auto drop_events = [&]() {
         for (cudaEvent_t& x : ev)
@@ -361,14 +363,13 @@ extern "C" gsp_status gsp_build_bvh_device(gsp_scene* s, int32_t link_sets, int3
     const bool wide = n > 1 && gsp_wide_usable(link_sets, 0, s->extent);  // the depth is not known yet
     if (wide) {
         k_wide_heads<<<nblocks(n - 1), kThreads>>>(n, parent, first, last, max_leaf, head);
-        e = gsp_scan_u32(head, windex, n - 1, windex + (n - 1), stemp, nullptr);
+        e = gsp_scan_u32(head, windex, n - 1, (uint32_t*)totals, stemp, nullptr);
     }
-    int32_t nfinal = 0;
-    uint32_t nwide = 0;
+    int32_t back[2] = {0, 0};
     if (e == cudaSuccess) e = cudaGetLastError();
-    if (e == cudaSuccess && wide)
-        e = cudaMemcpy(&nwide, windex + (n - 1), sizeof nwide, cudaMemcpyDeviceToHost);
-    if (e == cudaSuccess) e = cudaMemcpy(&nfinal, size, sizeof nfinal, cudaMemcpyDeviceToHost);  // root: node 0
+    if (e == cudaSuccess) e = cudaMemcpy(back, totals, sizeof back, cudaMemcpyDeviceToHost);
+    const int32_t nfinal = back[1];
+    uint32_t nwide = wide ? (uint32_t)back[0] : 0;
     if (e != cudaSuccess) return fail(e);
     cudaEventRecord(ev[1]);
     // final tree: nfinal nodes per link set (+ one padding node); triangles in Morton order
@@ -377,13 +378,12 @@ extern "C" gsp_status gsp_build_bvh_device(gsp_scene* s, int32_t link_sets, int3
     const int64_t nb = std::max<int64_t>(1, n - 1) * 4;
     e = cudaMalloc(&d_nodes, (size_t)link_sets * stride * 2 * sizeof(float4));
     if (e == cudaSuccess) e = cudaMalloc(&d_tri4, (size_t)nt * 3 * sizeof(float4));
-    if (e == cudaSuccess) e = cudaMalloc(&d_bin, (size_t)nb * sizeof(float4));
-    if (e == cudaSuccess && nwide) e = cudaMalloc(&d_wide, (size_t)nwide * 8 * sizeof(float4));
+    if (e == cudaSuccess) e = cudaMalloc(&d_bin, (size_t)(gsp_wide_at(nb) + 8 * (int64_t)nwide) * sizeof(float4));
+    if (nwide) d_wide = d_bin + gsp_wide_at(nb);
     if (e != cudaSuccess) {
         cudaFree(d_nodes);
         cudaFree(d_tri4);
         cudaFree(d_bin);
-        cudaFree(d_wide);
         return fail(e);
     }
     // (n == 1: the single leaf is node 0 of the radix numbering, n - 1 + 0 = 0)
@@ -418,12 +418,10 @@ extern "C" gsp_status gsp_build_bvh_device(gsp_scene* s, int32_t link_sets, int3
         cudaFree(d_nodes);
         cudaFree(d_tri4);
         cudaFree(d_bin);
-        cudaFree(d_wide);
         return fail(e);
     }
     for (void* p : tmp) cudaFree(p);
     if (!gsp_wide_usable(link_sets, depth, s->extent)) {
-        cudaFree(d_wide);
         d_wide = nullptr;
         nwide = 0;
     }
